@@ -6,6 +6,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "inv_cube.h"
 #include "nbody_internal.h"
 
 namespace nb {
@@ -154,6 +155,26 @@ __device__ __forceinline__ void interact_fp64(const double4_32a &j, double px, d
   ax = fma(f, dx, ax);
   ay = fma(f, dy, ay);
   az = fma(f, dz, az);
+}
+
+// Whether mu is one that the integer path of inv_cube.h takes.
+__device__ __forceinline__ bool mass_fits(double mu) { return ic::mass_in_range(ic::pack_mass(mu)); }
+
+// mu_j |d|^-3 and mu_i |d|^-3 of one pair, masses packed and in range: on the
+// integer pipes, or by the FP64 series where |d| is out of their range (a
+// choice of the pair alone, so its bits do not depend on its neighbours).
+__device__ __forceinline__ void pair_factors(double dx, double dy, double dz, const ic::Mass &mj, const ic::Mass &mi,
+                                             double &fj, double &fi) {
+  const uint32_t em = ic::max_exp(dx, dy, dz);
+  if (ic::exp_in_range(em)) {
+    const ic::Cube c = ic::inv_cube(ic::square_sum(dx, dy, dz, em), em, ic::Rsqrt{});
+    fj = ic::mass_times(mj, c);
+    fi = ic::mass_times(mi, c);
+  } else {
+    const double s3 = inv_r3(fma(dz, dz, fma(dy, dy, dx * dx)));
+    fj = ic::unpack_mass(mj) * s3;
+    fi = ic::unpack_mass(mi) * s3;
+  }
 }
 
 // Mixed: positions split as x = hi + lo (hi = fl32(x), lo = fl32(x - hi)).

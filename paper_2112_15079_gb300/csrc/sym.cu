@@ -1,11 +1,14 @@
 // Eq. 1 force kernel of the FP64 path, each pair once (Newton's third law).
 //
-// The FP64 pipe bounds this path, and one interaction of Eq. 1 takes 16 FP64
-// operations (3 differences, 3 for |d|^2, 6 for |d|^-3 from the MUFU seed and
-// its series, the product with mu_j, 3 accumulations).  The pair (p, j) and
-// its reaction share the first 12 of them: evaluating each unordered pair
-// once and accumulating both terms -- a_p += mu_j |d|^-3 d and
-// a_j -= mu_p |d|^-3 d -- takes 20 operations for two interactions.
+// The FP64 pipe bounds this path (an operation of a warp every 76 cycles per
+// SM sub-partition).  The pair (p, j) and its reaction share the difference
+// and |d|^-3, so evaluating each unordered pair once takes 20 FP64 operations
+// for two interactions; |d|^2, |d|^-3 and the mass products, 11 of them, run
+// on the integer pipes (inv_cube.h), about 120 instructions beside the 9 FP64
+// operations that are left: 3 differences and 6 accumulations.  Measured on
+// GB300, 10,425 bodies: 2.03 ms per step with 20 FP64 operations, 0.94 ms
+// with 9 (9 x 76 cycles a pair and warp step is 0.92 ms: the FP64 pipe stays
+// the bound).
 //
 // Decomposition: each system's bodies are cut into blocks of 64 (two warp
 // tiles of 32); the work items are the block pairs (I, J), I <= J, handed
@@ -53,6 +56,89 @@ __device__ __forceinline__ void sym_pair(double xi, double yi, double zi, double
   }
 }
 
+// Both terms of one pair with the factors mu_j |d|^-3, mu_i |d|^-3 from the
+// integer pipes (inv_cube.h): 9 FP64 operations instead of 20.
+__device__ __forceinline__ void sym_pair_int(double xi, double yi, double zi, const ic::Mass &mi, double xj, double yj,
+                                             double zj, const ic::Mass &mj, double &ax, double &ay, double &az,
+                                             double &bx, double &by, double &bz, bool react) {
+  const double dx = xj - xi, dy = yj - yi, dz = zj - zi;
+  double f, fr;
+  pair_factors(dx, dy, dz, mj, mi, f, fr);
+  ax = fma(f, dx, ax);
+  ay = fma(f, dy, ay);
+  az = fma(f, dz, az);
+  if (react) {
+    bx = fma(-fr, dx, bx);
+    by = fma(-fr, dy, by);
+    bz = fma(-fr, dz, bz);
+  }
+}
+
+// One tile pair: the 32 targets pi (one per lane) against the 32 sources pj,
+// rotated once around the warp; (ax, ay, az) take the targets' sums, (bx, by,
+// bz) return the sources' reaction sums, each in its source's own lane.
+// SELF: the tile with itself, offsets 1..15 both ways and 16 one way (lanes L
+// and L + 16 meet twice).  The sources are rotated a step ahead.  Masses
+// beyond the integer path's range (never in a physical model) take the FP64
+// arithmetic for the whole tile pair.
+template <bool SELF>
+__device__ __forceinline__ void sym_tile(const double4_32a &pi, const double4_32a &pj, int lane, double &ax,
+                                         double &ay, double &az, double &bx, double &by, double &bz) {
+  double xj = pj.x, yj = pj.y, zj = pj.z;
+  bx = by = bz = 0.0;
+  const int src = (lane + 1) & 31;
+  auto rotate = [&]() {
+    xj = __shfl_sync(0xffffffffu, xj, src);
+    yj = __shfl_sync(0xffffffffu, yj, src);
+    zj = __shfl_sync(0xffffffffu, zj, src);
+    bx = __shfl_sync(0xffffffffu, bx, src);
+    by = __shfl_sync(0xffffffffu, by, src);
+    bz = __shfl_sync(0xffffffffu, bz, src);
+  };
+  if (__all_sync(0xffffffffu, mass_fits(pi.w) && mass_fits(pj.w))) {
+    const ic::Mass mi = ic::pack_mass(pi.w);
+    ic::Mass mj = ic::pack_mass(pj.w);
+    auto rotate_mass = [&]() {
+      mj.u = __shfl_sync(0xffffffffu, mj.u, src);
+      mj.w = __shfl_sync(0xffffffffu, mj.w, src);
+    };
+    if (SELF) {
+#pragma unroll 1
+      for (int k = 1; k <= 16; ++k) {
+        rotate();
+        rotate_mass();
+        sym_pair_int(pi.x, pi.y, pi.z, mi, xj, yj, zj, mj, ax, ay, az, bx, by, bz, k < 16);
+      }
+    } else {
+#pragma unroll 2
+      for (int k = 0; k < 32; ++k) {
+        sym_pair_int(pi.x, pi.y, pi.z, mi, xj, yj, zj, mj, ax, ay, az, bx, by, bz, true);
+        rotate();
+        rotate_mass();
+      }
+    }
+  } else {
+    double mj = pj.w;
+    for (int k = SELF ? 1 : 0; k < (SELF ? 17 : 32); ++k) {
+      if (SELF) {
+        rotate();
+        mj = __shfl_sync(0xffffffffu, mj, src);
+      }
+      sym_pair(pi.x, pi.y, pi.z, pi.w, xj, yj, zj, mj, ax, ay, az, bx, by, bz, !SELF || k < 16);
+      if (!SELF) {
+        rotate();
+        mj = __shfl_sync(0xffffffffu, mj, src);
+      }
+    }
+  }
+  if (SELF) {  // lane L holds the sums of lane L + 16: hand them back
+    const int back = (lane + 16) & 31;
+    bx = __shfl_sync(0xffffffffu, bx, back);
+    by = __shfl_sync(0xffffffffu, by, back);
+    bz = __shfl_sync(0xffffffffu, bz, back);
+  }
+}
+
 }  // namespace
 
 __global__ void __launch_bounds__(kSymThreads) force_sym_kernel(const SymArgs a) {
@@ -77,35 +163,10 @@ __global__ void __launch_bounds__(kSymThreads) force_sym_kernel(const SymArgs a)
       double bx = 0.0, by = 0.0, bz = 0.0;
       if (!(I == J && t < w)) {  // tile pair (w, t) with t < w of a diagonal item is (t, w), warp t's
         const double4_32a pj0 = sym_load(a.cur, sb, J * kSymBlock + t * 32 + lane, ns, 1e15 * (lane + 1) + 5e14);
-        double xj = pj0.x, yj = pj0.y, zj = pj0.z, mj = pj0.w;
-        auto rotate = [&]() {
-          const int src = (lane + 1) & 31;
-          xj = __shfl_sync(0xffffffffu, xj, src);
-          yj = __shfl_sync(0xffffffffu, yj, src);
-          zj = __shfl_sync(0xffffffffu, zj, src);
-          mj = __shfl_sync(0xffffffffu, mj, src);
-          bx = __shfl_sync(0xffffffffu, bx, src);
-          by = __shfl_sync(0xffffffffu, by, src);
-          bz = __shfl_sync(0xffffffffu, bz, src);
-        };
-        if (I == J && t == w) {  // a tile with itself: offsets 1..15 both ways, 16 one way
-#pragma unroll 4
-          for (int k = 1; k <= 16; ++k) {
-            rotate();
-            sym_pair(pi.x, pi.y, pi.z, pi.w, xj, yj, zj, mj, ax, ay, az, bx, by, bz, k < 16);
-          }
-          // lane L holds the sums of lane L + 16: hand them back
-          const int back = (lane + 16) & 31;
-          bx = __shfl_sync(0xffffffffu, bx, back);
-          by = __shfl_sync(0xffffffffu, by, back);
-          bz = __shfl_sync(0xffffffffu, bz, back);
-        } else {
-#pragma unroll 4
-          for (int k = 0; k < 32; ++k) {
-            sym_pair(pi.x, pi.y, pi.z, pi.w, xj, yj, zj, mj, ax, ay, az, bx, by, bz, true);
-            rotate();
-          }
-        }
+        if (I == J && t == w)
+          sym_tile<true>(pi, pj0, lane, ax, ay, az, bx, by, bz);
+        else
+          sym_tile<false>(pi, pj0, lane, ax, ay, az, bx, by, bz);
       }
       s_b[w][t][0][lane] = bx;
       s_b[w][t][1][lane] = by;
@@ -197,35 +258,11 @@ __global__ void __launch_bounds__(kSymWideThreads) force_sym_wide_kernel(const S
         const int qn = (p + t + 1) & (T - 1);
         if (t + 1 < T) pn = sym_load(a.cur, sb, j0 + qn * 32 + lane, ns, 1e15 * (lane + 1) + 5e14);
         if (p_live && j0 + q * 32 < ns && !(diag && q < p)) {  // (q < p on a diagonal item: tile q's warp's pair)
-          double xj = pj0.x, yj = pj0.y, zj = pj0.z, mj = pj0.w;
-          double tx = 0.0, ty = 0.0, tz = 0.0, bx = 0.0, by = 0.0, bz = 0.0;
-          auto rotate = [&]() {
-            const int src = (lane + 1) & 31;
-            xj = __shfl_sync(0xffffffffu, xj, src);
-            yj = __shfl_sync(0xffffffffu, yj, src);
-            zj = __shfl_sync(0xffffffffu, zj, src);
-            mj = __shfl_sync(0xffffffffu, mj, src);
-            bx = __shfl_sync(0xffffffffu, bx, src);
-            by = __shfl_sync(0xffffffffu, by, src);
-            bz = __shfl_sync(0xffffffffu, bz, src);
-          };
-          if (diag && q == p) {  // a tile with itself: offsets 1..15 both ways, 16 one way
-#pragma unroll 4
-            for (int k = 1; k <= 16; ++k) {
-              rotate();
-              sym_pair(pi.x, pi.y, pi.z, pi.w, xj, yj, zj, mj, tx, ty, tz, bx, by, bz, k < 16);
-            }
-            const int back = (lane + 16) & 31;
-            bx = __shfl_sync(0xffffffffu, bx, back);
-            by = __shfl_sync(0xffffffffu, by, back);
-            bz = __shfl_sync(0xffffffffu, bz, back);
-          } else {
-#pragma unroll 4
-            for (int k = 0; k < 32; ++k) {
-              sym_pair(pi.x, pi.y, pi.z, pi.w, xj, yj, zj, mj, tx, ty, tz, bx, by, bz, true);
-              rotate();
-            }
-          }
+          double tx = 0.0, ty = 0.0, tz = 0.0, bx, by, bz;
+          if (diag && q == p)
+            sym_tile<true>(pi, pj0, lane, tx, ty, tz, bx, by, bz);
+          else
+            sym_tile<false>(pi, pj0, lane, tx, ty, tz, bx, by, bz);
           ax += tx;
           ay += ty;
           az += tz;

@@ -306,3 +306,22 @@ def test_mixed_energy_drift(nb):
         drift[prec] = worst
         b.close()
     assert drift["mixed"] <= 2.0 * drift["fp64"], drift
+
+
+@pytest.mark.parametrize("block", [64, 256])
+@pytest.mark.parametrize("r_scale, m_scale", [(2.0**230, 1.0), (2.0**-230, 1.0), (1.0, 2.0**-420), (1.0, 2.0**410),
+                                              (2.0**198, 2.0**-398)])
+def test_magnitudes_beyond_the_integer_path(nb, block, r_scale, m_scale):
+    """Differences beyond 2^+-200 and masses beyond 2^+-400 leave the integer
+    evaluation of |d|^-3 for the FP64 series (pair by pair, tile by tile); a
+    power-of-two scale of a model must only scale its accelerations.  Same
+    gate, against the oracle on the unscaled model."""
+    s = inputs.solar_system(1283)
+    m = s.m.copy()
+    m[700:] = 0.0  # massless bodies among them
+    b = nb.NBody(s.r * r_scale, s.v, m * m_scale, G=1.0, dt=1e-3, precision="fp64", small=False,
+                 pair_once_block=block)
+    assert b.pair_once_block == block
+    a = b.accel().cpu().numpy() * (r_scale * r_scale / m_scale)
+    b.close()
+    assert _rel(a, oracle.accel(1.0, s.r, m)) <= 1e-13
