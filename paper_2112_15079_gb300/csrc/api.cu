@@ -151,7 +151,7 @@ struct nbody_ctx {
 
   bool small = false;  // the single-launch cluster kernel serves nbody_step
   bool grid = false;   // the single-launch cooperative grid kernel serves nbody_step
-  int grid_warps = 0, grid_ctas = 0;
+  int grid_warps = 0, grid_parts = 1, grid_ctas = 0;
   double *xg = nullptr;      // grid kernel: [2][3][N] position exchange
   unsigned *gbar = nullptr;  // grid kernel: barrier arrivals
   std::map<int, cudaGraphExec_t> graphs;
@@ -1324,7 +1324,7 @@ nbody_status nbody_init(nbody_ctx **out, int64_t n_systems, const int64_t *offse
     c->small = false;
   }
   c->grid = single && !c->small && c->N <= nb::grid_max_bodies() &&
-            nb::grid_shape(c->N, c->nsm, &c->grid_warps, &c->grid_ctas) == cudaSuccess;
+            nb::grid_shape(c->N, c->nsm, &c->grid_warps, &c->grid_parts, &c->grid_ctas) == cudaSuccess;
   cudaGetLastError();
   if (c->grid) {
     if ((st = dalloc(c, reinterpret_cast<void **>(&c->xg), sizeof(double) * 6 * c->N)) != NBODY_OK) return bail(st);
@@ -1371,6 +1371,7 @@ nbody_status nbody_step(nbody_ctx *c, int64_t n_steps) {
     sa.xg = c->xg;
     sa.gbar = c->gbar;
     sa.N = c->N;
+    sa.parts = c->grid_parts;
     sa.G = c->o.G;
     sa.dt = c->o.dt;
     sa.half_dt = 0.5 * c->o.dt;

@@ -131,12 +131,12 @@ NB_HD Mass pack_mass(double mu) {
   const uint64_t b = bits(mu);
   const uint32_t lo = lo32(b), hi = hi32(b);
   Mass m;
-  m.u = mu == 0.0 ? 0u : fshl(lo, hi, 11) | 0x80000000u;
+  m.u = ((hi << 1) | lo) == 0u ? 0u : fshl(lo, hi, 11) | 0x80000000u;  // (an FP64 compare would cost a pipe slot)
   m.w = (lo << 11) | ((hi >> 20) & 0x7ffu);
   return m;
 }
 NB_HD bool mass_in_range(const Mass &m) { return m.u == 0u || (m.w & 0x7ffu) - kMExpMin <= kMExpSpan; }
-NB_HD double unpack_mass(const Mass &m) {  // of a mass in range
+NB_HD double unpack_mass(const Mass &m) {  // exact for every mu >= 0
   return from_bits((m.w >> 11) | (m.u << 21), m.u ? ((m.w & 0x7ffu) << 20) | ((m.u & 0x7fffffffu) >> 11) : 0u);
 }
 

@@ -143,15 +143,30 @@ __device__ __forceinline__ double inv_r1(double r2) {
 // difference is then exactly zero and r2 is replaced by 1 so the term is 0.
 // ---------------------------------------------------------------------------
 
+// mu |d|^-3 of one source: on the integer pipes (inv_cube.h; leaves the FP64
+// pipe 6 of the interaction's 16 operations), or by the FP64 series where |d|
+// or mu is out of their range.  MASK: where `self`, |d|^2 = 0 is taken as 1.
 template <bool MASK>
-__device__ __forceinline__ void interact_fp64(const double4_32a &j, double px, double py, double pz, bool self,
-                                              double &ax, double &ay, double &az) {
-  const double dx = j.x - px;
-  const double dy = j.y - py;
-  const double dz = j.z - pz;
-  double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-  if (MASK) r2 = self ? 1.0 : r2;
-  const double f = j.w * inv_r3(r2);
+__device__ __forceinline__ double source_factor(double dx, double dy, double dz, const ic::Mass &mu, bool self) {
+  // (The integer result first and the rare case after it: a branch around the
+  // integer chain would keep the compiler from interleaving several.)
+  const uint32_t em = ic::max_exp(dx, dy, dz);
+  double f = ic::mass_times(mu, ic::inv_cube(ic::square_sum(dx, dy, dz, em), em, ic::Rsqrt{}));
+  if (!(ic::exp_in_range(em) && ic::mass_in_range(mu))) {
+    double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
+    if (MASK) r2 = self ? 1.0 : r2;
+    f = ic::unpack_mass(mu) * inv_r3(r2);
+  }
+  return f;
+}
+
+template <bool MASK>
+__device__ __forceinline__ void interact_fp64(double jx, double jy, double jz, const ic::Mass &mu, double px, double py,
+                                              double pz, bool self, double &ax, double &ay, double &az) {
+  const double dx = jx - px;
+  const double dy = jy - py;
+  const double dz = jz - pz;
+  const double f = source_factor<MASK>(dx, dy, dz, mu, self);
   ax = fma(f, dx, ax);
   ay = fma(f, dy, ay);
   az = fma(f, dz, az);
@@ -166,11 +181,10 @@ __device__ __forceinline__ bool mass_fits(double mu) { return ic::mass_in_range(
 __device__ __forceinline__ void pair_factors(double dx, double dy, double dz, const ic::Mass &mj, const ic::Mass &mi,
                                              double &fj, double &fi) {
   const uint32_t em = ic::max_exp(dx, dy, dz);
-  if (ic::exp_in_range(em)) {
-    const ic::Cube c = ic::inv_cube(ic::square_sum(dx, dy, dz, em), em, ic::Rsqrt{});
-    fj = ic::mass_times(mj, c);
-    fi = ic::mass_times(mi, c);
-  } else {
+  const ic::Cube c = ic::inv_cube(ic::square_sum(dx, dy, dz, em), em, ic::Rsqrt{});
+  fj = ic::mass_times(mj, c);
+  fi = ic::mass_times(mi, c);
+  if (!ic::exp_in_range(em)) {
     const double s3 = inv_r3(fma(dz, dz, fma(dy, dy, dx * dx)));
     fj = ic::unpack_mass(mj) * s3;
     fi = ic::unpack_mass(mi) * s3;

@@ -119,6 +119,7 @@ struct SmallArgs {
   double *xg;      // grid kernel: [2][3][N] position exchange buffers
   unsigned *gbar;  // grid kernel: barrier arrivals, zero at launch
   int32_t N;
+  int32_t parts;  // grid kernel: warps to a target
   int64_t n_steps;
   double G, dt, half_dt, half_dt2;
   int32_t stall;  // test hook: CTA 0 skips one barrier arrival (the waits run out)
@@ -285,9 +286,9 @@ int small_max_bodies();
 cudaError_t small_prepare();
 cudaError_t launch_small(const SmallArgs &a, cudaStream_t s);
 int grid_max_bodies();
-// Shape of the grid kernel for N bodies on nsm SMs: warps (targets) per CTA
-// and CTAs, all resident at once; an error if no shape fits.
-cudaError_t grid_shape(int N, int nsm, int *warps, int *ctas);
+// Shape of the grid kernel for N bodies on nsm SMs: warps per CTA, warps to a
+// target and CTAs, all resident at once; an error if no shape fits.
+cudaError_t grid_shape(int N, int nsm, int *warps, int *parts, int *ctas);
 cudaError_t launch_grid(const SmallArgs &a, int warps, int ctas, cudaStream_t s);
 size_t vjp_smem_bytes(int precision, int tj);
 int vjp_threads(int precision);

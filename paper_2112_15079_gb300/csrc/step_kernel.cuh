@@ -391,27 +391,23 @@ __global__ void __launch_bounds__(THREADS, (MinBlocks<PREC, THREADS, IPT>::value
 #pragma unroll
         for (int k = 0; k < IPT; ++k) tx[k] = ty[k] = tz[k] = 0.0;
         if (!diag) {
-          int jj = 0;
-          for (; jj + 4 <= cnt; jj += 4) {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const double4_32a sj = src[jj + u];
-#pragma unroll
-              for (int k = 0; k < IPT; ++k) interact_fp64<false>(sj, px[k], py[k], pz[k], false, tx[k], ty[k], tz[k]);
-            }
-          }
-          for (; jj < cnt; ++jj) {
-            const double4_32a sj = src[jj];
-#pragma unroll
-            for (int k = 0; k < IPT; ++k) interact_fp64<false>(sj, px[k], py[k], pz[k], false, tx[k], ty[k], tz[k]);
-          }
-        } else {
+#pragma unroll 2
           for (int jj = 0; jj < cnt; ++jj) {
             const double4_32a sj = src[jj];
+            const ic::Mass mu = ic::pack_mass(sj.w);
+#pragma unroll
+            for (int k = 0; k < IPT; ++k)
+              interact_fp64<false>(sj.x, sj.y, sj.z, mu, px[k], py[k], pz[k], false, tx[k], ty[k], tz[k]);
+          }
+        } else {
+#pragma unroll 1
+          for (int jj = 0; jj < cnt; ++jj) {
+            const double4_32a sj = src[jj];
+            const ic::Mass mu = ic::pack_mass(sj.w);
             const int jg = jt0 + jj;
 #pragma unroll
             for (int k = 0; k < IPT; ++k)
-              interact_fp64<true>(sj, px[k], py[k], pz[k], jg == tq[k], tx[k], ty[k], tz[k]);
+              interact_fp64<true>(sj.x, sj.y, sj.z, mu, px[k], py[k], pz[k], jg == tq[k], tx[k], ty[k], tz[k]);
           }
         }
 #pragma unroll

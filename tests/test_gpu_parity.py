@@ -191,6 +191,43 @@ def test_grid_kernel_vs_general_and_oracle(nb, n, steps):
         assert np.max(np.linalg.norm(a - a_ref, axis=0) / np.linalg.norm(a_ref, axis=0)) <= FP64_TOL
 
 
+@pytest.mark.parametrize("n", [152, 153, 305, 456, 457, 609, 1216, 1217, 2432, 2433])
+def test_grid_kernel_shapes(nb, n):
+    """The edges of the grid kernel's shapes (1 to 16 targets to a CTA, 4, 2
+    or 1 warps to a target, on 152 SMs; 2,433 bodies take the general path)
+    against the oracle, in the tolerance of the test above."""
+    steps = 5
+    s = inputs.solar_system(n, seed=74, n_moons=0)
+    b = nb.NBody(s.r, s.v, s.m, G=s.G, dt=s.dt, precision="fp64")
+    b.step(steps)
+    b.sync()
+    r_ref, v_ref, a_ref = oracle.verlet(s.G, s.dt, steps, s.r, s.v, s.m, openmp=True)
+    assert np.abs(b.r.cpu().numpy() - r_ref).max() <= 1e-11 * max(1.0, np.abs(r_ref).max())
+    assert np.abs(b.v.cpu().numpy() - v_ref).max() <= 1e-11 * np.abs(v_ref).max()
+    a = b.accel().cpu().numpy()
+    assert np.max(np.linalg.norm(a - a_ref, axis=0) / np.linalg.norm(a_ref, axis=0)) <= FP64_TOL
+
+
+@pytest.mark.parametrize("n", [31, 131, 521])
+@pytest.mark.parametrize("r_scale, m_scale", [(2.0**230, 1.0), (2.0**-230, 1.0), (1.0, 2.0**-420)])
+def test_small_systems_beyond_the_integer_path(nb, n, r_scale, m_scale):
+    """Magnitudes whose |d|^-3 the FP64 series takes (the cluster and grid
+    kernels, and the general path's first force): a power-of-two scale of a
+    model must only scale its accelerations after a step that is too short
+    to move it."""
+    s = inputs.solar_system(n, n_moons=0)
+    m = s.m.copy()
+    m[20:] = 0.0
+    b = nb.NBody(s.r * r_scale, 0.0 * s.v, m * m_scale, G=1.0, dt=1e-200, precision="fp64")
+    ref = oracle.accel(1.0, s.r, m) * (m_scale / (r_scale * r_scale))
+    for _ in range(2):
+        a = b.accel().cpu().numpy()
+        scale = np.abs(ref).max()
+        assert np.max(np.linalg.norm((a - ref) / scale, axis=0) / np.linalg.norm(ref / scale, axis=0)) <= FP64_TOL
+        b.step(1)
+    b.close()
+
+
 def test_grid_kernel_wait_timeout_reports_and_recovers(nb, monkeypatch):
     """NBODY_INJECT_WAIT_STALL=1 makes CTA 0 of the cooperative grid kernel
     (257 bodies) skip its first barrier arrival: every CTA's bounded wait
