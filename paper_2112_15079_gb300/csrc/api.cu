@@ -27,8 +27,6 @@
 #define NBODY_KERNEL_HASH "unknown"
 #endif
 
-using nb::Item;
-
 namespace {
 
 thread_local std::string g_init_error;
@@ -138,11 +136,11 @@ struct nbody_ctx {
   double *rk = nullptr;              // RK4: [3][3N] stage velocity V, sums AR and AV
   double *snap = nullptr;            // [6][N] r0, v0 for nbody_grad
   unsigned *flags = nullptr;
-  int64_t *offsets_dev = nullptr;
-  double *e_body = nullptr;          // [2][N]
+  double *e_part = nullptr;          // energy: [items][4]
   double *e_out = nullptr;           // [2][n_sys]
-  Item *eitems = nullptr;
-  int n_eitems = 0;
+  int4 *eitems = nullptr;
+  int32_t *eitem_off = nullptr;      // [n_sys + 1] items of each system
+  int n_eitems = 0, e_tiles = 0;
 
   // tile-dependent scratch (stream-K work tables of the force kernel)
   nbody_tiles tiles{};
@@ -1061,29 +1059,34 @@ nbody_status alloc_scratch(nbody_ctx *c) {
   if (c->o.integrator == NBODY_RK4) NB_ALLOC(c->rk, sizeof(double) * 9 * N);
   NB_ALLOC(c->snap, sizeof(double) * 6 * N);
   NB_ALLOC(c->flags, sizeof(unsigned));
-  NB_ALLOC(c->offsets_dev, sizeof(int64_t) * (c->n_sys + 1));
-  NB_ALLOC(c->e_body, sizeof(double) * 2 * N);
   NB_ALLOC(c->e_out, sizeof(double) * 2 * c->n_sys);
 #undef NB_ALLOC
   NB_CUDA(c, cudaMemset(c->flags, 0, sizeof(unsigned)));
-  NB_CUDA(c, cudaMemcpy(c->offsets_dev, c->offsets.data(), sizeof(int64_t) * (c->n_sys + 1), cudaMemcpyHostToDevice));
-  // energy items: blocks of kEnergyBlock targets against the whole system
-  std::vector<Item> e;
+  // energy items: the block pairs (I, J), I <= J, of each system
+  std::vector<int64_t> sizes(static_cast<size_t>(c->n_sys));
+  for (int64_t s = 0; s < c->n_sys; ++s) sizes[s] = c->offsets[s + 1] - c->offsets[s];
+  c->e_tiles = nb::kEnergyMinTiles;
+  const int64_t nmax = *std::max_element(sizes.begin(), sizes.end());
+  while (32 * int64_t(c->e_tiles) < nmax && nb::pair_once_items(sizes, 32 * int64_t(c->e_tiles)) > nb::kEnergyItems)
+    c->e_tiles *= 2;
+  std::vector<int4> e;
+  std::vector<int32_t> e_off{0};
   for (int64_t s = 0; s < c->n_sys; ++s) {
-    for (int64_t i0 = c->offsets[s]; i0 < c->offsets[s + 1]; i0 += nb::kEnergyBlock) {
-      Item it{};
-      it.i0 = static_cast<int32_t>(i0);
-      it.i1 = static_cast<int32_t>(std::min<int64_t>(i0 + nb::kEnergyBlock, c->offsets[s + 1]));
-      it.j0 = static_cast<int32_t>(c->offsets[s]);
-      it.j1 = static_cast<int32_t>(c->offsets[s + 1]);
-      it.nsplit = 1;
-      it.sys = static_cast<int32_t>(s);
-      e.push_back(it);
-    }
+    const int64_t B = 32 * int64_t(c->e_tiles);
+    const int nb = static_cast<int>((sizes[s] + B - 1) / B);
+    for (int I = 0; I < nb; ++I)
+      for (int J = I; J < nb; ++J)
+        e.push_back(make_int4(static_cast<int>(c->offsets[s]), static_cast<int>(sizes[s]), I, J));
+    if (e.size() > static_cast<size_t>(INT32_MAX)) return fail(c, NBODY_EINVAL, "too many energy blocks");
+    e_off.push_back(static_cast<int32_t>(e.size()));
   }
   c->n_eitems = static_cast<int>(e.size());
-  if ((st = dalloc(c, reinterpret_cast<void **>(&c->eitems), sizeof(Item) * e.size())) != NBODY_OK) return st;
-  NB_CUDA(c, cudaMemcpy(c->eitems, e.data(), sizeof(Item) * e.size(), cudaMemcpyHostToDevice));
+  if ((st = dalloc(c, reinterpret_cast<void **>(&c->eitems), sizeof(int4) * e.size())) != NBODY_OK ||
+      (st = dalloc(c, reinterpret_cast<void **>(&c->eitem_off), sizeof(int32_t) * e_off.size())) != NBODY_OK ||
+      (st = dalloc(c, reinterpret_cast<void **>(&c->e_part), sizeof(double) * 4 * e.size())) != NBODY_OK)
+    return st;
+  NB_CUDA(c, cudaMemcpy(c->eitems, e.data(), sizeof(int4) * e.size(), cudaMemcpyHostToDevice));
+  NB_CUDA(c, cudaMemcpy(c->eitem_off, e_off.data(), sizeof(int32_t) * e_off.size(), cudaMemcpyHostToDevice));
   return NBODY_OK;
 }
 
@@ -1497,22 +1500,17 @@ nbody_status nbody_energy(nbody_ctx *c, double *e_host) {
   if (!e_host) return fail(c, NBODY_EINVAL, "e_host is NULL");
   nbody_status st;
   if ((st = begin_work(c)) != NBODY_OK) return st;
-  const size_t N = c->N;
   nb::EnergyArgs ea{};
   ea.x = c->x; ea.y = c->y; ea.z = c->z; ea.vx = c->vx; ea.vy = c->vy; ea.vz = c->vz; ea.m = c->m;
-  ea.e_kin = c->e_body;
-  ea.e_pot = c->e_body + N;
   ea.items = c->eitems;
+  ea.item_off = c->eitem_off;
+  ea.part = c->e_part;
+  ea.out = c->e_out;
   ea.n_items = c->n_eitems;
+  ea.n_systems = static_cast<int32_t>(c->n_sys);
+  ea.tiles = c->e_tiles;
   ea.G = c->o.G;
   NB_CUDA(c, nb::launch_energy(ea, c->stream));
-  nb::ReduceArgs ra{};
-  ra.e_kin = c->e_body;
-  ra.e_pot = c->e_body + N;
-  ra.offsets = c->offsets_dev;
-  ra.out = c->e_out;
-  ra.n_systems = static_cast<int32_t>(c->n_sys);
-  NB_CUDA(c, nb::launch_energy_reduce(ra, c->stream));
   std::vector<double> h(2 * c->n_sys);
   NB_CUDA(c, cudaMemcpyAsync(h.data(), c->e_out, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, c->stream));
   if ((st = end_work(c)) != NBODY_OK) return st;

@@ -140,8 +140,8 @@ NB_HD double unpack_mass(const Mass &m) {  // exact for every mu >= 0
   return from_bits((m.w >> 11) | (m.u << 21), m.u ? ((m.w & 0x7ffu) << 20) | ((m.u & 0x7fffffffu) >> 11) : 0u);
 }
 
-// |d|^-3 as (mantissa, exponent): the mantissa's leading one at bit 63,
-// |d|^-3 = m 2^(e - 4089 - ...), e as mass_times takes it.
+// |d|^-3 (or |d|^-1) as a 64-bit mantissa, its leading one at bit 63, and the
+// exponent that mass_times adds to the mass's own exponent field.
 struct Cube {
   uint32_t lo, hi;
   int32_t e;
@@ -191,11 +191,18 @@ NB_HD uint64_t square_sum(double dx, double dy, double dz, uint32_t em20) {
   return R + (C >> 31);
 }
 
-// |d|^-3 from R and em20, steps (2) .. (5).
+// Steps (2) .. (4): R scaled by 2^k (k = 0 or 2), Y and T2 = Y^2 = (th, tl), and
+// e = 1 - R Y^2 / 2^102: ne = -e in units of 2^-70, q = e^2 in units of 2^-66.
+struct Root {
+  uint32_t k, Y, th, tl;
+  int64_t ne;
+  int32_t q;
+};
 template <class Rsq>
-NB_HD Cube inv_cube(uint64_t R, uint32_t em20, const Rsq &rsq) {
-  const uint32_t k = hi32(R) < (1u << 28) ? 2u : 0u;  // scale by 4 below 2^60
-  const uint32_t Rh = fshl(lo32(R), hi32(R), k), Rl = lo32(R) << k;
+NB_HD Root inv_root(uint64_t R, const Rsq &rsq) {
+  Root o;
+  o.k = hi32(R) < (1u << 28) ? 2u : 0u;  // scale by 4 below 2^60
+  const uint32_t Rh = fshl(lo32(R), hi32(R), o.k), Rl = lo32(R) << o.k;
   const float y = rsq(static_cast<float>(Rh));  // Rh in [2^28, 2^30)
 #ifdef __CUDA_ARCH__
   const uint32_t Yr = static_cast<uint32_t>(__float_as_int(__fmaf_rn(y, 34359738368.0f, 8388608.0f))) - 0x4b000000u;
@@ -205,18 +212,36 @@ NB_HD Cube inv_cube(uint64_t R, uint32_t em20, const Rsq &rsq) {
   std::memcpy(&zb, &z, 4);
   const uint32_t Yr = zb - 0x4b000000u;
 #endif
-  const uint32_t Y = Yr < 0x1fffffu ? Yr : 0x1fffffu;  // T < 2^63
-  const uint64_t t = wide(Y, Y);
-  const uint32_t th = hi32(t), tl = lo32(t);
-  // Q = R t / 2^32 mod 2^64 = -e in units of 2^-70
-  uint64_t Q = wide(Rh, tl) + wide(Rl, th) + mulhi(Rl, tl);
-  Q += static_cast<uint64_t>(Rh * th) << 32;
-  const int64_t sQ = static_cast<int64_t>(Q);
-  const int32_t e1 = static_cast<int32_t>(sQ >> 21);  // -e in units of 2^-49
-  const int32_t q = mulhi_s(e1, e1);                  // e^2 in units of 2^-66
-  const int64_t g = static_cast<int64_t>(q) * 30 - (sQ + (sQ >> 1));  // 3e/2 + 15e^2/8 in units of 2^-70
-  uint64_t T = wide(Y, tl);  // Y^3
-  T += static_cast<uint64_t>(Y * th) << 32;
+  o.Y = Yr < 0x1fffffu ? Yr : 0x1fffffu;  // Y^3 < 2^63
+  const uint64_t t = wide(o.Y, o.Y);
+  o.th = hi32(t);
+  o.tl = lo32(t);
+  // R t / 2^32 mod 2^64 = -e in units of 2^-70
+  uint64_t Q = wide(Rh, o.tl) + wide(Rl, o.th) + mulhi(Rl, o.tl);
+  Q += static_cast<uint64_t>(Rh * o.th) << 32;
+  o.ne = static_cast<int64_t>(Q);
+  const int32_t e1 = static_cast<int32_t>(o.ne >> 21);  // -e in units of 2^-49
+  o.q = mulhi_s(e1, e1);
+  return o;
+}
+
+// The mantissa S, its leading one shifted to bit 63, and the exponent.
+NB_HD Cube normalised(uint64_t S, int32_t e) {
+  const uint32_t n = clz32(hi32(S));
+  Cube c;
+  c.hi = fshl(lo32(S), hi32(S), n);
+  c.lo = lo32(S) << n;
+  c.e = e - static_cast<int32_t>(n);
+  return c;
+}
+
+// |d|^-3 from R and em20, step (5).
+template <class Rsq>
+NB_HD Cube inv_cube(uint64_t R, uint32_t em20, const Rsq &rsq) {
+  const Root o = inv_root(R, rsq);
+  const int64_t g = static_cast<int64_t>(o.q) * 30 - (o.ne + (o.ne >> 1));  // 3e/2 + 15e^2/8 in units of 2^-70
+  uint64_t T = wide(o.Y, o.tl);  // Y^3
+  T += static_cast<uint64_t>(o.Y * o.th) << 32;
   // T g / 2^70 = (Th 2^32 + Tl) (gh 2^32 + gl) / 2^70
   const uint32_t Th = hi32(T), Tl = lo32(T);
   const int32_t gh = static_cast<int32_t>(g >> 32);
@@ -224,16 +249,26 @@ NB_HD Cube inv_cube(uint64_t R, uint32_t em20, const Rsq &rsq) {
   int64_t V = static_cast<int64_t>(static_cast<int32_t>(Th)) * gh;
   V += mulhi(Th, gl);
   V += 2 * static_cast<int64_t>(mulhi_s(static_cast<int32_t>(Tl >> 1), gh));
-  const uint64_t S = T + static_cast<uint64_t>(V >> 6);
-  const uint32_t n = clz32(hi32(S));
-  Cube c;
-  c.hi = fshl(lo32(S), hi32(S), n);
-  c.lo = lo32(S) << n;
-  c.e = 3065 + static_cast<int32_t>(k + (k >> 1)) - static_cast<int32_t>(n) - 3 * static_cast<int32_t>(em20 >> 20);
-  return c;
+  return normalised(T + static_cast<uint64_t>(V >> 6),
+                    3065 + static_cast<int32_t>(o.k + (o.k >> 1)) - 3 * static_cast<int32_t>(em20 >> 20));
 }
 
-// mu |d|^-3, rounded to FP64 (half up in the 63-bit product).
+// |d|^-1 likewise: 2^-51 Y (1 - e)^-1/2 = 2^-51 Y (1 + e/2 + 3e^2/8 + ...)
+// (the dropped 5/16 e^3 is below 2^-59).
+template <class Rsq>
+NB_HD Cube inv_dist(uint64_t R, uint32_t em20, const Rsq &rsq) {
+  const Root o = inv_root(R, rsq);
+  const int64_t g = static_cast<int64_t>(o.q) * 6 - (o.ne >> 1);  // e/2 + 3e^2/8 in units of 2^-70
+  const int32_t gh = static_cast<int32_t>(g >> 32);
+  const uint32_t gl = lo32(static_cast<uint64_t>(g));
+  // S = 2^42 Y (1 + g): Y g / 2^28 from the two words of g
+  const int64_t V = ((static_cast<int64_t>(static_cast<int32_t>(o.Y)) * gh) << 4) +
+                    static_cast<int64_t>(wide(o.Y, gl) >> 28);
+  const uint64_t S = make64(0u, o.Y << 10) + static_cast<uint64_t>(V);
+  return normalised(S, 1021 + static_cast<int32_t>(o.k >> 1) - static_cast<int32_t>(em20 >> 20));
+}
+
+// mu |d|^-3 (mu |d|^-1), rounded to FP64 (half up in the 63-bit product).
 NB_HD double mass_times(const Mass &m, const Cube &c) {
   const uint32_t ul = m.w & 0xfffff800u;
   const uint64_t F = wide(m.u, c.hi) + mulhi(m.u, c.lo) + mulhi(ul, c.hi);  // [2^62, 2^64)

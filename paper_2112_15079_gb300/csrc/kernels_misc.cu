@@ -1,7 +1,6 @@
 // Per-body kernels around the Eq. 1 force launches: the Verlet step
 // completion (Eqs. 4 and 3), the RK4 stage completion and stage-1 prep, the
-// staging / pre-drift kernel, the energy kernels, and the force-launch
-// dispatcher.
+// staging / pre-drift kernel, and the force-launch dispatcher.
 #include <mutex>
 #include <type_traits>
 
@@ -657,106 +656,6 @@ cudaError_t launch_pad_fill(void *stage, int64_t n_pairs, cudaStream_t s) {
   if (n_pairs <= 0) return cudaSuccess;
   const int64_t n = n_pairs * 16;
   pad_fill_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, s>>>(static_cast<float *>(stage), n_pairs);
-  return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------------------
-// Energy (Sections 2 and 4): per body p,
-//   e_kin[p] = (1/2) m_p |v_p|^2,   e_pot[p] = -(1/2) m_p sum_{j != p} G m_j / |r_j - r_p|,
-// so that sum_p e_pot[p] = -sum_{p<j} G m_p m_j / |r_j - r_p|.  FP64, one
-// CTA per block of kEnergyBlock targets, sources staged through shared memory.
-// Each body's potential is compensated as the force is: the terms of one
-// source tile are summed plainly, and each tile's sub-sum enters a (hi, lo)
-// pair through TwoSum, so the many small asteroid terms of a moon's sum are
-// not lost below half an ulp of its host's term.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kEnergyBlock) energy_kernel(const EnergyArgs a) {
-  __shared__ double4_32a tile[kEnergyBlock];
-  const Item it = a.items[blockIdx.x];
-  const int p = it.i0 + threadIdx.x;
-  const bool valid = p < it.i1;
-  const int pp = valid ? p : it.i0;
-  const double px = a.x[pp], py = a.y[pp], pz = a.z[pp];
-  double phi = 0.0, phi_lo = 0.0;
-  for (int j0 = it.j0; j0 < it.j1; j0 += kEnergyBlock) {
-    const int j = j0 + threadIdx.x;
-    __syncthreads();
-    if (j < it.j1) tile[threadIdx.x] = make_double4_32a(a.x[j], a.y[j], a.z[j], a.G * a.m[j]);
-    __syncthreads();
-    const int cnt = min(kEnergyBlock, it.j1 - j0);
-    double t = 0.0;
-    for (int u = 0; u < cnt; ++u) {
-      const double4_32a s = tile[u];
-      const double dx = s.x - px, dy = s.y - py, dz = s.z - pz;
-      double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-      const bool self = (j0 + u) == pp;
-      r2 = self ? 1.0 : r2;
-      t += self ? 0.0 : s.w * inv_r1(r2);
-    }
-    two_sum_acc(phi, phi_lo, t);
-  }
-  if (valid) {
-    const double m = a.m[p];
-    const double v2 = fma(a.vz[p], a.vz[p], fma(a.vy[p], a.vy[p], a.vx[p] * a.vx[p]));
-    a.e_kin[p] = 0.5 * m * v2;
-    a.e_pot[p] = -0.5 * m * (phi + phi_lo);
-  }
-}
-
-cudaError_t launch_energy(const EnergyArgs &a, cudaStream_t s) {
-  if (a.n_items <= 0) return cudaSuccess;
-  energy_kernel<<<a.n_items, kEnergyBlock, 0, s>>>(a);
-  return cudaGetLastError();
-}
-
-// Double-double accumulation: Knuth's TwoSum for the error-free sum of two
-// doubles, and Dekker's Fast2Sum to renormalise.
-struct DD {
-  double hi, lo;
-};
-__device__ __forceinline__ DD two_sum(double a, double b) {
-  const double s = a + b;
-  const double bb = s - a;
-  const double e = (a - (s - bb)) + (b - bb);
-  return {s, e};
-}
-__device__ __forceinline__ DD dd_add(DD a, DD b) {
-  DD s = two_sum(a.hi, b.hi);
-  const double e = s.lo + (a.lo + b.lo);
-  const double hi = s.hi + e;
-  return {hi, e - (hi - s.hi)};
-}
-
-// One CTA per system: strided double-double partial sums per thread, then a
-// fixed-shape tree in shared memory (deterministic).
-__global__ void __launch_bounds__(256) energy_reduce_kernel(const ReduceArgs a) {
-  __shared__ DD sk[256], sp[256];
-  const int s = blockIdx.x;
-  const int64_t b = a.offsets[s], e = a.offsets[s + 1];
-  DD k = {0.0, 0.0}, q = {0.0, 0.0};
-  for (int64_t i = b + threadIdx.x; i < e; i += 256) {
-    k = dd_add(k, DD{a.e_kin[i], 0.0});
-    q = dd_add(q, DD{a.e_pot[i], 0.0});
-  }
-  sk[threadIdx.x] = k;
-  sp[threadIdx.x] = q;
-  __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if (threadIdx.x < w) {
-      sk[threadIdx.x] = dd_add(sk[threadIdx.x], sk[threadIdx.x + w]);
-      sp[threadIdx.x] = dd_add(sp[threadIdx.x], sp[threadIdx.x + w]);
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    a.out[s] = sk[0].hi + sk[0].lo;
-    a.out[a.n_systems + s] = sp[0].hi + sp[0].lo;
-  }
-}
-
-cudaError_t launch_energy_reduce(const ReduceArgs &a, cudaStream_t s) {
-  if (a.n_systems <= 0) return cudaSuccess;
-  energy_reduce_kernel<<<a.n_systems, 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 

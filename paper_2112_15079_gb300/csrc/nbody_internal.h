@@ -17,14 +17,6 @@ enum : unsigned {
   kFlagBadInput = 4u,   // negative mass or non-finite state at staging time
 };
 
-// Work description shared by the energy kernel: targets [i0, i1) against
-// sources [j0, j1) of the same system.
-struct Item {
-  int32_t i0, i1, j0, j1;
-  int32_t slot, nsplit, ib, sys;
-};
-static_assert(sizeof(Item) == 32, "Item layout");
-
 // Blk (target block) and Seg (segment of a block's sources): work_plan.h.
 
 // Arguments of one force launch (Eq. 1 partial sums).  The work is cut into
@@ -207,19 +199,17 @@ struct CloseArgs {
   double G, dt, half_dt;
 };
 
+// Energy (energy.cu): items are block pairs (I, J), I <= J, of blocks of 32
+// tiles bodies of one system; system s's are items[item_off[s] ..].
 struct EnergyArgs {
   const double *x, *y, *z, *vx, *vy, *vz, *m;
-  double *e_kin, *e_pot;  // per body
-  const Item *items;      // one item per 256-body target block, j = whole system
-  int32_t n_items;
+  const int4 *items;        // (first body of the system, its bodies, I, J)
+  const int32_t *item_off;  // [n_systems + 1]
+  double *part;             // [items][4]: kinetic (diagonal items) and potential, (hi, lo) each
+  double *out;              // [2][n_systems]: kinetic, potential
+  int32_t n_items, n_systems;
+  int32_t tiles;
   double G;
-};
-
-struct ReduceArgs {
-  const double *e_kin, *e_pot;
-  const int64_t *offsets;  // device copy, n_systems+1
-  double *out;             // [2][n_systems]: kinetic, potential
-  int32_t n_systems;
 };
 
 // Launchers (return the launch's cudaError_t).  `chained`: launch with
@@ -280,7 +270,6 @@ size_t force_msym_smem_bytes(int tiles, int warps);
 cudaError_t launch_close(const CloseArgs &a, int n_clusters, cudaStream_t s, bool chained);
 cudaError_t launch_close_far(const CloseArgs &a, cudaStream_t s, bool chained);
 cudaError_t launch_energy(const EnergyArgs &a, cudaStream_t s);
-cudaError_t launch_energy_reduce(const ReduceArgs &a, cudaStream_t s);
 cudaError_t run_peaks(double *out);
 int small_max_bodies();
 cudaError_t small_prepare();
@@ -311,6 +300,10 @@ constexpr float kPadCoord = 1e15f;  // mixed padding source: far away and massle
 constexpr int kBoxPairs = 32;
 constexpr float kFarEps = 1e-6f;
 constexpr float kFarKappa = 2.0f / kFarEps + 1.0f;
-constexpr int kEnergyBlock = 256;
+// Energy blocks: kEnergyMinTiles tiles of 32 bodies (an item's warps then have
+// four tile pairs each, enough to hide its reduction), doubled while the
+// systems hold more than kEnergyItems block pairs.
+constexpr int kEnergyMinTiles = 4;
+constexpr int64_t kEnergyItems = 65536;
 
 }  // namespace nb

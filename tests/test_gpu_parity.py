@@ -256,6 +256,29 @@ def test_grid_kernel_wait_timeout_reports_and_recovers(nb, monkeypatch):
     assert np.array_equal(b.state.cpu().numpy(), want)
 
 
+@pytest.mark.parametrize("sizes", [[1], [2], [33], [127], [128], [129], [1283], [40, 1, 300, 129, 7]])
+@pytest.mark.parametrize("r_scale", [1.0, 2.0**210, 2.0**-210])
+def test_energy_blocks(nb, sizes, r_scale):
+    """The energy kernel's tiles and blocks (32 and 128 bodies), several
+    systems in one context, massless bodies, and distances that the FP64
+    series takes instead of the integer path.  Tolerance as above: a system's
+    energy within 1e-13 of the sum of the magnitudes of its two parts."""
+    parts = [inputs.solar_system(max(k, 31), seed=90 + i, n_moons=0) for i, k in enumerate(sizes)]
+    r = [p.r[:, :k] * r_scale for p, k in zip(parts, sizes)]
+    v = [p.v[:, :k] / np.sqrt(r_scale) for p, k in zip(parts, sizes)]
+    m = [p.m[:k].copy() for p, k in zip(parts, sizes)]
+    for t in m:
+        t[3::5] = 0.0
+    off = np.concatenate([[0], np.cumsum(sizes)])
+    b = nb.NBody(np.concatenate(r, 1), np.concatenate(v, 1), np.concatenate(m), off, G=inputs.G_AU_DAY, dt=0.1,
+                 precision="fp64")
+    got = b.energy()
+    b.close()
+    for e, x, u, w in zip(got, r, v, m):
+        kin, pot = oracle.energy(inputs.G_AU_DAY, np.ascontiguousarray(x), np.ascontiguousarray(u), w)
+        assert abs(e - (kin + pot)) <= 1e-13 * (abs(kin) + abs(pot))
+
+
 def test_mixed_energy_drift_31_bodies(nb):
     """Energy drift of the mixed path within 2x the oracle's (3650 steps)."""
     s = inputs.solar_system(31)
