@@ -321,7 +321,7 @@ nbody_status nbody_kernel_times(nbody_ctx *ctx, int32_t n_steps, double *out);
  * allocator owns the device memory, where one more cudaMalloc may fail or
  * stall.  This call uses no context and calls no cudaMalloc/cudaFree: its
  * scratch (staged sources, partial sums, work tables, fault flags) lives in one
- * fixed-size __device__ array inside the library, about 3.7 MB, which every
+ * fixed-size __device__ array inside the library, about 8.6 MB, which every
  * GPU that loads the library holds until the process exits.
  *   n        bodies, 1 <= n <= NBODY_STATIC_MAX_BODIES, else NBODY_EINVAL.
  *   G        gravitational constant, > 0.

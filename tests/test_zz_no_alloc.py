@@ -145,3 +145,15 @@ def test_static_accel_refuses_a_capturing_stream(nb):
     _call(nb, s, r, m, out)
     want = oracle.accel(s.G, s.r, s.m)
     assert _rel(out.cpu().numpy(), want).max() <= FP64_TOL
+
+
+@pytest.mark.parametrize("n", [2, 31, 64, 127, 128, 129, 255, 521, 1031, 5003, 20011])
+def test_pieces_and_blocks(nb, n):
+    """Sizes around the target block (128 bodies), with one piece, a few, and
+    a full set of pieces over the blocks; same gate."""
+    torch = pytest.importorskip("torch")
+    s = inputs.solar_system(max(n, 31), seed=12)
+    s.r, s.v, s.m = (np.ascontiguousarray(t[..., :n]) for t in (s.r, s.v, s.m))
+    a = _static_accel(nb, torch, s)
+    ref = oracle.accel(s.G, s.r, s.m, openmp=True)
+    assert np.max(np.linalg.norm(a - ref, axis=0) / np.linalg.norm(ref, axis=0)) <= FP64_TOL
