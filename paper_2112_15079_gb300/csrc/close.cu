@@ -52,8 +52,7 @@ __global__ void __launch_bounds__(kFarThreads) close_far_kernel(const CloseArgs 
     for (int u = 0; u < ne; ++u) partner |= s_part[u] == j;
     if (partner) continue;
     const double dx = a.x[j] - px, dy = a.y[j] - py, dz = a.z[j] - pz;
-    const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-    const double f = (a.G * a.m[j]) * inv_r3(r2);
+    const double f = source_factor<false>(dx, dy, dz, ic::pack_mass(a.G * a.m[j]), false);
     sx = fma(f, dx, sx);
     sy = fma(f, dy, sy);
     sz = fma(f, dz, sz);
@@ -70,109 +69,184 @@ __global__ void __launch_bounds__(kFarThreads) close_far_kernel(const CloseArgs 
     for (int d = 0; d < 3; ++d) a.far_part[static_cast<size_t>(d) * a.n_chunks + g] = s_red[d][0];
 }
 
-__global__ void __launch_bounds__(kCloseThreads) close_kernel(const CloseArgs a) {
-  __shared__ double s_r[3][kCloseThreads], s_mu[kCloseThreads];
-  // per pair (a, b): the term on a (mu_b s d) and on b (-mu_a s d), d = r_b - r_a
-  __shared__ double s_ua[3][kCloseMaxPairs], s_ub[3][kCloseMaxPairs];
-  grid_dependency_wait();    // the far forces, and the state and stage the Verlet kernel wrote
-  grid_dependency_launch();  // the next kernel may start launching (it waits for us)
-  const int c = blockIdx.x, t = threadIdx.x;
-  const int m0 = a.cl_off[c], nm = a.cl_off[c + 1] - m0;
-  const int p0 = a.pr_off[c], np = a.pr_off[c + 1] - p0;
-  const int k = a.cl_k[c];
-  const double h = a.dt / k, hh = 0.5 * h;
-  const bool own = t < nm;
-  const int mi = m0 + t;  // this thread's member
-  const int b = own ? a.mem_body[mi] : 0;
-  const size_t M = static_cast<size_t>(a.n_mem);
-  double v[3] = {0.0, 0.0, 0.0}, an[3] = {0.0, 0.0, 0.0}, af[3] = {0.0, 0.0, 0.0};
-  if (own) {
-    s_r[0][t] = a.x[b];
-    s_r[1][t] = a.y[b];
-    s_r[2][t] = a.z[b];
-    s_mu[t] = a.G * a.m[b];
-    for (int g = a.mch_off[mi]; g < a.mch_off[mi + 1]; ++g)  // chunks in order
-      for (int d = 0; d < 3; ++d) af[d] += a.far_part[static_cast<size_t>(d) * a.n_chunks + g];
-    if (a.complete) {
-      for (int d = 0; d < 3; ++d) {
-        an[d] = a.an[d * M + mi];
-        v[d] = fma(a.half_dt, af[d], a.vh[d * M + mi]);
-      }
-      a.vx[b] = v[0];
-      a.vy[b] = v[1];
-      a.vz[b] = v[2];
-    } else {
-      v[0] = a.vx[b];
-      v[1] = a.vy[b];
-      v[2] = a.vz[b];
-    }
+// Component c of body b's position for the next force launch.
+__device__ __forceinline__ void close_stage(const CloseArgs &a, int b, int c, double r, double *Rc) {
+  if (a.precision == 0) {
+    double *q = reinterpret_cast<double *>(static_cast<double4_32a *>(a.stage) + b);
+    q[c] = r;
+    if (c == 0) q[3] = a.G * a.m[b];
+  } else {
+    Rc[b] = r;
+    float *w = static_cast<float *>(a.stage) + pair_off(a.qidx[b]);
+    const float h = hi_part(r);
+    w[kXh + 2 * c] = h;
+    w[kXl + 2 * c] = lo_part(r, h);
   }
-  // A_near at the positions in s_r, into an (members only).
-  auto near = [&]() {
-    __syncthreads();  // positions written
-    for (int q = t; q < np; q += kCloseThreads) {
-      const int ia = a.pr_a[p0 + q] - m0, ib = a.pr_b[p0 + q] - m0;
-      const double d[3] = {s_r[0][ib] - s_r[0][ia], s_r[1][ib] - s_r[1][ia], s_r[2][ib] - s_r[2][ia]};
-      const double sq = inv_r3(fma(d[2], d[2], fma(d[1], d[1], d[0] * d[0])));
-      const double fa = s_mu[ib] * sq, fb = s_mu[ia] * sq;  // as the force kernel: mu_j |d|^-3
-      for (int u = 0; u < 3; ++u) {
-        s_ua[u][q] = fa * d[u];
-        s_ub[u][q] = fb * -d[u];
-      }
+}
+
+// One cluster.  A sub-step is a chain of dependent operations on a handful of
+// bodies, so the work is spread by component: groups of three lanes, lane c of
+// a group working on component c, ten groups to a warp.  Group t evaluates
+// the force term on one side of one pair (t = 2 pair + side), another group
+// holds one member; positions and terms pass through shared memory, with a
+// barrier over the warps in use only (one warp up to 5 pairs).  mu |d|^-3
+// comes from the integer pipes.  The chain of a sub-step is then 4 FP64
+// operations (drift, difference, term, kick; plus one per further partner)
+// and one integer chain.  Measured on GB300, 10,425 bodies with 23 close pairs
+// in 13 clusters, k <= 292: 2.1 -> 0.78 us per sub-step, 0.76 -> 0.32 ms per
+// mixed step (one thread per pair and per member, 29 FP64 operations and two
+// barriers of 256 threads a sub-step before).
+constexpr int kGroups = 10;  // groups of three lanes per warp
+constexpr int kCloseWarps = kCloseThreads / 32;
+// Members a group holds at most: one unless every warp is in use.
+constexpr int kHeldMax = (kCloseThreads + kGroups * kCloseWarps - 1) / (kGroups * kCloseWarps);
+
+struct CloseShared {
+  double (*r)[3];       // positions of the members
+  double (*u)[3];       // term of side t & 1 of pair t >> 1
+  const ic::Mass *mu;
+  const int16_t *ia, *ib;  // the pairs' members
+  const int16_t *task;     // the members' terms, each in ascending partner order
+};
+
+// The cluster with `W` warps; each group holds up to HELD members: group,
+// group + 10 W, ...
+template <int HELD>
+__device__ __forceinline__ void close_run(const CloseArgs &a, const CloseShared &sh, int cl, int W, int warp,
+                                          int lane) {
+  const int m0 = a.cl_off[cl], nm = a.cl_off[cl + 1] - m0, np = a.pr_off[cl + 1] - a.pr_off[cl];
+  const int e0 = a.mp_off[m0], k = a.cl_k[cl];
+  const int g = lane / 3, c = lane % 3;  // (lanes 30 and 31: no group)
+  const bool live = g < kGroups;
+  const int stride = kGroups * W, group = warp * kGroups + g;
+  auto sync = [&]() {
+    if (W == 1)
+      __syncwarp();
+    else
+      asm volatile("bar.sync 1, %0;" ::"r"(32 * W) : "memory");
+  };
+  const size_t M = static_cast<size_t>(a.n_mem);
+  const double h = a.dt / k, hh = 0.5 * h;
+  auto pick = [&](double *x, double *y, double *z) { return c == 0 ? x : c == 1 ? y : z; };
+  double *const Xc = pick(a.x, a.y, a.z), *const Vc = pick(a.vx, a.vy, a.vz), *const Rc = pick(a.Rx, a.Ry, a.Rz);
+  double r[HELD], vh[HELD], an[HELD];
+  int eb[HELD], ee[HELD], first[HELD];  // the member's terms: task[eb .. ee), the first of them
+  bool own[HELD];
+#pragma unroll
+  for (int s = 0; s < HELD; ++s) {
+    const int t = group + s * stride;
+    own[s] = live && t < nm;
+    r[s] = vh[s] = an[s] = 0.0;
+    eb[s] = ee[s] = first[s] = 0;
+    if (!own[s]) continue;
+    const int mi = m0 + t, b = a.mem_body[mi];
+    eb[s] = a.mp_off[mi] - e0;
+    ee[s] = a.mp_off[mi + 1] - e0;
+    first[s] = sh.task[eb[s]];  // (a member has a partner)
+    double af = 0.0, v;
+    for (int f = a.mch_off[mi]; f < a.mch_off[mi + 1]; ++f) af += a.far_part[static_cast<size_t>(c) * a.n_chunks + f];
+    if (a.complete) {
+      an[s] = a.an[c * M + mi];
+      v = fma(a.half_dt, af, a.vh[c * M + mi]);
+      Vc[b] = v;
+    } else {
+      v = Vc[b];
     }
-    __syncthreads();  // pair terms written (and every read of the positions done)
-    if (own) {
-      double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-      for (int e = a.mp_off[mi]; e < a.mp_off[mi + 1]; ++e) {  // partners in ascending body order
-        const int q = a.mp_pair[e] - p0;
-        const bool first = a.pr_a[p0 + q] - m0 == t;  // this member is the pair's lower body
-        s0 += first ? s_ua[0][q] : s_ub[0][q];
-        s1 += first ? s_ua[1][q] : s_ub[1][q];
-        s2 += first ? s_ua[2][q] : s_ub[2][q];
-      }
-      an[0] = s0;
-      an[1] = s1;
-      an[2] = s2;
+    r[s] = Xc[b];
+    vh[s] = fma(a.half_dt, af, v);
+  }
+  // This lane's first pair side (with few pairs the only one).
+  const int t1 = live && group < 2 * np ? group : 0;
+  const int ia1 = sh.ia[t1 >> 1], ib1 = sh.ib[t1 >> 1];
+  const ic::Mass mu1 = sh.mu[t1 & 1 ? ia1 : ib1];
+  auto term = [&](int t, int ia, int ib, const ic::Mass &mu, bool real) {
+    const double d = sh.r[ib][c] - sh.r[ia][c];
+    const int l0 = lane - c;
+    const double dx = __shfl_sync(0xffffffffu, d, l0), dy = __shfl_sync(0xffffffffu, d, min(l0 + 1, 31)),
+                 dz = __shfl_sync(0xffffffffu, d, min(l0 + 2, 31));
+    if (real) sh.u[t][c] = source_factor<false>(dx, dy, dz, mu, false) * (t & 1 ? -d : d);
+  };
+  // A_near at the positions in sh.r, into an.
+  auto near = [&]() {
+    sync();  // positions written
+    term(t1, ia1, ib1, mu1, live && group < 2 * np);
+    for (int t0 = warp * kGroups + stride; t0 < 2 * np; t0 += stride) {  // warp-uniform
+      const bool real = live && t0 + g < 2 * np;
+      const int t = real ? t0 + g : 0, ia = sh.ia[t >> 1], ib = sh.ib[t >> 1];
+      term(t, ia, ib, sh.mu[t & 1 ? ia : ib], real);
+    }
+    sync();  // terms written (and every read of the positions done)
+#pragma unroll
+    for (int s = 0; s < HELD; ++s) {
+      if (!own[s]) continue;
+      double sum = sh.u[first[s]][c];
+      for (int e = eb[s] + 1; e < ee[s]; ++e) sum += sh.u[sh.task[e]][c];
+      an[s] = sum;
     }
   };
   if (!a.complete) near();
-  double vh[3];
-  for (int d = 0; d < 3; ++d) vh[d] = fma(a.half_dt, af[d], v[d]);
+#pragma unroll 1
   for (int sub = 0; sub < k; ++sub) {
     // (the previous near() ended with a barrier after its last read of the
     // positions, so they may be overwritten now)
-    if (own)
-      for (int d = 0; d < 3; ++d) {
-        vh[d] = fma(hh, an[d], vh[d]);
-        s_r[d][t] = fma(h, vh[d], s_r[d][t]);
-      }
+    const double kick = sub == 0 ? hh : h;  // the half kicks of two sub-steps at once
+#pragma unroll
+    for (int s = 0; s < HELD; ++s) {
+      if (!own[s]) continue;
+      vh[s] = fma(kick, an[s], vh[s]);
+      r[s] = fma(h, vh[s], r[s]);
+      sh.r[group + s * stride][c] = r[s];
+    }
     near();
-    for (int d = 0; d < 3; ++d) vh[d] = fma(hh, an[d], vh[d]);
   }
-  if (!own) return;
-  if (!(isfinite(an[0]) && isfinite(an[1]) && isfinite(an[2]) && isfinite(vh[0]) && isfinite(vh[1]) &&
-        isfinite(vh[2])))
-    atomicOr(a.flags, kFlagNonFinite);
-  for (int d = 0; d < 3; ++d) {
-    a.vh[d * M + mi] = vh[d];
-    a.an[d * M + mi] = an[d];
+#pragma unroll
+  for (int s = 0; s < HELD; ++s) {
+    if (!own[s]) continue;
+    const int mi = m0 + group + s * stride, b = a.mem_body[mi];
+    vh[s] = fma(hh, an[s], vh[s]);
+    if (!(isfinite(an[s]) && isfinite(vh[s]))) atomicOr(a.flags, kFlagNonFinite);
+    a.vh[c * M + mi] = vh[s];
+    a.an[c * M + mi] = an[s];
+    close_stage(a, b, c, r[s], Rc);
   }
-  const double rx = s_r[0][t], ry = s_r[1][t], rz = s_r[2][t];
-  if (a.precision == 0) {
-    static_cast<double4_32a *>(a.stage)[b] = make_double4_32a(rx, ry, rz, s_mu[t]);
-  } else {
-    a.Rx[b] = rx;
-    a.Ry[b] = ry;
-    a.Rz[b] = rz;
-    float *w = static_cast<float *>(a.stage) + pair_off(a.qidx[b]);
-    const float hx = hi_part(rx), hy = hi_part(ry), hz = hi_part(rz);
-    w[kXh] = hx;
-    w[kYh] = hy;
-    w[kZh] = hz;
-    w[kXl] = lo_part(rx, hx);
-    w[kYl] = lo_part(ry, hy);
-    w[kZl] = lo_part(rz, hz);
+}
+
+__global__ void __launch_bounds__(kCloseThreads) close_kernel(const CloseArgs a) {
+  __shared__ double s_r[kCloseThreads][3];
+  __shared__ double s_u[2 * kCloseMaxPairs][3];  // term of side t & 1 of pair t >> 1
+  __shared__ ic::Mass s_mu[kCloseThreads];
+  __shared__ int16_t s_ia[kCloseMaxPairs], s_ib[kCloseMaxPairs];
+  __shared__ int16_t s_task[2 * kCloseMaxPairs];  // the members' terms, each in ascending partner order
+  grid_dependency_wait();    // the far forces, and the state and stage the Verlet kernel wrote
+  grid_dependency_launch();  // the next kernel may start launching (it waits for us)
+  const int cl = blockIdx.x;
+  const int m0 = a.cl_off[cl], nm = a.cl_off[cl + 1] - m0;
+  const int p0 = a.pr_off[cl], np = a.pr_off[cl + 1] - p0;
+  const int e0 = a.mp_off[m0];
+  for (int t = threadIdx.x; t < np; t += kCloseThreads) {
+    s_ia[t] = static_cast<int16_t>(a.pr_a[p0 + t] - m0);
+    s_ib[t] = static_cast<int16_t>(a.pr_b[p0 + t] - m0);
   }
+  for (int t = threadIdx.x; t < nm; t += kCloseThreads) {
+    const int b = a.mem_body[m0 + t];
+    s_mu[t] = ic::pack_mass(a.G * a.m[b]);
+    s_r[t][0] = a.x[b];
+    s_r[t][1] = a.y[b];
+    s_r[t][2] = a.z[b];
+    for (int e = a.mp_off[m0 + t]; e < a.mp_off[m0 + t + 1]; ++e) {
+      const int q = a.mp_pair[e] - p0;
+      s_task[e - e0] = static_cast<int16_t>(2 * q + (a.pr_a[p0 + q] - m0 == t ? 0 : 1));
+    }
+  }
+  __syncthreads();
+  const int W = min(kCloseWarps, (max(2 * np, nm) + kGroups - 1) / kGroups);  // warps in use
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (warp >= W) return;
+  const CloseShared sh{s_r, s_u, s_mu, s_ia, s_ib, s_task};
+  if (W < kCloseWarps)
+    close_run<1>(a, sh, cl, W, warp, lane);
+  else
+    close_run<kHeldMax>(a, sh, cl, W, warp, lane);
 }
 
 namespace {

@@ -216,3 +216,35 @@ def test_reset_rebuilds_the_close_set(nb):
     assert np.array_equal(b.state.cpu().numpy(), c.state.cpu().numpy())
     b.close()
     c.close()
+
+
+@pytest.mark.parametrize("hosts,moons", [(1, 1), (1, 5), (1, 6), (1, 39), (1, 63), (2, 2), (2, 45)])
+def test_cluster_sizes(nb, hosts, moons):
+    """Clusters of one warp (up to 5 pairs), several, all eight, and with more
+    than one member to a lane group (92 bodies): hosts that are themselves a
+    close pair, with moons of their own, two steps of up to ~400 sub-steps
+    against the oracle.  Tolerance: the rounding of 800 sub-steps moves an
+    orbit of 5e-4 AU by about 800^2 u 5e-4 = 4e-14 AU; 1e-11 leaves room for
+    the partners' order."""
+    G = inputs.G_AU_DAY
+    rng = np.random.default_rng(hosts * 100 + moons)
+    r, v, m = [], [], []
+    for k in range(hosts):
+        at, vel = np.zeros(3), np.zeros(3)
+        if hosts == 2:
+            at[0], vel[1] = (k - 0.5) * 2.8e-3, (k - 0.5) * math.sqrt(G * 2e-3 / 2.8e-3)
+        r.append(at), v.append(vel), m.append(1e-3)
+        for _ in range(moons):
+            u = rng.normal(size=3)
+            u /= np.linalg.norm(u)
+            w = np.cross(u, rng.normal(size=3))
+            w /= np.linalg.norm(w)
+            d = rng.uniform(2e-4, 5e-4)
+            r.append(at + d * u), v.append(vel + math.sqrt(G * 1e-3 / d) * w), m.append(1e-13)
+    s = _Sys(np.stack(r, 1), np.stack(v, 1), np.array(m))
+    rg, vg, info = _run(nb, s, "fp64", 2)
+    ro, vo, _, npairs, kmax = oracle.respa(s.G, s.dt, 2, s.r, s.v, s.m, TC, TS)
+    assert info["pairs"] == npairs == hosts * moons + hosts - 1 and info["k_max"] == kmax
+    assert info["members"] == s.n
+    assert np.abs(rg - ro).max() <= 1e-11
+    assert np.abs(vg - vo).max() <= 1e-9 * np.abs(vo).max()
