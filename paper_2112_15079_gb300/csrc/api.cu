@@ -699,6 +699,7 @@ nbody_status launch_force_kernel(nbody_ctx *c, const void *cur, cudaStream_t st,
       m.perm = c->perm;
       m.n_pairs = c->fw.n_sym;
       m.ctr = c->fw.dyn_ctr;
+      m.flags = c->flags;
       m.N = static_cast<int32_t>(c->N);
       m.tiles = c->fw.sym_tiles;
       m.warps = c->fw.sym_tiles / 4;

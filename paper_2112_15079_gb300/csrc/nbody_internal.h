@@ -155,6 +155,7 @@ struct MsymArgs {
   const int32_t *perm;     // [stage entries] body of each entry
   int32_t n_pairs;
   int32_t *ctr;            // [2]: next item, CTAs done (the last one resets both)
+  unsigned *flags;
   int32_t N;
   int32_t tiles;           // T: 32-entry tiles per block, kMsymMinTiles .. kMsymMaxTiles (a power of two)
   int32_t warps;           // W = T / 4 warps per CTA

@@ -21,9 +21,11 @@
 // packed as f32x2 operands: in 32 steps every source meets every target
 // once, eight pairs per lane and step, the two sources of a lane in one
 // packed instruction.  The sources' reaction sums rotate around the warp
-// with shuffles, one lane per step; a CTA barrier closes each phase, and
-// within a phase the warps' chunks differ, so each chunk belongs to one
-// warp and its sums in shared memory take their terms in phase order.
+// with shuffles, one lane per step.  A chunk passes from warp p + 1 (phase
+// t - 2) to warp p (phase t), so its sums in shared memory take their terms
+// in phase order; a warp waits for that one neighbour only, two phases back,
+// so warps with near chunks and warps with far ones drift instead of meeting
+// at a barrier per phase (262,144 bodies: 25.4 -> 23.3 ms per step, 21.7 with the unrolled steps).
 //
 // Sums, all float pairs (hi, lo) fed through TwoSum: a target's packed
 // per-slot sums every two phases (64 terms per half), a source's reaction
@@ -46,6 +48,10 @@
 namespace nb {
 
 namespace {
+
+// Polls of a neighbour's progress in shared memory before it is given up
+// (tens of milliseconds; a phase takes tens of microseconds).
+constexpr int kMsymPolls = 1 << 21;
 
 // Per-warp shared scratch: two chunk buffers, the targets' negated lo parts
 // (duplicated in both halves, read by the near path) and their running
@@ -105,41 +111,29 @@ __device__ __forceinline__ float4 msym_lo(const float *cur, int s0, int e, int n
   return make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-// One chunk: 32 rotation steps of the chunk's sources past the lane's four
-// targets; at step k lane l takes the two entries of pair block
-// (l + k) mod 32 from the chunk buffer cb.  Reaction sums fold into the
-// chunk's shared sums s_j (local chunk entries jc + 2 m + h for pair block
-// m) half way and at the end.  MASKED (a diagonal item): a pair counts only
-// if the target's entry, et0 + 32 a, precedes the source's, jc + 2 m + h.
-// MU_SMEM: the targets' mu come from wmu ([slot a][lane], shared memory)
-// instead of registers.
-template <bool NEAR, bool MASKED, bool MU_SMEM>
-__device__ __forceinline__ void msym_chunk(const float4 (*cb)[32], const f2 (&nxh)[4], const f2 (&nyh)[4],
-                                           const f2 (&nzh)[4], const f2 (&tmu)[4], const f2 (*wmu)[32],
-                                           const MsymWarp &ws, int lane,
-                                           int et0, f2 (&ax)[4], f2 (&ay)[4], f2 (&az)[4], float *s_j, int BT,
-                                           int jc) {
-  f2 bx = 0ull, by = 0ull, bz = 0ull;
-  // the reaction sums held here belong to the sources of pair block m
-  auto fold = [&](int m) {
-    const f2 b[3] = {bx, by, bz};
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      float b0, b1;
-      upk(b[d], b0, b1);
-      const int e0 = jc + 2 * m;
-      two_sum_acc(s_j[(2 * d) * BT + e0], s_j[(2 * d + 1) * BT + e0], -b0);
-      two_sum_acc(s_j[(2 * d) * BT + e0 + 1], s_j[(2 * d + 1) * BT + e0 + 1], -b1);
-    }
-  };
+// Steps [K0, K0 + 16) of a chunk's rotation past the lane's four targets: at
+// step k lane l takes the two entries of pair block m = (l + k) mod 32 of the
+// chunk (cb: its first piece; piece q of block m at cb[q PS + m]), and the
+// block's reaction sums, (bx, by, bz), move one lane down.  The sums start at
+// zero, and end as those of pair block (l + K0 + 16) mod 32.  MASKED (a
+// diagonal item): a pair counts only if the target's entry, et0 + 32 a,
+// precedes the source's, jc + 2 m + h.  MU_SMEM: the targets' mu come from wmu
+// ([slot a][lane], shared memory) instead of registers; tlo: the targets'
+// negated lo parts, [slot][component][lane], both halves alike.
+template <bool NEAR, bool MASKED, bool MU_SMEM, int PS>
+__device__ __forceinline__ void msym_half(const float4 *cb, const f2 (&nxh)[4], const f2 (&nyh)[4],
+                                          const f2 (&nzh)[4], const f2 (&tmu)[4], const f2 (*wmu)[32],
+                                          const f2 (*tlo)[3][32], int lane, int et0, f2 (&ax)[4], f2 (&ay)[4],
+                                          f2 (&az)[4], f2 &bx, f2 &by, f2 &bz, int jc, int K0) {
+  bx = by = bz = 0ull;
   auto step = [&](int k) {
     const int m = (lane + k) & 31;
-    const float4 A = cb[0][m], B = cb[1][m];
+    const float4 A = cb[m], B = cb[PS + m];
     const f2 sx = pk(A.x, A.y), sy = pk(A.z, A.w), sz = pk(B.x, B.y), sm = pk(B.z, B.w);
     f2 sxl = 0ull, syl = 0ull, szl = 0ull;
     if (NEAR) {
-      const float4 C = cb[2][m];
-      const float2 D = *reinterpret_cast<const float2 *>(&cb[3][m]);  // (zl0, zl1)
+      const float4 C = cb[2 * PS + m];
+      const float2 D = *reinterpret_cast<const float2 *>(cb + 3 * PS + m);  // (zl0, zl1)
       sxl = pk(C.x, C.y);
       syl = pk(C.z, C.w);
       szl = pk(D.x, D.y);
@@ -148,9 +142,9 @@ __device__ __forceinline__ void msym_chunk(const float4 (*cb)[32], const f2 (&nx
     for (int a = 0; a < 4; ++a) {
       f2 dx = add2(sx, nxh[a]), dy = add2(sy, nyh[a]), dz = add2(sz, nzh[a]);
       if (NEAR) {
-        dx = add2(dx, add2(sxl, ws.tlo[a][0][lane]));
-        dy = add2(dy, add2(syl, ws.tlo[a][1][lane]));
-        dz = add2(dz, add2(szl, ws.tlo[a][2][lane]));
+        dx = add2(dx, add2(sxl, tlo[a][0][lane]));
+        dy = add2(dy, add2(syl, tlo[a][1][lane]));
+        dz = add2(dz, add2(szl, tlo[a][2][lane]));
       }
       f2 r2 = mul2(dx, dx);
       r2 = fma2(dy, dy, r2);
@@ -185,13 +179,35 @@ __device__ __forceinline__ void msym_chunk(const float4 (*cb)[32], const f2 (&nx
     by = __shfl_sync(0xffffffffu, by, src);
     bz = __shfl_sync(0xffffffffu, bz, src);
   };
+  // (Unrolled 4 deep against 1: 65,536 bodies 1.62 -> 1.50 ms per step with the
+  // waits above; 8 is 2 % better with mu in shared memory, 1 % worse without.)
+#pragma unroll(MU_SMEM ? 8 : 4)
+  for (int k = 0; k < 16; ++k) step(K0 + k);
+}
+
+// One chunk, all 32 steps: every source meets every target once.  The
+// reaction sums fold into the chunk's float pairs s_j (local chunk entries
+// jc + 2 m + h for pair block m) half way and at the end.
+template <bool NEAR, bool MASKED, bool MU_SMEM>
+__device__ __forceinline__ void msym_chunk(const float4 (*cb)[32], const f2 (&nxh)[4], const f2 (&nyh)[4],
+                                           const f2 (&nzh)[4], const f2 (&tmu)[4], const f2 (*wmu)[32],
+                                           const MsymWarp &ws, int lane, int et0, f2 (&ax)[4], f2 (&ay)[4],
+                                           f2 (&az)[4], float *s_j, int BT, int jc) {
 #pragma unroll 1
-  for (int k = 0; k < 16; ++k) step(k);
-  fold((lane + 16) & 31);
-  bx = by = bz = 0ull;
-#pragma unroll 1
-  for (int k = 16; k < 32; ++k) step(k);
-  fold(lane);
+  for (int K0 = 0; K0 < 32; K0 += 16) {
+    f2 bx, by, bz;
+    msym_half<NEAR, MASKED, MU_SMEM, 32>(cb[0], nxh, nyh, nzh, tmu, wmu, ws.tlo, lane, et0, ax, ay, az, bx, by, bz, jc,
+                                         K0);
+    const f2 b[3] = {bx, by, bz};
+    const int e0 = jc + 2 * ((lane + K0 + 16) & 31);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      float b0, b1;
+      upk(b[d], b0, b1);
+      two_sum_acc(s_j[(2 * d) * BT + e0], s_j[(2 * d + 1) * BT + e0], -b0);
+      two_sum_acc(s_j[(2 * d) * BT + e0 + 1], s_j[(2 * d + 1) * BT + e0 + 1], -b1);
+    }
+  }
 }
 
 }  // namespace
@@ -199,12 +215,14 @@ __device__ __forceinline__ void msym_chunk(const float4 (*cb)[32], const f2 (&nx
 // MU_SMEM: the targets' mu in shared memory, which frees 8 registers in the
 // rotation loop.  Used with 2,048-entry blocks (16-warp CTAs, one per SM),
 // where it measured faster on GB300 (1,048,576 bodies: 395 against 403 ms
-// per step); with 512-entry blocks its 4 KB per CTA cost an SM its fourth
-// CTA (65,536 bodies: 1.71 against 1.64 ms), so they keep mu in registers.
+// per step, then with a barrier per phase); with 512-entry blocks its 4 KB per
+// CTA cost an SM its fourth CTA (65,536 bodies: 1.71 against 1.64 ms), so
+// they keep mu in registers.
 template <bool MU_SMEM>
 __global__ void __launch_bounds__(32 * kMsymMaxWarps, 1) force_msym_kernel(const MsymArgs a) {
   extern __shared__ __align__(16) unsigned char msym_smem[];
   __shared__ int s_item;
+  __shared__ volatile int s_done[kMsymMaxWarps];  // phases each warp has finished
   grid_dependency_wait();    // staged sources and boxes of this step are complete
   grid_dependency_launch();  // the Verlet kernel may start launching
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
@@ -219,6 +237,7 @@ __global__ void __launch_bounds__(32 * kMsymMaxWarps, 1) force_msym_kernel(const
   for (;;) {
     __syncthreads();  // the previous item's shared sums are consumed
     if (tid == 0) s_item = atomicAdd(a.ctr, 1);
+    if (lane == 0) s_done[w] = 0;
     for (int k = tid; k < 6 * BT; k += 32 * W) s_j[k] = 0.f;
     __syncthreads();
     const int item = s_item;
@@ -313,8 +332,21 @@ __global__ void __launch_bounds__(32 * kMsymMaxWarps, 1) force_msym_kernel(const
           }
         }
         if ((t & 1) || t + 1 == NC) fold_targets();
-        __syncthreads();  // phase done: the chunks change hands
+        // Phase done.  The chunk of the next phase was the neighbour's two
+        // phases before it: wait for that one only.
+        if (W > 1) {
+          __syncwarp();
+          __threadfence_block();
+          if (lane == 0) s_done[w] = t + 1;
+          const int next = w + 1 < W ? w + 1 : 0;
+          int polls = 0;
+          while (s_done[next] < t && polls < kMsymPolls) ++polls;
+          if (polls == kMsymPolls && lane == 0) atomicOr(a.flags, kFlagTimeout);
+          __syncwarp();
+          __threadfence_block();
+        }
       }
+      __syncthreads();  // all phases done
       if (p_live) {
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
