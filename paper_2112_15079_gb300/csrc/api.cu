@@ -364,7 +364,9 @@ int sym_block(const nbody_ctx *c) {
   if (c->sh_world > 0 || (c->o.flags & NBODY_FLAG_NO_SYM)) return 0;
   std::vector<int64_t> sizes(static_cast<size_t>(c->n_sys));
   for (int64_t s = 0; s < c->n_sys; ++s) sizes[s] = c->offsets[s + 1] - c->offsets[s];
-  return nb::pair_once_block(sizes, c->o.precision == NBODY_MIXED, c->nsm, c->o.pair_once_block);
+  const bool mixed = c->o.precision == NBODY_MIXED;
+  const int B = nb::pair_once_block(sizes, mixed, c->nsm, c->o.pair_once_block);
+  return B == 0 && mixed ? nb::msym_small_block(sizes, c->nsm) : B;
 }
 
 // Work tables of the pair-once kernels: the block pairs (I, J), I <= J, of
@@ -388,8 +390,17 @@ nbody_status build_sym_work(nbody_ctx *c, Work &wk, int row_doubles, int B) {
       for (int J = I; J < nb; ++J)
         (I == J ? diag : off_diag).push_back(make_int4(static_cast<int>(c->soff[s]), static_cast<int>(ns), I, J));
   }
-  std::vector<int4> pairs = std::move(off_diag);
-  pairs.insert(pairs.end(), diag.begin(), diag.end());
+  std::vector<int4> pairs;
+  if (mixed && B == 32 * nb::kMsymMinTiles) {
+    // small mixed items: the near (and masked) ones cost more, so they go first
+    // and the last round is of far ones
+    pairs = std::move(diag);
+    std::stable_sort(off_diag.begin(), off_diag.end(), [](const int4 &p, const int4 &q) { return p.w - p.z < q.w - q.z; });
+    pairs.insert(pairs.end(), off_diag.begin(), off_diag.end());
+  } else {
+    pairs = std::move(off_diag);
+    pairs.insert(pairs.end(), diag.begin(), diag.end());
+  }
   if (rows > 65535 || pairs.size() > static_cast<size_t>(INT32_MAX))
     return fail(c, NBODY_EINVAL, "too many pair-once blocks (%lld in a system)", static_cast<long long>(rows));
   const int occ = mixed ? nb::force_msym_ctas_per_sm(B / 32, B / 128) : nb::force_sym_ctas_per_sm(B / 32);

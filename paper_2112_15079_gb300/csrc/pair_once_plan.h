@@ -14,13 +14,12 @@
 //   60.8 against 55.3 us per step, 1,283 bodies / 231 pairs 62.5 against
 //   96.2).
 //   Mixed (stage entries per block): for a largest system of at least
-//   kMsymMinBodies (measured on GB300: 65,536 bodies 1.63 against 1.82 ms
-//   per step, 1,048,576 bodies 395 against 430 ms; 10,425 bodies 75 against
-//   68 us, where the per-body kernel reads 82 rows per body and does not
-//   overlap), the narrowest block (128 .. 2,048 entries) that leaves the
-//   largest system at most kMsymMaxRows rows per body, if the rows fit in
-//   kSymRowLimit and the block pairs give at least 8 warps per SM (each warp
-//   holds 128 targets).
+//   kMsymMinBodies (measured on GB300: 65,536 bodies 1.50 against 1.82 ms
+//   per step, 1,048,576 bodies 340 against 430 ms), the narrowest block (128 ..
+//   2,048 entries) that leaves the largest system at most kMsymMaxRows rows
+//   per body, if the rows fit in kSymRowLimit and the block pairs give at
+//   least 8 warps per SM (each warp holds 128 targets); smaller systems:
+//   msym_small_block.
 // A requested block size is used as asked (nbody_init checks its rows
 // against kSymRowLimit and 65,535 blocks per system).
 #pragma once
@@ -95,6 +94,48 @@ inline int pair_once_block(const std::vector<int64_t> &sizes, bool mixed, int64_
     if (pair_once_row_bytes(sizes, B) > kSymRowLimit) return 0;
   }
   return 2 * pair_once_items(sizes, B) >= 3 * nsm ? static_cast<int>(B) : 0;
+}
+
+// Mixed systems below kMsymMinBodies: 128-entry blocks (force_msym_block_kernel,
+// four warps to a block pair), or 512, or 0 for the every-ordered-pair
+// kernel.  Measured on GB300, us per step, every ordered pair / 128 / 512:
+//   bodies          31    300   1,031  2,131  4,096  5,003  8,192  10,425  20,011  32,768  50,001
+//   ordered        9.6   10.5    14.3   17.7   23.3   26.8   45.7    68.1     208     517    1077
+//   128            9.8   10.1    10.2   12.9   20.2   35.6   47.5    61.3     185     702    2057
+//   512                                                              86.9     194     431     915
+//   systems x bodies  64 x 40..400  2,000 x 500  10 x 5,000  100 x 5,000  64 x 1,000..20,000
+//   ordered                   22.4          610         171         1338                4529
+//   128                       14.1          484         140         1871                9027
+//   512                       54.9          534         154         1135                3745
+// 128: while the rows written per step (24 B per body and block) stay in the
+// L2 cache (kMsymRowBytes) or are few (kMsymFewRows per body), and the block
+// pairs fill the GPU's 4 x SMs CTAs once at most or at least five times
+// (between, the second round runs half empty), for a largest system of at
+// least kMsymSmallBodies or block pairs enough for five rounds (a few smaller
+// systems keep the ordered-pair kernel, whose tiles the caller can set, and
+// whose far test, a warp's 32 targets at a time, is finer); else 512 where
+// that gives 8 warps per SM and the rows would have left the cache.
+constexpr int64_t kMsymRowBytes = 80000000;
+constexpr int64_t kMsymFewRows = 8;
+constexpr int64_t kMsymSmallBodies = 2048;
+
+inline int msym_small_block(const std::vector<int64_t> &sizes, int64_t nsm) {
+  constexpr int64_t B = 32 * kMsymMinTiles, Bw = 4 * B;
+  int64_t nmax = 0, N = 0, rows = 0;
+  for (int64_t n : sizes) {
+    nmax = std::max(nmax, n);
+    N += n;
+    rows += (n + B - 1) / B * n;
+  }
+  if (nmax >= kMsymMinBodies) return 0;  // pair_once_block decides
+  if (24 * rows > kMsymRowBytes && rows > kMsymFewRows * N)
+    return pair_once_row_bytes(sizes, Bw) <= kSymRowLimit / 4 && pair_once_items(sizes, Bw) * (Bw / B) >= 8 * nsm
+               ? static_cast<int>(Bw)
+               : 0;
+  if (pair_once_row_bytes(sizes, B) > kSymRowLimit / 4) return 0;
+  const int64_t items = pair_once_items(sizes, B);
+  const bool fills = items >= 20 * nsm;
+  return fills || (nmax >= kMsymSmallBodies && items <= 4 * nsm) ? static_cast<int>(B) : 0;
 }
 
 }  // namespace nb

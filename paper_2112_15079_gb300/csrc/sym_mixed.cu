@@ -388,11 +388,221 @@ __global__ void __launch_bounds__(32 * kMsymMaxWarps, 1) force_msym_kernel(const
   }
 }
 
+// 128-entry blocks (force_msym_block_kernel): an item is small, so a CTA of
+// four warps takes it together.  All four hold block I's 128 targets; warp w
+// takes the 16 rotation steps from 16 (w & 1) of chunk w >> 1 of block J.
+// Block I and block J (4 KB each) and their boxes are copied to shared memory
+// an item ahead, descriptors fetched two and item numbers three ahead, so
+// only the barriers at an item's ends and its sums' combination are left
+// outside the rotation (loading them at the item's start kept the warps
+// waiting for memory 2.4 issue slots in 7: 65.4 us per step at 10,425 bodies,
+// 61.3 so).  One warp per item, two 32-step chunks one after the other, left
+// an SM with 1.4 rounds of long items: 70 us.  ncu at 10,425 bodies: FMA pipe
+// 52 % busy while SMs are active, of the ~76 % its register reads allow.
+//
+// Sums: a target has 16 terms per warp and half; the two halves and the two
+// warps of a chunk are added plainly (64 terms, as everywhere in the mixed
+// path), the two chunks' sums through TwoSum.  A source has 64 terms from each
+// of its two warps, added through TwoSum.  Every order is fixed.
+constexpr int kBlkWarps = 4;
+
+struct MsymBlockShared {
+  float4 src[2][2][4][64];        // [buffer][block I, J][piece][pair block]
+  float4 box[2][2][3][2];         // [buffer][block I, J][stage group of its entries][low, high corner]
+  f2 ti[kBlkWarps][4][3][32];     // per warp: the targets' negated lo parts, then their packed sums
+  f2 tj[kBlkWarps][3][32];        // per warp: reaction sums of its chunk's pair blocks
+};
+
+__global__ void __launch_bounds__(32 * kBlkWarps, 4) force_msym_block_kernel(const MsymArgs a) {
+  extern __shared__ __align__(16) unsigned char msym_smem[];
+  MsymBlockShared &sh = *reinterpret_cast<MsymBlockShared *>(msym_smem);
+  __shared__ int s_item;
+  grid_dependency_wait();    // staged sources and boxes of this step are complete
+  grid_dependency_launch();  // the Verlet kernel may start launching
+  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+  const int chunk = w >> 1, K0 = 16 * (w & 1);
+  const size_t N = static_cast<size_t>(a.N);
+  // An item's descriptor: (first stage entry of the system, its bodies, block
+  // I, block J); no bodies past the last item.
+  auto describe = [&](int item) { return item < a.n_pairs ? a.pairs[item] : make_int4(0, 0, 0, 0); };
+  // Blocks I and J of an item, and the boxes of the stage groups they touch,
+  // into buffer bb.
+  auto stage_item = [&](const int4 &pr, int bb) {
+    if (pr.y > 0) {
+      const int nst = (pr.y + 1) & ~1;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {  // (4 x 128 threads: 2 blocks x 64 pair blocks x 4 pieces)
+        const int blk = u >> 1, pb = tid >> 1, q = 2 * (u & 1) + (tid & 1);
+        const int e0 = 128 * (blk ? pr.w : pr.z) + 2 * pb;
+        float4 *dst = &sh.src[bb][blk][q][pb];
+        if (e0 < nst) {
+          cp_async16(dst, reinterpret_cast<const float4 *>(a.cur) + static_cast<size_t>((pr.x + e0) >> 1) * 4 + q);
+        } else {  // past the end of the system: inert, each entry at a position of its own
+          const float x0 = 2.f * kPadCoord + 1e12f * static_cast<float>(e0 - nst), x1 = x0 + 1e12f;
+          *dst = q == 0 ? make_float4(x0, x1, x0, x1) : q == 1 ? make_float4(x0, x1, 0.f, 0.f)
+                                                               : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+      }
+      if (tid < 12) {
+        const int blk = tid / 6, u = (tid % 6) >> 1, e0 = 128 * (blk ? pr.w : pr.z);
+        const int g = ((pr.x + e0) >> 1) / kBoxPairs + u, last = ((pr.x + min(e0 + 128, nst) - 1) >> 1) / kBoxPairs;
+        float4 *dst = &sh.box[bb][blk][u][tid & 1];
+        if (g <= last)
+          cp_async16(dst, a.boxes + 2 * g + (tid & 1));
+        else  // empty
+          *dst = tid & 1 ? make_float4(-INFINITY, -INFINITY, -INFINITY, 0.f)
+                         : make_float4(INFINITY, INFINITY, INFINITY, 0.f);
+      }
+    }
+    cp_async_commit();
+  };
+  // The item numbers run three ahead (the first is the CTA's own, the others
+  // from the counter), descriptors two, data one.
+  int fetched = 0;  // thread 0
+  if (tid == 0) {
+    s_item = static_cast<int>(gridDim.x) + atomicAdd(a.ctr, 1);
+    fetched = static_cast<int>(gridDim.x) + atomicAdd(a.ctr, 1);
+  }
+  int4 pr = describe(blockIdx.x);
+  stage_item(pr, 0);
+  __syncthreads();
+  int4 pn = describe(s_item);
+  int bb = 0;
+  while (pr.y > 0) {
+    cp_async_wait_all();
+    __syncthreads();  // this item's blocks are in; the previous item's sums (and s_item) are consumed
+    if (tid == 0) {
+      s_item = fetched;
+      fetched = static_cast<int>(gridDim.x) + atomicAdd(a.ctr, 1);  // used an item later
+    }
+    stage_item(pn, bb ^ 1);
+    const int s0 = pr.x, ns = pr.y, I = pr.z, J = pr.w;
+    const int nst = (ns + 1) & ~1;
+    const bool diag = I == J;
+    const int i0 = 128 * I, j0 = 128 * J, jc = 64 * chunk;
+    const int bi = i0 + tid < ns ? a.perm[s0 + i0 + tid] : -1, bj = j0 + tid < ns ? a.perm[s0 + j0 + tid] : -1;
+    bool far = false;
+    {
+      float4 ilo = sh.box[bb][0][0][0], ihi = sh.box[bb][0][0][1];
+#pragma unroll
+      for (int u = 1; u < 3; ++u) {
+        const float4 l = sh.box[bb][0][u][0], h = sh.box[bb][0][u][1];
+        ilo = make_float4(fminf(ilo.x, l.x), fminf(ilo.y, l.y), fminf(ilo.z, l.z), 0.f);
+        ihi = make_float4(fmaxf(ihi.x, h.x), fmaxf(ihi.y, h.y), fmaxf(ihi.z, h.z), 0.f);
+      }
+      // the chunk's entries lie in one or two of block J's groups
+      const int gj = ((s0 + j0) >> 1) / kBoxPairs, g0 = ((s0 + j0 + jc) >> 1) / kBoxPairs - gj,
+                g1 = ((s0 + min(j0 + jc + 64, nst) - 1) >> 1) / kBoxPairs - gj;
+      if (j0 + jc < nst)
+        far = boxes_apart(ilo, ihi, sh.box[bb][1][g0][0], sh.box[bb][1][g0][1]) &&
+              boxes_apart(ilo, ihi, sh.box[bb][1][g1][0], sh.box[bb][1][g1][1]);
+    }
+    f2 ax[4], ay[4], az[4], bx = 0ull, by = 0ull, bz = 0ull;
+#pragma unroll
+    for (int s = 0; s < 4; ++s) ax[s] = ay[s] = az[s] = 0ull;
+    if (j0 + jc < nst) {  // (warp-uniform; a diagonal item's chunk 1 meets targets of both halves, chunk 0 too)
+      f2 nxh[4], nyh[4], nzh[4], tmu[4];
+#pragma unroll
+      for (int s = 0; s < 4; ++s) {
+        // target entry 32 s + lane: pair block 16 s + lane / 2, half lane & 1
+        const float *p0 = reinterpret_cast<const float *>(&sh.src[bb][0][0][16 * s + (lane >> 1)]) + (lane & 1);
+        const float *p1 = reinterpret_cast<const float *>(&sh.src[bb][0][1][16 * s + (lane >> 1)]) + (lane & 1);
+        const float *p2 = reinterpret_cast<const float *>(&sh.src[bb][0][2][16 * s + (lane >> 1)]) + (lane & 1);
+        const float *p3 = reinterpret_cast<const float *>(&sh.src[bb][0][3][16 * s + (lane >> 1)]) + (lane & 1);
+        nxh[s] = pk(-p0[0], -p0[0]);
+        nyh[s] = pk(-p0[2], -p0[2]);
+        nzh[s] = pk(-p1[0], -p1[0]);
+        tmu[s] = pk(p1[2], p1[2]);
+        sh.ti[w][s][0][lane] = pk(-p2[0], -p2[0]);
+        sh.ti[w][s][1][lane] = pk(-p2[2], -p2[2]);
+        sh.ti[w][s][2][lane] = pk(-p3[0], -p3[0]);
+      }
+      __syncwarp();
+      const float4 *cb = &sh.src[bb][1][0][32 * chunk];
+      if (diag)
+        msym_half<true, true, false, 64>(cb, nxh, nyh, nzh, tmu, nullptr, sh.ti[w], lane, lane, ax, ay, az, bx, by, bz,
+                                         jc, K0);
+      else if (far)
+        msym_half<false, false, false, 64>(cb, nxh, nyh, nzh, tmu, nullptr, sh.ti[w], lane, lane, ax, ay, az, bx, by,
+                                           bz, jc, K0);
+      else
+        msym_half<true, false, false, 64>(cb, nxh, nyh, nzh, tmu, nullptr, sh.ti[w], lane, lane, ax, ay, az, bx, by,
+                                          bz, jc, K0);
+      __syncwarp();  // the lo parts are read
+    }
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+      sh.ti[w][s][0][lane] = ax[s];
+      sh.ti[w][s][1][lane] = ay[s];
+      sh.ti[w][s][2][lane] = az[s];
+    }
+    const int m = (lane + K0 + 16) & 31;  // the pair block whose sums this lane holds
+    sh.tj[w][0][m] = bx;
+    sh.tj[w][1][m] = by;
+    sh.tj[w][2][m] = bz;
+    __syncthreads();
+    // thread t: target entry t and source entry t
+    float hi[3], lo[3], rh[3], rl[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      float e[kBlkWarps], o[kBlkWarps];
+#pragma unroll
+      for (int k = 0; k < kBlkWarps; ++k) upk(sh.ti[k][tid >> 5][d][lane], e[k], o[k]);
+      hi[d] = (e[0] + o[0]) + (e[1] + o[1]);
+      lo[d] = 0.f;
+      two_sum_acc(hi[d], lo[d], (e[2] + o[2]) + (e[3] + o[3]));
+      // source entry t: chunk t / 64, pair block (t / 2) % 32, half t % 2
+      const int c2 = 2 * (tid >> 6), mb = (tid >> 1) & 31;
+      const float *r0 = reinterpret_cast<const float *>(&sh.tj[c2][d][mb]) + (tid & 1);
+      const float *r1 = reinterpret_cast<const float *>(&sh.tj[c2 + 1][d][mb]) + (tid & 1);
+      rh[d] = -*r0;
+      rl[d] = 0.f;
+      two_sum_acc(rh[d], rl[d], -*r1);
+    }
+    float2 *part = reinterpret_cast<float2 *>(a.partial);
+    if (diag) {
+      if (bi >= 0) {
+        float2 *row = part + static_cast<size_t>(I) * 3 * N + bi;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          two_sum_acc(hi[d], lo[d], rh[d]);
+          row[d * N] = make_float2(hi[d], lo[d] + rl[d]);
+        }
+      }
+    } else {
+      if (bi >= 0) {
+        float2 *row = part + static_cast<size_t>(J) * 3 * N + bi;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) row[d * N] = make_float2(hi[d], lo[d]);
+      }
+      if (bj >= 0) {
+        float2 *row = part + static_cast<size_t>(I) * 3 * N + bj;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) row[d * N] = make_float2(rh[d], rl[d]);
+      }
+    }
+    pr = pn;
+    pn = describe(s_item);  // (written before the barrier above; used an item later)
+    bb ^= 1;
+  }
+  cp_async_wait_all();
+  __syncthreads();
+  // The last CTA out resets the item counter for the next launch.
+  if (tid == 0) {
+    __threadfence();
+    if (atomicAdd(a.ctr + 1, 1) == static_cast<int>(gridDim.x) - 1) {
+      atomicExch(a.ctr, 0);
+      atomicExch(a.ctr + 1, 0);
+    }
+  }
+}
+
 namespace {
 bool msym_mu_smem(int tiles) { return tiles == kMsymMaxTiles; }
 }  // namespace
 
 size_t force_msym_smem_bytes(int tiles, int warps) {
+  if (tiles == kMsymMinTiles) return sizeof(MsymBlockShared);
   return static_cast<size_t>(warps) * sizeof(MsymWarp) + sizeof(float) * 6 * 32 * static_cast<size_t>(tiles) +
          (msym_mu_smem(tiles) ? sizeof(f2) * 4 * 32 * static_cast<size_t>(warps) : 0);
 }
@@ -400,7 +610,7 @@ size_t force_msym_smem_bytes(int tiles, int warps) {
 cudaError_t launch_force_msym(const MsymArgs &a, int grid, cudaStream_t s, bool chained) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(32 * a.warps);
+  cfg.blockDim = dim3(a.tiles == kMsymMinTiles ? 32 * kBlkWarps : 32 * a.warps);
   cfg.dynamicSmemBytes = force_msym_smem_bytes(a.tiles, a.warps);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -408,6 +618,7 @@ cudaError_t launch_force_msym(const MsymArgs &a, int grid, cudaStream_t s, bool 
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = chained ? 1 : 0;
+  if (a.tiles == kMsymMinTiles) return cudaLaunchKernelEx(&cfg, force_msym_block_kernel, a);
   if (msym_mu_smem(a.tiles)) return cudaLaunchKernelEx(&cfg, force_msym_kernel<true>, a);
   return cudaLaunchKernelEx(&cfg, force_msym_kernel<false>, a);
 }
@@ -415,13 +626,13 @@ cudaError_t launch_force_msym(const MsymArgs &a, int grid, cudaStream_t s, bool 
 int force_msym_ctas_per_sm(int tiles, int warps) {
   int occ = 0;
   const int max_smem = static_cast<int>(force_msym_smem_bytes(kMsymMaxTiles, kMsymMaxWarps));
-  cudaError_t e = cudaFuncSetAttribute(force_msym_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+  const auto kernel = tiles == kMsymMinTiles ? force_msym_block_kernel
+                      : msym_mu_smem(tiles)  ? force_msym_kernel<true>
+                                             : force_msym_kernel<false>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(force_msym_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
-  if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, msym_mu_smem(tiles) ? force_msym_kernel<true>
-                                                                               : force_msym_kernel<false>,
-                                                      32 * warps, force_msym_smem_bytes(tiles, warps));
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, tiles == kMsymMinTiles ? 32 * kBlkWarps : 32 * warps,
+                                                      force_msym_smem_bytes(tiles, warps));
   if (e != cudaSuccess) {
     cudaGetLastError();
     return 0;

@@ -325,3 +325,23 @@ def test_magnitudes_beyond_the_integer_path(nb, block, r_scale, m_scale):
     a = b.accel().cpu().numpy() * (r_scale * r_scale / m_scale)
     b.close()
     assert _rel(a, oracle.accel(1.0, s.r, m)) <= 1e-13
+
+
+@pytest.mark.parametrize("sizes,want", [([1283], 0), ([2049], 128), ([4352], 128), ([5003], 0), ([21001], 512),
+                                        ([2049, 400, 129, 128, 127, 31, 2, 1], 128), ([31, 129, 2] * 700, 128)])
+def test_mixed_small_systems_take_blocks(nb, sizes, want):
+    """The automatic choice below 65,536 bodies (128- and 512-entry blocks, the
+    ordered-pair kernel between), several systems whose stage offsets are no
+    multiples of the 64-entry groups: the mixed gate on every body."""
+    parts = [inputs.solar_system(max(k, 31), seed=60 + i) for i, k in enumerate(sizes)]
+    r = np.concatenate([p.r[:, :k] for p, k in zip(parts, sizes)], 1)
+    v = np.concatenate([p.v[:, :k] for p, k in zip(parts, sizes)], 1)
+    m = np.concatenate([p.m[:k] for p, k in zip(parts, sizes)])
+    off = np.concatenate([[0], np.cumsum(sizes)])
+    a, used = _mixed_accel(nb, r, v, m, off)
+    assert used == want
+    for b, e in zip(off[:-1], off[1:]):
+        x, w = np.ascontiguousarray(r[:, b:e]), m[b:e]
+        ref, t = oracle.accel(inputs.G_AU_DAY, x, w, openmp=True), oracle.term_norm(inputs.G_AU_DAY, x, w)
+        err = np.linalg.norm(a[:, b:e] - ref, axis=0)
+        assert np.all(err <= 2e-6 * t)
