@@ -235,10 +235,8 @@ NB_HD Cube normalised(uint64_t S, int32_t e) {
   return c;
 }
 
-// |d|^-3 from R and em20, step (5).
-template <class Rsq>
-NB_HD Cube inv_cube(uint64_t R, uint32_t em20, const Rsq &rsq) {
-  const Root o = inv_root(R, rsq);
+// |d|^-3, step (5).
+NB_HD Cube cube_of(const Root &o, uint32_t em20) {
   const int64_t g = static_cast<int64_t>(o.q) * 30 - (o.ne + (o.ne >> 1));  // 3e/2 + 15e^2/8 in units of 2^-70
   uint64_t T = wide(o.Y, o.tl);  // Y^3
   T += static_cast<uint64_t>(o.Y * o.th) << 32;
@@ -251,6 +249,34 @@ NB_HD Cube inv_cube(uint64_t R, uint32_t em20, const Rsq &rsq) {
   V += 2 * static_cast<int64_t>(mulhi_s(static_cast<int32_t>(Tl >> 1), gh));
   return normalised(T + static_cast<uint64_t>(V >> 6),
                     3065 + static_cast<int32_t>(o.k + (o.k >> 1)) - 3 * static_cast<int32_t>(em20 >> 20));
+}
+template <class Rsq>
+NB_HD Cube inv_cube(uint64_t R, uint32_t em20, const Rsq &rsq) {
+  return cube_of(inv_root(R, rsq), em20);
+}
+
+// |d|^-3 and |d|^-2 of one difference: R^-1 = 2^-102 Y^2 (1 - e)^-1 = 2^-102 Y^2 (1 + e +
+// e^2 + ...) (the dropped e^3 is below 2^-57).
+NB_HD int64_t mulhi64(int64_t a, int64_t b) {
+#ifdef __CUDA_ARCH__
+  return __mul64hi(a, b);
+#else
+  return static_cast<int64_t>((static_cast<__int128>(a) * b) >> 64);
+#endif
+}
+struct CubeSquare {
+  Cube cube, square;
+};
+template <class Rsq>
+NB_HD CubeSquare inv_cube_square(uint64_t R, uint32_t em20, const Rsq &rsq) {
+  const Root o = inv_root(R, rsq);
+  CubeSquare r;
+  r.cube = cube_of(o, em20);
+  const uint64_t t = make64(o.tl, o.th);  // <= 2^42
+  const int64_t g = static_cast<int64_t>(o.q) * 16 - o.ne;  // e + e^2 in units of 2^-70
+  const uint64_t S = (t << 20) + static_cast<uint64_t>(mulhi64(static_cast<int64_t>(t << 14), g));  // 2^20 t (1 + g)
+  r.square = normalised(S, 2044 + static_cast<int32_t>(o.k) - 2 * static_cast<int32_t>(em20 >> 20));
+  return r;
 }
 
 // |d|^-1 likewise: 2^-51 Y (1 - e)^-1/2 = 2^-51 Y (1 + e/2 + 3e^2/8 + ...)

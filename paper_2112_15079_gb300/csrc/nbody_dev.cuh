@@ -191,6 +191,31 @@ __device__ __forceinline__ void pair_factors(double dx, double dy, double dz, co
   }
 }
 
+// The factors of one pair's vector-Jacobian product (vjp.cu): mu_q |d|^-3,
+// mu_j |d|^-3, |d|^-3 and 3 |d|^-2, as pair_factors above; 0 where `self`.
+struct VjpFactors {
+  double fq, fj, s3, z;
+};
+__device__ __forceinline__ VjpFactors vjp_factors(double dx, double dy, double dz, const ic::Mass &mq,
+                                                  const ic::Mass &mj, const ic::Mass &one, const ic::Mass &three, bool self) {
+  const uint32_t em = ic::max_exp(dx, dy, dz);
+  const ic::CubeSquare c = ic::inv_cube_square(ic::square_sum(dx, dy, dz, em), em, ic::Rsqrt{});
+  VjpFactors f;
+  f.fq = ic::mass_times(mq, c.cube);
+  f.fj = ic::mass_times(mj, c.cube);
+  f.s3 = ic::mass_times(one, c.cube);
+  f.z = ic::mass_times(three, c.square);
+  if (!(ic::exp_in_range(em) && ic::mass_in_range(mq) && ic::mass_in_range(mj))) {
+    const double y = self ? 0.0 : inv_r1(fma(dz, dz, fma(dy, dy, dx * dx)));
+    const double y2 = y * y;
+    f.s3 = y * y2;
+    f.fq = ic::unpack_mass(mq) * f.s3;
+    f.fj = ic::unpack_mass(mj) * f.s3;
+    f.z = 3.0 * y2;
+  }
+  return f;
+}
+
 // Mixed: positions split as x = hi + lo (hi = fl32(x), lo = fl32(x - hi)).
 // d = (hi_j - hi_p) + (lo_j - lo_p): the hi difference is exact whenever the
 // two coordinates are within a factor 2 (Sterbenz), so close pairs keep the

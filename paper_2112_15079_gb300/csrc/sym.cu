@@ -312,14 +312,21 @@ __global__ void __launch_bounds__(kSymWideThreads) force_sym_wide_kernel(const S
 // once.  For the pair (q, j), d = r_j - r_q, s3 = |d|^-3, s5 = |d|^-5 and
 // u = mu_q w_j - mu_j w_q, the q term s3 u - 3 s5 (d.u) d changes sign
 // under q <-> j (K(d) is even in d, u is odd), and the mass terms are
-// s3 (w_j . d) for q and -s3 (w_q . d) for j.  Rows hold 4 values per body
-// (the three components and the mass sum), block I's sums in row J, block
-// J's in row I, as in force_sym_kernel.
+// s3 (w_j . d) for q and -s3 (w_q . d) for j.  With f_q = mu_q s3,
+// f_j = mu_j s3, a = w_j . d, b = w_q . d and z = 3 |d|^-2 the q term is
+//   f_q w_j - f_j w_q - z (f_q a - f_j b) d:
+// f_q, f_j, s3 and z come from the integer pipes (inv_cube.h), which leaves 29
+// FP64 operations to a pair (3 differences, 6 for a and b, 3 for the last
+// factor, 9 for the term, 6 + 2 accumulations) of the 48 that |d|^-1, its
+// powers and u took: 2,131 bodies 240 -> 156 us per product and reverse
+// step.  Rows hold 4 values per body (the three components and the mass
+// sum), block I's sums in row J, block J's in row I, as in force_sym_kernel.
 __global__ void __launch_bounds__(kSymThreads) vjp_sym_kernel(const VjpSymArgs a) {
   __shared__ double s_b[2][2][4][32];  // reaction sums [warp][J tile][component][lane]
   __shared__ int s_item;
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   const size_t N = static_cast<size_t>(a.N);
+  const ic::Mass one = ic::pack_mass(1.0), three = ic::pack_mass(3.0);
   for (;;) {
     __syncthreads();
     if (tid == 0) s_item = atomicAdd(a.ctr, 1);
@@ -332,6 +339,7 @@ __global__ void __launch_bounds__(kSymThreads) vjp_sym_kernel(const VjpSymArgs a
     const int iq = I * kSymBlock + w * 32 + lane;
     const double4_32a pq = sym_load(a.pos, sb, iq, ns, 1e15 * (lane + 1));
     const double4_32a wq = iq < ns ? a.w[sb + iq] : make_double4_32a(0.0, 0.0, 0.0, 0.0);
+    const ic::Mass mq = ic::pack_mass(pq.w);
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
     for (int t = 0; t < 2; ++t) {
       double b[4] = {0.0, 0.0, 0.0, 0.0};
@@ -339,13 +347,15 @@ __global__ void __launch_bounds__(kSymThreads) vjp_sym_kernel(const VjpSymArgs a
         const int ij = J * kSymBlock + t * 32 + lane;
         const double4_32a pj0 = sym_load(a.pos, sb, ij, ns, 1e15 * (lane + 1) + 5e14);
         const double4_32a wj0 = ij < ns ? a.w[sb + ij] : make_double4_32a(0.0, 0.0, 0.0, 0.0);
-        double xj = pj0.x, yj = pj0.y, zj = pj0.z, mj = pj0.w, wjx = wj0.x, wjy = wj0.y, wjz = wj0.z;
+        double xj = pj0.x, yj = pj0.y, zj = pj0.z, wjx = wj0.x, wjy = wj0.y, wjz = wj0.z;
+        ic::Mass mj = ic::pack_mass(pj0.w);
         auto rotate = [&]() {
           const int src = (lane + 1) & 31;
           xj = __shfl_sync(0xffffffffu, xj, src);
           yj = __shfl_sync(0xffffffffu, yj, src);
           zj = __shfl_sync(0xffffffffu, zj, src);
-          mj = __shfl_sync(0xffffffffu, mj, src);
+          mj.u = __shfl_sync(0xffffffffu, mj.u, src);
+          mj.w = __shfl_sync(0xffffffffu, mj.w, src);
           wjx = __shfl_sync(0xffffffffu, wjx, src);
           wjy = __shfl_sync(0xffffffffu, wjy, src);
           wjz = __shfl_sync(0xffffffffu, wjz, src);
@@ -354,28 +364,26 @@ __global__ void __launch_bounds__(kSymThreads) vjp_sym_kernel(const VjpSymArgs a
         };
         auto pair = [&](bool react) {
           const double dx = xj - pq.x, dy = yj - pq.y, dz = zj - pq.z;
-          const double y = inv_r1(fma(dz, dz, fma(dy, dy, dx * dx)));
-          const double y2 = y * y;
-          const double s3 = y * y2;
-          const double s5 = s3 * y2;
-          const double ux = fma(-mj, wq.x, pq.w * wjx);
-          const double uy = fma(-mj, wq.y, pq.w * wjy);
-          const double uz = fma(-mj, wq.z, pq.w * wjz);
-          const double t3 = 3.0 * s5 * fma(dz, uz, fma(dy, uy, dx * ux));
-          const double tx = fma(-t3, dx, s3 * ux), ty = fma(-t3, dy, s3 * uy), tz = fma(-t3, dz, s3 * uz);
+          const VjpFactors f = vjp_factors(dx, dy, dz, mq, mj, one, three, false);
+          const double al = fma(wjz, dz, fma(wjy, dy, wjx * dx));
+          const double be = fma(wq.z, dz, fma(wq.y, dy, wq.x * dx));
+          const double c = f.z * fma(-f.fj, be, f.fq * al);
+          const double tx = fma(-c, dx, fma(-f.fj, wq.x, f.fq * wjx));
+          const double ty = fma(-c, dy, fma(-f.fj, wq.y, f.fq * wjy));
+          const double tz = fma(-c, dz, fma(-f.fj, wq.z, f.fq * wjz));
           acc[0] += tx;
           acc[1] += ty;
           acc[2] += tz;
-          acc[3] = fma(s3, fma(wjz, dz, fma(wjy, dy, wjx * dx)), acc[3]);
+          acc[3] = fma(f.s3, al, acc[3]);
           if (react) {
             b[0] -= tx;
             b[1] -= ty;
             b[2] -= tz;
-            b[3] = fma(-s3, fma(wq.z, dz, fma(wq.y, dy, wq.x * dx)), b[3]);
+            b[3] = fma(-f.s3, be, b[3]);
           }
         };
         if (I == J && t == w) {
-#pragma unroll 2
+#pragma unroll 1
           for (int k = 1; k <= 16; ++k) {
             rotate();
             pair(k < 16);

@@ -187,26 +187,21 @@ __global__ void __launch_bounds__(THREADS) vjp_kernel(const VjpArgs a) {
         const double4_32a *sp = reinterpret_cast<const double4_32a *>(pos_ptr(s));
         const double4_32a *sw = reinterpret_cast<const double4_32a *>(w_ptr(s));
         double tacc[4] = {0, 0, 0, 0};
+        const ic::Mass mq = ic::pack_mass(qmu), one = ic::pack_mass(1.0), three = ic::pack_mass(3.0);
+#pragma unroll 1
         for (int jj = 0; jj < cnt; ++jj) {
           const double4_32a r = sp[jj], w = sw[jj];
           const double dx = r.x - qx, dy = r.y - qy, dz = r.z - qz;
-          double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-          // The target itself: r2 = 1 and |d|^-1 = 0, so all its terms are 0
-          // (u = mu_q w_q - mu_q w_q need not round to exactly 0).
+          // (the target itself: d = 0 leaves the integer path, and its factors are 0)
           const bool self = diag && jt0 + jj == tq;
-          r2 = self ? 1.0 : r2;
-          const double y = self ? 0.0 : inv_r1(r2);
-          const double y2 = y * y;
-          const double s3 = y * y2;
-          const double s5 = s3 * y2;
-          const double ux = fma(-r.w, wqx, qmu * w.x);
-          const double uy = fma(-r.w, wqy, qmu * w.y);
-          const double uz = fma(-r.w, wqz, qmu * w.z);
-          const double t3 = 3.0 * s5 * fma(dz, uz, fma(dy, uy, dx * ux));
-          tacc[0] = fma(-t3, dx, fma(s3, ux, tacc[0]));
-          tacc[1] = fma(-t3, dy, fma(s3, uy, tacc[1]));
-          tacc[2] = fma(-t3, dz, fma(s3, uz, tacc[2]));
-          tacc[3] = fma(s3, fma(w.z, dz, fma(w.y, dy, w.x * dx)), tacc[3]);
+          const VjpFactors f = vjp_factors(dx, dy, dz, mq, ic::pack_mass(r.w), one, three, self);
+          const double al = fma(w.z, dz, fma(w.y, dy, w.x * dx));
+          const double be = fma(wqz, dz, fma(wqy, dy, wqx * dx));
+          const double c = f.z * fma(-f.fj, be, f.fq * al);
+          tacc[0] = fma(-c, dx, fma(-f.fj, wqx, fma(f.fq, w.x, tacc[0])));
+          tacc[1] = fma(-c, dy, fma(-f.fj, wqy, fma(f.fq, w.y, tacc[1])));
+          tacc[2] = fma(-c, dz, fma(-f.fj, wqz, fma(f.fq, w.z, tacc[2])));
+          tacc[3] = fma(f.s3, al, tacc[3]);
         }
 #pragma unroll
         for (int c = 0; c < 4; ++c) two_sum_acc(acc[c], cmp[c], tacc[c]);
@@ -294,72 +289,89 @@ __global__ void __launch_bounds__(THREADS) vjp_kernel(const VjpArgs a) {
 // update and stage w = alpha' + dt/2 nu'; mode 1: the same but stage
 // w = alpha' (the next product is the last one, at r_0); mode 2: the last
 // product only (rho, g_m updated, nothing staged).
+//
+// A CTA takes 32 bodies: warp c adds component c of their rows (3: the mass
+// sum), lane l body l, and then updates that component, so a body's row sums
+// and update, FP64 work whose cost does not depend on the active lanes, are
+// spread over four sub-partitions and N / 32 CTAs.  (One thread per body in
+// CTAs of 256 kept 9 SMs busy at 2,131 bodies, with 276 FP64 operations in a
+// row where a warp now has 69.)  Mixed
+// rows are many at 128-entry blocks, so kAdjParts warps share a component's
+// rows, part p taking rows p, p + kAdjParts, ...
 template <int PREC>
-__global__ void __launch_bounds__(256) adjoint_kernel(const AdjArgs a) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= a.N) return;
+struct AdjShape {
+  static constexpr int kParts = PREC == 0 ? 1 : 2;
+  static constexpr int kThreads = 32 * 4 * kParts;
+  static constexpr int kUnroll = 8;
+};
+
+template <int PREC>
+__global__ void __launch_bounds__(AdjShape<PREC>::kThreads) adjoint_kernel(const AdjArgs a) {
+  constexpr int U = AdjShape<PREC>::kUnroll, P = AdjShape<PREC>::kParts;
+  __shared__ float2 s_part[P][4][32];
+  const int lane = threadIdx.x & 31, c = (threadIdx.x >> 5) & 3, part = threadIdx.x >> 7;
+  const int p = blockIdx.x * 32 + lane;
   const size_t N = static_cast<size_t>(a.N);
-  const int rows = a.nsl[p];
-  double s[4], e[4];
+  const bool live = p < a.N;
+  const int rows = live ? a.nsl[p] : 0;
+  double sum;
   if (PREC == 0) {
     // rows in groups of 8, added plainly in row order, each group sum then
     // through TwoSum (the pair-once VJP leaves a row per 64-body block)
+    double s = 0.0, e = 0.0;
+    for (int r0 = 0; r0 < rows; r0 += U) {
+      double v[U], g = 0.0;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) s[c] = e[c] = 0.0;
-    for (int r0 = 0; r0 < rows; r0 += 8) {
-      double g[4] = {0.0, 0.0, 0.0, 0.0};
-      for (int r = r0; r < min(rows, r0 + 8); ++r) {
-        const double *row = a.partial + static_cast<size_t>(r) * 4 * N;
+      for (int u = 0; u < U; ++u) v[u] = r0 + u < rows ? __ldg(a.partial + (static_cast<size_t>(r0 + u) * 4 + c) * N + p) : 0.0;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) g[c] += row[c * N + p];
-      }
-#pragma unroll
-      for (int c = 0; c < 4; ++c) two_sum_acc(s[c], e[c], g[c]);
+      for (int u = 0; u < U; ++u)
+        if (r0 + u < rows) g += v[u];
+      two_sum_acc(s, e, g);
     }
+    sum = s + e;
   } else {
-    float fs[4] = {0.f, 0.f, 0.f, 0.f}, fe[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int r = 0; r < rows; ++r) {
-      const float2 *row = reinterpret_cast<const float2 *>(a.partial + static_cast<size_t>(r) * 4 * N);
+    const float2 *rp = reinterpret_cast<const float2 *>(a.partial);
+    float fs = 0.f, fe = 0.f;
+    for (int r0 = part; r0 < rows; r0 += U * P) {
+      float2 v[U];
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const float2 v = row[c * N + p];
-        two_sum_acc(fs[c], fe[c], v.x);
-        fe[c] += v.y;
+      for (int u = 0; u < U; ++u)
+        v[u] = r0 + u * P < rows ? __ldg(rp + (static_cast<size_t>(r0 + u * P) * 4 + c) * N + p) : make_float2(0.f, 0.f);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        two_sum_acc(fs, fe, v[u].x);
+        fe += v[u].y;
       }
     }
+    s_part[part][c][lane] = make_float2(fs, fe);
+    __syncthreads();
+    if (part != 0) return;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      s[c] = static_cast<double>(fs[c]);
-      e[c] = static_cast<double>(fe[c]);
+    for (int k = 1; k < P; ++k) {
+      const float2 o = s_part[k][c][lane];
+      two_sum_acc(fs, fe, o.x);
+      fe += o.y;
     }
+    sum = static_cast<double>(fs) + static_cast<double>(fe);
   }
-  double jtw[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) jtw[c] = s[c] + e[c];
-  const double gsum = s[3] + e[3];
-  if (!finite3(jtw[0], jtw[1], jtw[2]) || !isfinite(gsum)) atomicOr(a.flags, kFlagNonFinite);
-  a.gm[p] += -a.G * gsum;
-  double rho[3], nu[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    rho[c] = a.rho[c * N + p] + jtw[c];
-    a.rho[c * N + p] = rho[c];
-    nu[c] = a.nu[c * N + p];
+  if (!live) return;
+  if (!isfinite(sum)) atomicOr(a.flags, kFlagNonFinite);
+  if (c == 3) {
+    a.gm[p] += -a.G * sum;
+    return;
   }
+  const double rho = a.rho[c * N + p] + sum, nu = a.nu[c * N + p];
+  a.rho[c * N + p] = rho;
   if (a.mode == 2) return;
-  double w[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const double nun = fma(a.dt, rho[c], nu[c]);               // nu' = nu + dt rho
-    const double al = fma(a.half_dt2, rho[c], a.half_dt * nu[c]);  // alpha' = dt/2 nu + dt^2/2 rho
-    a.nu[c * N + p] = nun;
-    w[c] = a.mode == 0 ? fma(a.half_dt, nun, al) : al;         // next w
-  }
+  const double nun = fma(a.dt, rho, nu);                  // nu' = nu + dt rho
+  const double al = fma(a.half_dt2, rho, a.half_dt * nu);  // alpha' = dt/2 nu + dt^2/2 rho
+  a.nu[c * N + p] = nun;
+  const double w = a.mode == 0 ? fma(a.half_dt, nun, al) : al;  // next w
   const int q = a.qidx ? a.qidx[p] : p;
   if (PREC == 0)
-    static_cast<double4_32a *>(a.w)[q] = make_double4_32a(w[0], w[1], w[2], 0.0);
+    static_cast<double *>(a.w)[4 * static_cast<size_t>(q) + c] = w;  // (w's fourth entry is never read)
   else
-    w_pair_store(a.w, q, static_cast<float>(w[0]), static_cast<float>(w[1]), static_cast<float>(w[2]));
+    static_cast<float *>(a.w)[8 * static_cast<size_t>(q >> 1) + (q & 1) + 2 * c] = static_cast<float>(w);
 }
 
 // rho = dL/dr_T, nu = dL/dv_T (or 0), g_m = 0, and the first w = dt/2 nu
@@ -416,11 +428,11 @@ cudaError_t launch_vjp(int precision, int grid, size_t smem, const VjpArgs &a, c
 
 cudaError_t launch_adjoint(int precision, const AdjArgs &a, cudaStream_t s) {
   if (a.N <= 0) return cudaSuccess;
-  const int grid = (a.N + 255) / 256;
+  const int grid = (a.N + 31) / 32;
   if (precision == 0)
-    adjoint_kernel<0><<<grid, 256, 0, s>>>(a);
+    adjoint_kernel<0><<<grid, AdjShape<0>::kThreads, 0, s>>>(a);
   else
-    adjoint_kernel<1><<<grid, 256, 0, s>>>(a);
+    adjoint_kernel<1><<<grid, AdjShape<1>::kThreads, 0, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -13,8 +13,8 @@ struct Seed {
 };
 }  // namespace
 
-// out[i] = mu[i] |d_i|^-3; taken[i] = whether the integer path takes the pair.
-extern "C" void ic_factors(int64_t n, const double *dx, const double *dy, const double *dz, const double *mu,
+// out[i] = mu[i] |d_i|^-power (power 1, 2 or 3); taken[i] = whether the integer path takes the pair.
+extern "C" void ic_factors(int64_t n, int32_t power, const double *dx, const double *dy, const double *dz, const double *mu,
                            const double *off, double *out, int32_t *taken) {
   using namespace nb::ic;
   for (int64_t i = 0; i < n; ++i) {
@@ -22,7 +22,12 @@ extern "C" void ic_factors(int64_t n, const double *dx, const double *dy, const 
     const Mass m = pack_mass(mu[i]);
     taken[i] = exp_in_range(em) && mass_in_range(m);
     if (!taken[i]) continue;
-    out[i] = mass_times(m, inv_cube(square_sum(dx[i], dy[i], dz[i], em), em, Seed{off[i]}));
+    const uint64_t R = square_sum(dx[i], dy[i], dz[i], em);
+    const Seed seed{off[i]};
+    const CubeSquare c = inv_cube_square(R, em, seed);
+    out[i] = mass_times(m, power == 3 ? c.cube : power == 2 ? c.square : inv_dist(R, em, seed));
+    const Cube q = inv_cube(R, em, seed);
+    if (q.lo != c.cube.lo || q.hi != c.cube.hi || q.e != c.cube.e) taken[i] = -2;
     if (unpack_mass(m) != mu[i]) taken[i] = -1;
   }
 }
