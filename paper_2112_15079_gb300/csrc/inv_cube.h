@@ -6,7 +6,8 @@
 // factors mu_j |d|^-3, mu_i |d|^-3 -- |d|^2, the reciprocal cube and the two
 // mass products, 11 of a pair's 20 FP64 operations -- is therefore done in
 // 64-bit fixed point, about 120 integer instructions, which run beside the
-// 9 FP64 operations that are left (3 differences, 6 accumulations).
+// 9 FP64 operations that are left (3 differences, 6 accumulations).  The
+// differences too can be had in fixed point (further below).
 //
 // Method (own derivation; the numbers are integers, errors in brackets are
 // relative):
@@ -235,8 +236,8 @@ NB_HD Cube normalised(uint64_t S, int32_t e) {
   return c;
 }
 
-// |d|^-3, step (5).
-NB_HD Cube cube_of(const Root &o, uint32_t em20) {
+// |d|^-3, step (5); em: the exponent field of |d|'s largest component.
+NB_HD Cube cube_of(const Root &o, uint32_t em) {
   const int64_t g = static_cast<int64_t>(o.q) * 30 - (o.ne + (o.ne >> 1));  // 3e/2 + 15e^2/8 in units of 2^-70
   uint64_t T = wide(o.Y, o.tl);  // Y^3
   T += static_cast<uint64_t>(o.Y * o.th) << 32;
@@ -248,11 +249,11 @@ NB_HD Cube cube_of(const Root &o, uint32_t em20) {
   V += mulhi(Th, gl);
   V += 2 * static_cast<int64_t>(mulhi_s(static_cast<int32_t>(Tl >> 1), gh));
   return normalised(T + static_cast<uint64_t>(V >> 6),
-                    3065 + static_cast<int32_t>(o.k + (o.k >> 1)) - 3 * static_cast<int32_t>(em20 >> 20));
+                    3065 + static_cast<int32_t>(o.k + (o.k >> 1)) - 3 * static_cast<int32_t>(em));
 }
 template <class Rsq>
 NB_HD Cube inv_cube(uint64_t R, uint32_t em20, const Rsq &rsq) {
-  return cube_of(inv_root(R, rsq), em20);
+  return cube_of(inv_root(R, rsq), em20 >> 20);
 }
 
 // |d|^-3 and |d|^-2 of one difference: R^-1 = 2^-102 Y^2 (1 - e)^-1 = 2^-102 Y^2 (1 + e +
@@ -271,7 +272,7 @@ template <class Rsq>
 NB_HD CubeSquare inv_cube_square(uint64_t R, uint32_t em20, const Rsq &rsq) {
   const Root o = inv_root(R, rsq);
   CubeSquare r;
-  r.cube = cube_of(o, em20);
+  r.cube = cube_of(o, em20 >> 20);
   const uint64_t t = make64(o.tl, o.th);  // <= 2^42
   const int64_t g = static_cast<int64_t>(o.q) * 16 - o.ne;  // e + e^2 in units of 2^-70
   const uint64_t S = (t << 20) + static_cast<uint64_t>(mulhi64(static_cast<int64_t>(t << 14), g));  // 2^20 t (1 + g)
@@ -304,6 +305,84 @@ NB_HD double mass_times(const Mass &m, const Cube &c) {
   const uint32_t lo = fshr(lo32(M), hi32(M), 10);
   const uint32_t hi = (hi32(M) >> 10) + ((static_cast<uint32_t>(c.e) + (m.w & 0x7ffu) + b) << 20);
   return from_bits(lo, m.u ? hi : 0u);
+}
+
+// ---------------------------------------------------------------------------
+// Differences in fixed point.  Within a pair of 32-body tiles the coordinates
+// become integers X = x 2^(1083 - E), E the largest exponent field among them, so
+// |X| < 2^61, exact for a coordinate within 2^-8 of the largest and within half
+// a unit otherwise.  D = Xj - Xi then gives the difference to one unit, at most
+// 2^-54 of |d| where its largest component is at least 2^54 units (FP64's own
+// rounding: 2^-53), already aligned for the square sum, and rounds once more to
+// FP64 for the accumulations -- without the FP64 pipe.  Closer pairs, and
+// those with a component below 2^-30 of the largest, are left to FP64.
+// ---------------------------------------------------------------------------
+
+// Exponent fields E for which every difference taken is in the range above.
+NB_HD bool fix_in_range(uint32_t E) { return E - (kDExpMin + 8) <= kDExpSpan - 16; }
+
+NB_HD int64_t to_fix(double x, uint32_t E) {
+  const uint64_t b = bits(x);
+  const uint32_t hi = hi32(b), ex = (hi >> 20) & 0x7ffu;
+  const uint32_t s = E - ex < 63u ? E - ex : 63u;
+  const uint64_t m = make64(lo32(b), (hi & 0x000fffffu) | 0x00100000u);  // (a subnormal x: shifted out)
+  const int64_t v = static_cast<int64_t>((((m << 9) >> s) + 1) >> 1);
+  return static_cast<int32_t>(hi) < 0 ? -v : v;
+}
+
+// A difference from fixed point: magnitudes (h, l) with the largest h in
+// [2^29, 2^30), signs, em as above; ok false where FP64 has to take it.
+struct FixDiff {
+  uint32_t h[3], l[3], sign[3];
+  uint32_t em;
+  bool ok;
+};
+NB_HD FixDiff fix_diff(const int64_t (&xj)[3], const int64_t (&xi)[3], uint32_t E) {
+  FixDiff f;
+  uint32_t mx = 0u, mn = ~0u;
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+  for (int c = 0; c < 3; ++c) {
+    const int64_t d = xj[c] - xi[c];
+    const int64_t s = d >> 63;
+    const uint64_t a = static_cast<uint64_t>((d ^ s) - s);
+    f.sign[c] = hi32(static_cast<uint64_t>(s)) & 0x80000000u;
+    f.h[c] = hi32(a);
+    f.l[c] = lo32(a);
+    mx = f.h[c] > mx ? f.h[c] : mx;
+  }
+  f.ok = mx >= (1u << 22);
+  const uint32_t n = clz32(mx), s = n - 2u;  // (|D| < 2^62: n >= 2)
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+  for (int c = 0; c < 3; ++c) {
+    f.h[c] = fshl(f.l[c], f.h[c], s);
+    f.l[c] <<= s & 31u;
+    mn = f.h[c] < mn ? f.h[c] : mn;
+  }
+  f.ok = f.ok && mn != 0u;
+  f.em = E + 3u - n;
+  return f;
+}
+NB_HD uint64_t square_sum(const FixDiff &f) {
+  uint64_t R = 0, C = uint64_t(3) << 30;
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+  for (int c = 0; c < 3; ++c) {
+    R += wide(f.h[c], f.h[c]);
+    C += wide(f.h[c], f.l[c]);
+  }
+  return R + (C >> 31);
+}
+// Component c, rounded to FP64.
+NB_HD double fix_value(const FixDiff &f, int c) {
+  const uint32_t m = clz32(f.h[c]), s = m - 1u;  // (2 <= m < 32)
+  const uint64_t v = make64(f.l[c] << (s & 31u), fshl(f.l[c], f.h[c], s)) + 0x200u;  // leading one at bit 62
+  const uint32_t hi = (hi32(v) >> 10) + ((f.em + 1u - m) << 20);
+  return from_bits(fshr(lo32(v), hi32(v), 10), hi | f.sign[c]);
 }
 
 }  // namespace ic

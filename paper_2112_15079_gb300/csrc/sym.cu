@@ -3,12 +3,12 @@
 // The FP64 pipe bounds this path (an operation of a warp every 76 cycles per
 // SM sub-partition).  The pair (p, j) and its reaction share the difference
 // and |d|^-3, so evaluating each unordered pair once takes 20 FP64 operations
-// for two interactions; |d|^2, |d|^-3 and the mass products, 11 of them, run
-// on the integer pipes (inv_cube.h), about 120 instructions beside the 9 FP64
-// operations that are left: 3 differences and 6 accumulations.  Measured on
-// GB300, 10,425 bodies: 2.03 ms per step with 20 FP64 operations, 0.94 ms
-// with 9 (9 x 76 cycles a pair and warp step is 0.92 ms: the FP64 pipe stays
-// the bound).
+// for two interactions.  |d|^2, |d|^-3 and the mass products, 11 of them, and
+// the differences run on the integer pipes (inv_cube.h), about 170
+// instructions beside the 6 FP64 accumulations that are left.  Measured on
+// GB300, 10,425 bodies: 2.03 ms per step with 20 FP64 operations, 0.94 ms with
+// 9 (FP64 differences), 0.67 ms with 6 (the launch 0.60 ms, 6 x 76 cycles a pair
+// and warp step: the FP64 pipe stays the bound).
 //
 // Decomposition: each system's bodies are cut into blocks of 64 (two warp
 // tiles of 32); the work items are the block pairs (I, J), I <= J, handed
@@ -78,56 +78,111 @@ __device__ __forceinline__ void sym_pair_int(double xi, double yi, double zi, co
 // rotated once around the warp; (ax, ay, az) take the targets' sums, (bx, by,
 // bz) return the sources' reaction sums, each in its source's own lane.
 // SELF: the tile with itself, offsets 1..15 both ways and 16 one way (lanes L
-// and L + 16 meet twice).  The sources are rotated a step ahead.  Masses
-// beyond the integer path's range (never in a physical model) take the FP64
-// arithmetic for the whole tile pair.
+// and L + 16 meet twice).  ri, rj: whether this lane's target and source are
+// real bodies of the system.
+//
+// The differences are taken in fixed point (inv_cube.h), which leaves 6 FP64
+// operations to a pair, the accumulations; pairs too close for it take 3
+// FP64 differences (their sources' coordinates come from their own lanes, so
+// the whole warp takes part).  A tile pair with many of them (planets among
+// their moons: after kCloseSteps steps that had one), or with magnitudes
+// beyond the fixed-point range, goes on with FP64 differences throughout,
+// and masses beyond the integer range (never in a physical model) take the
+// FP64 series.
+constexpr int kCloseSteps = 3;
+
 template <bool SELF>
-__device__ __forceinline__ void sym_tile(const double4_32a &pi, const double4_32a &pj, int lane, double &ax,
-                                         double &ay, double &az, double &bx, double &by, double &bz) {
-  double xj = pj.x, yj = pj.y, zj = pj.z;
+__device__ __forceinline__ void sym_tile(const double4_32a &pi, const double4_32a &pj, bool ri, bool rj, int lane,
+                                         double &ax, double &ay, double &az, double &bx, double &by, double &bz) {
+  constexpr int kFirst = SELF ? 1 : 0, kEnd = SELF ? 17 : 32;
   bx = by = bz = 0.0;
   const int src = (lane + 1) & 31;
   auto rotate = [&]() {
-    xj = __shfl_sync(0xffffffffu, xj, src);
-    yj = __shfl_sync(0xffffffffu, yj, src);
-    zj = __shfl_sync(0xffffffffu, zj, src);
     bx = __shfl_sync(0xffffffffu, bx, src);
     by = __shfl_sync(0xffffffffu, by, src);
     bz = __shfl_sync(0xffffffffu, bz, src);
   };
-  if (__all_sync(0xffffffffu, mass_fits(pi.w) && mass_fits(pj.w))) {
+  const uint32_t ei = ri ? ic::max_exp(pi.x, pi.y, pi.z) : 0u, ej = rj ? ic::max_exp(pj.x, pj.y, pj.z) : 0u;
+  const uint32_t E = __reduce_max_sync(0xffffffffu, max(ei, ej)) >> 20;
+  const bool masses = __all_sync(0xffffffffu, mass_fits(pi.w) && mass_fits(pj.w));
+  int k = kFirst;
+  if (masses && ic::fix_in_range(E)) {
     const ic::Mass mi = ic::pack_mass(pi.w);
     ic::Mass mj = ic::pack_mass(pj.w);
-    auto rotate_mass = [&]() {
+    // (a lane outside the system: beyond every body of the tiles, massless)
+    const int64_t pad = int64_t(1) << 61;
+    const int64_t xi[3] = {ri ? ic::to_fix(pi.x, E) : pad, ri ? ic::to_fix(pi.y, E) : pad,
+                           ri ? ic::to_fix(pi.z, E) : pad};
+    int64_t xj[3] = {rj ? ic::to_fix(pj.x, E) : pad, rj ? ic::to_fix(pj.y, E) : pad, rj ? ic::to_fix(pj.z, E) : pad};
+    auto rotate_source = [&]() {
+      xj[0] = __shfl_sync(0xffffffffu, xj[0], src);
+      xj[1] = __shfl_sync(0xffffffffu, xj[1], src);
+      xj[2] = __shfl_sync(0xffffffffu, xj[2], src);
       mj.u = __shfl_sync(0xffffffffu, mj.u, src);
       mj.w = __shfl_sync(0xffffffffu, mj.w, src);
     };
-    if (SELF) {
-#pragma unroll 1
-      for (int k = 1; k <= 16; ++k) {
-        rotate();
-        rotate_mass();
-        sym_pair_int(pi.x, pi.y, pi.z, mi, xj, yj, zj, mj, ax, ay, az, bx, by, bz, k < 16);
-      }
-    } else {
+    int close = 0;  // steps that had a close pair
 #pragma unroll 2
-      for (int k = 0; k < 32; ++k) {
-        sym_pair_int(pi.x, pi.y, pi.z, mi, xj, yj, zj, mj, ax, ay, az, bx, by, bz, true);
-        rotate();
-        rotate_mass();
-      }
-    }
-  } else {
-    double mj = pj.w;
-    for (int k = SELF ? 1 : 0; k < (SELF ? 17 : 32); ++k) {
+    for (; k < kEnd && close < kCloseSteps; ++k) {
       if (SELF) {
         rotate();
-        mj = __shfl_sync(0xffffffffu, mj, src);
+        rotate_source();
       }
-      sym_pair(pi.x, pi.y, pi.z, pi.w, xj, yj, zj, mj, ax, ay, az, bx, by, bz, !SELF || k < 16);
+      const ic::FixDiff f = ic::fix_diff(xj, xi, E);
+      double dx = ic::fix_value(f, 0), dy = ic::fix_value(f, 1), dz = ic::fix_value(f, 2);
+      const ic::Cube c = ic::cube_of(ic::inv_root(ic::square_sum(f), ic::Rsqrt{}), f.em);
+      double fj = ic::mass_times(mj, c), fi = ic::mass_times(mi, c);
+      if (__any_sync(0xffffffffu, !f.ok)) {
+        ++close;
+        const int from = (lane + k) & 31;
+        const double sx = __shfl_sync(0xffffffffu, pj.x, from), sy = __shfl_sync(0xffffffffu, pj.y, from),
+                     sz = __shfl_sync(0xffffffffu, pj.z, from);
+        if (!f.ok) {
+          dx = sx - pi.x;
+          dy = sy - pi.y;
+          dz = sz - pi.z;
+          pair_factors(dx, dy, dz, mj, mi, fj, fi);
+        }
+      }
+      ax = fma(fj, dx, ax);
+      ay = fma(fj, dy, ay);
+      az = fma(fj, dz, az);
+      if (!SELF || k < 16) {
+        bx = fma(-fi, dx, bx);
+        by = fma(-fi, dy, by);
+        bz = fma(-fi, dz, bz);
+      }
       if (!SELF) {
         rotate();
-        mj = __shfl_sync(0xffffffffu, mj, src);
+        rotate_source();
+      }
+    }
+  }
+  if (k < kEnd) {
+    const int at = (lane + k - kFirst) & 31;  // the source here before step k
+    double xj = __shfl_sync(0xffffffffu, pj.x, at), yj = __shfl_sync(0xffffffffu, pj.y, at),
+           zj = __shfl_sync(0xffffffffu, pj.z, at), wj = __shfl_sync(0xffffffffu, pj.w, at);
+    auto rotate_source = [&]() {
+      xj = __shfl_sync(0xffffffffu, xj, src);
+      yj = __shfl_sync(0xffffffffu, yj, src);
+      zj = __shfl_sync(0xffffffffu, zj, src);
+      wj = __shfl_sync(0xffffffffu, wj, src);
+    };
+    const ic::Mass mi = ic::pack_mass(pi.w);
+#pragma unroll 1
+    for (; k < kEnd; ++k) {
+      if (SELF) {
+        rotate();
+        rotate_source();
+      }
+      const bool react = !SELF || k < 16;
+      if (masses)
+        sym_pair_int(pi.x, pi.y, pi.z, mi, xj, yj, zj, ic::pack_mass(wj), ax, ay, az, bx, by, bz, react);
+      else
+        sym_pair(pi.x, pi.y, pi.z, pi.w, xj, yj, zj, wj, ax, ay, az, bx, by, bz, react);
+      if (!SELF) {
+        rotate();
+        rotate_source();
       }
     }
   }
@@ -163,10 +218,11 @@ __global__ void __launch_bounds__(kSymThreads) force_sym_kernel(const SymArgs a)
       double bx = 0.0, by = 0.0, bz = 0.0;
       if (!(I == J && t < w)) {  // tile pair (w, t) with t < w of a diagonal item is (t, w), warp t's
         const double4_32a pj0 = sym_load(a.cur, sb, J * kSymBlock + t * 32 + lane, ns, 1e15 * (lane + 1) + 5e14);
+        const bool ri = I * kSymBlock + w * 32 + lane < ns, rj = J * kSymBlock + t * 32 + lane < ns;
         if (I == J && t == w)
-          sym_tile<true>(pi, pj0, lane, ax, ay, az, bx, by, bz);
+          sym_tile<true>(pi, pj0, ri, rj, lane, ax, ay, az, bx, by, bz);
         else
-          sym_tile<false>(pi, pj0, lane, ax, ay, az, bx, by, bz);
+          sym_tile<false>(pi, pj0, ri, rj, lane, ax, ay, az, bx, by, bz);
       }
       s_b[w][t][0][lane] = bx;
       s_b[w][t][1][lane] = by;
@@ -259,10 +315,11 @@ __global__ void __launch_bounds__(kSymWideThreads) force_sym_wide_kernel(const S
         if (t + 1 < T) pn = sym_load(a.cur, sb, j0 + qn * 32 + lane, ns, 1e15 * (lane + 1) + 5e14);
         if (p_live && j0 + q * 32 < ns && !(diag && q < p)) {  // (q < p on a diagonal item: tile q's warp's pair)
           double tx = 0.0, ty = 0.0, tz = 0.0, bx, by, bz;
+          const bool ri = i0 + p * 32 + lane < ns, rj = j0 + q * 32 + lane < ns;
           if (diag && q == p)
-            sym_tile<true>(pi, pj0, lane, tx, ty, tz, bx, by, bz);
+            sym_tile<true>(pi, pj0, ri, rj, lane, tx, ty, tz, bx, by, bz);
           else
-            sym_tile<false>(pi, pj0, lane, tx, ty, tz, bx, by, bz);
+            sym_tile<false>(pi, pj0, ri, rj, lane, tx, ty, tz, bx, by, bz);
           ax += tx;
           ay += ty;
           az += tz;

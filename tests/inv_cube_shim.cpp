@@ -31,3 +31,23 @@ extern "C" void ic_factors(int64_t n, int32_t power, const double *dx, const dou
     if (unpack_mass(m) != mu[i]) taken[i] = -1;
   }
 }
+
+// Fixed-point differences xj - xi (three components each, [3][n]) at the
+// exponent field E[i]: out[c][i], the factor |d|^-3 in cube[i], and whether the
+// pair is taken.
+extern "C" void ic_differences(int64_t n, const double *xi, const double *xj, const int32_t *E, double *out,
+                               double *cube, int32_t *taken) {
+  using namespace nb::ic;
+  for (int64_t i = 0; i < n; ++i) {
+    int64_t a[3], b[3];
+    for (int c = 0; c < 3; ++c) {
+      a[c] = to_fix(xi[c * n + i], static_cast<uint32_t>(E[i]));
+      b[c] = to_fix(xj[c * n + i], static_cast<uint32_t>(E[i]));
+    }
+    const FixDiff f = fix_diff(b, a, static_cast<uint32_t>(E[i]));
+    taken[i] = fix_in_range(static_cast<uint32_t>(E[i])) && f.ok;
+    if (!taken[i]) continue;
+    for (int c = 0; c < 3; ++c) out[c * n + i] = fix_value(f, c);
+    cube[i] = mass_times(pack_mass(1.0), cube_of(inv_root(square_sum(f), Rsqrt{}), f.em));
+  }
+}

@@ -345,3 +345,31 @@ def test_mixed_small_systems_take_blocks(nb, sizes, want):
         ref, t = oracle.accel(inputs.G_AU_DAY, x, w, openmp=True), oracle.term_norm(inputs.G_AU_DAY, x, w)
         err = np.linalg.norm(a[:, b:e] - ref, axis=0)
         assert np.all(err <= 2e-6 * t)
+
+
+@pytest.mark.parametrize("block", [64, 256])
+@pytest.mark.parametrize("kind", ["flat", "tight cluster", "cluster far from the origin", "one outlier"])
+def test_pairs_left_to_fp64_differences(nb, block, kind):
+    """Configurations in which many pairs, or all, leave the fixed-point
+    differences (a component that vanishes; bodies much closer to each other
+    than to the origin or to an outlier that sets the scale): the FP64 gate on
+    every body, at a ragged size."""
+    rng = np.random.default_rng(8)
+    n = 1300
+    r = rng.normal(size=(3, n))
+    if kind == "flat":
+        r[2] = 0.0
+    elif kind == "tight cluster":
+        r[:, :200] *= 1e-6
+    elif kind == "cluster far from the origin":
+        r += 2.0**14
+    else:
+        r[:, 5] = 1e7
+    m = rng.uniform(0.1, 1.0, n)
+    m[::7] = 0.0
+    b = nb.NBody(r, 0 * r, m, G=1.0, dt=1e-9, precision="fp64", small=False, pair_once_block=block)
+    a = b.accel().cpu().numpy()
+    b.close()
+    # (the sums of a random cluster cancel: relative to the terms' magnitudes)
+    err = np.linalg.norm(a - oracle.accel(1.0, r, m, openmp=True), axis=0) / oracle.term_norm(1.0, r, m, openmp=True)
+    assert err.max() <= 1e-13

@@ -35,6 +35,14 @@ def ic(tmp_path_factory):
                     os.path.join(HERE, "inv_cube_shim.cpp"), "-o", out], check=True)
     lib = ctypes.CDLL(out)
 
+    def differences(xi, xj, E):
+        xi, xj, E = np.ascontiguousarray(xi), np.ascontiguousarray(xj), np.ascontiguousarray(E, dtype=np.int32)
+        n = E.shape[0]
+        d, cube, taken = np.zeros((3, n)), np.zeros(n), np.zeros(n, dtype=np.int32)
+        P = lambda a: a.ctypes.data_as(ctypes.c_void_p)  # noqa: E731
+        lib.ic_differences(ctypes.c_int64(n), P(xi), P(xj), P(E), P(d), P(cube), P(taken))
+        return d, cube, taken == 1
+
     def factors(d, mu, off, power=3):
         d, mu, off = (np.ascontiguousarray(t, dtype=np.float64) for t in (d, mu, off))
         n = mu.shape[0]
@@ -42,6 +50,7 @@ def ic(tmp_path_factory):
         P = lambda a: a.ctypes.data_as(ctypes.c_void_p)  # noqa: E731
         lib.ic_factors(ctypes.c_int64(n), ctypes.c_int32(power), P(d[0]), P(d[1]), P(d[2]), P(mu), P(off), P(res), P(taken))
         return res, taken
+    factors.differences = differences
     return factors
 
 
@@ -96,3 +105,50 @@ def test_massless_gives_zero(ic):
 def test_left_to_the_series(ic, d, mu):
     _, taken = ic(np.array([[0.0], [d], [0.0]]), np.array([mu]), np.zeros(1))
     assert taken[0] == 0
+
+
+@pytest.mark.parametrize("kind", ["any", "near the origin", "pairs far from it", "flat", "another body sets the scale"])
+def test_fixed_point_differences(ic, kind):
+    """x in units of 2^(E - 1083) (exact within 2^-8 of the largest coordinate,
+    half a unit else) gives a difference within one unit, 2^-54 of its largest
+    component at least, plus the rounding to FP64, 2^-53 of each component:
+    1.5 x 2^-53 of the largest.  |d|^-3 then is off by 3 x sqrt(3) 2^-54 at
+    most, plus its own 0.77 units in the last place."""
+    if np.finfo(np.longdouble).nmant < 63:
+        pytest.skip("no extended precision here")
+    rng = np.random.default_rng(9)
+    n = 300_000
+    scale = np.exp2(rng.integers(-150, 150, n).astype(float))
+    xi, xj = rng.uniform(-1, 1, (3, n)) * scale, rng.uniform(-1, 1, (3, n)) * scale
+    if kind == "near the origin":
+        xi *= np.exp2(-rng.uniform(0, 30, (3, n)))
+    elif kind == "pairs far from it":
+        xj = xi + xj * np.exp2(-rng.uniform(0, 12, n))
+    elif kind == "flat":
+        xi[2] = xj[2] = 0.0
+    # the field of the largest coordinate, or of a further body's
+    E = np.frexp(np.abs(np.concatenate([xi, xj])).max(0))[1] + 1022
+    if kind == "another body sets the scale":
+        E = E + rng.integers(0, 7, n)
+    got, cube, ok = ic.differences(xi, xj, E)
+    if kind == "flat":
+        assert not ok.any()  # a component below 2^-30 of the largest: left to FP64
+        return
+    assert ok.mean() > (0.2 if kind in ("pairs far from it", "another body sets the scale") else 0.9)
+    want = xj.astype(np.longdouble) - xi.astype(np.longdouble)
+    big = np.abs(want).max(0)
+    assert (np.abs(got - want) / big)[:, ok].max() <= 1.5 * 2.0**-53
+    r2 = (want * want).sum(0)
+    ref = (1 / (r2 * np.sqrt(r2)))[ok]
+    err = np.abs((cube[ok] - ref) / ref).astype(float)
+    assert err.max() <= 3 * np.sqrt(3) * 2.0**-54 + 0.77 * 2.0**-52
+
+
+def test_fixed_point_leaves_close_pairs(ic):
+    one, E = np.ones((3, 1)), np.array([1023])
+    near = one * (1 + 2.0**-9)   # closer than 2^-7 of the scale
+    far = one * np.array([[-1.0], [0.5], [0.25]])
+    assert not ic.differences(one, near, E)[2][0]
+    assert ic.differences(one, far, E)[2][0]
+    assert not ic.differences(one, far, np.array([1023 - 195]))[2][0]  # a scale beyond the range
+    assert not ic.differences(one, one, E)[2][0]
