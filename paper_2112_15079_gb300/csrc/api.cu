@@ -642,6 +642,18 @@ nb::ForceArgs force_args(nbody_ctx *c, const void *cur) {
   return a;
 }
 
+// Whether the per-body kernel lets the next kernel launch at once.  With one
+// force CTA per SM the next force grid lands evenly however early it comes.
+// On the mixed path the next kernel is the tiny box kernel, so it may always
+// come early, and does where that measured faster on GB300: pair-once items
+// are handed out dynamically (2,131 bodies 12.8 -> 11.8 us per step), and up
+// to 2,048 bodies the launches dominate (1,500: 15.7 -> 15.2); with larger
+// static shares it costs a little (6,001: 31.3 -> 31.8).
+int release_early(const nbody_ctx *c) {
+  const bool mixed = c->o.precision == NBODY_MIXED;
+  return c->fw.occ == 1 || (mixed && (c->fw.sym_pairs || c->N <= 2048)) ? 1 : 0;
+}
+
 nb::VerletArgs verlet_args(nbody_ctx *c, const State &s, const void *cur, void *nxt, int mode) {
   const size_t N = c->N;
   nb::VerletArgs a{};
@@ -660,7 +672,7 @@ nb::VerletArgs verlet_args(nbody_ctx *c, const State &s, const void *cur, void *
   a.p_begin = c->sh_world > 0 ? static_cast<int32_t>(c->sh_begin) : 0;  // a row shard completes its own bodies
   a.p_end = c->sh_world > 0 ? static_cast<int32_t>(c->sh_end) : c->N;
   a.mode = mode;
-  a.release_early = c->fw.occ == 1 ? 1 : 0;
+  a.release_early = release_early(c);
   a.dt = c->o.dt;
   a.half_dt = 0.5 * c->o.dt;
   a.half_dt2 = 0.5 * c->o.dt * c->o.dt;
@@ -684,7 +696,7 @@ nb::RkArgs rk_args(nbody_ctx *c, const State &s, const void *cur, void *nxt, int
   a.flags = c->flags;
   a.N = c->N;
   a.stage = stage;
-  a.release_early = c->fw.occ == 1 ? 1 : 0;
+  a.release_early = release_early(c);
   a.G = c->o.G;
   a.dt = c->o.dt;
   return a;

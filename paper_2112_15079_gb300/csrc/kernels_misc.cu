@@ -262,10 +262,9 @@ __device__ __forceinline__ void stage_position(void *nxt, int q, size_t o, doubl
 
 template <int PREC, int MODE>  // MODE: kModeForce, kModeStep or kModeLeapfrog (a.mode)
 __global__ void __launch_bounds__(VerletShape<PREC>::kBlock) verlet_kernel(const VerletArgs a) {
-  // When at most one force CTA fits on an SM, the next force grid can only
-  // land one CTA per SM, however early it launches: let it launch now, so its
-  // launch overlaps this kernel (its own griddepcontrol.wait still waits for
-  // our completion).  Otherwise release only at the end (below).
+  // Where the host says so the next kernel may launch now, so that its launch
+  // overlaps this kernel (its own griddepcontrol.wait still waits for our
+  // completion).  Otherwise release only at the end (below).
   if (a.release_early) grid_dependency_launch();
   typedef typename std::conditional<PREC == 0, double, float>::type T;
   constexpr int L = VerletShape<PREC>::kLanes, NB = VerletShape<PREC>::kBodies;

@@ -66,7 +66,7 @@ struct VerletArgs {
   int32_t N;
   int32_t p_begin, p_end;  // the bodies this launch completes: [p_begin, p_end) (all: 0, N)
   int32_t mode;
-  int32_t release_early;  // 1: the next force grid may launch at once (it fits one CTA per SM)
+  int32_t release_early;  // 1: the next kernel may launch at once
   double dt, half_dt, half_dt2;
 };
 
