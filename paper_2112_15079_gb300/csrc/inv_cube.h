@@ -309,57 +309,99 @@ NB_HD double mass_times(const Mass &m, const Cube &c) {
 
 // ---------------------------------------------------------------------------
 // Differences in fixed point.  Within a pair of 32-body tiles the coordinates
-// become integers X = x 2^(1083 - E), E the largest exponent field among them, so
-// |X| < 2^61, exact for a coordinate within 2^-8 of the largest and within half
-// a unit otherwise.  D = Xj - Xi then gives the difference to one unit, at most
-// 2^-54 of |d| where its largest component is at least 2^54 units (FP64's own
-// rounding: 2^-53), already aligned for the square sum, and rounds once more to
-// FP64 for the accumulations -- without the FP64 pipe.  Closer pairs, and
-// those with a component below 2^-30 of the largest, are left to FP64.
+// become 96-bit integers X = x 2^(1115 - E), E the largest exponent field among
+// them, so |X| < 2^93: exact for a coordinate of at least 2^-40 of the largest,
+// to one unit otherwise.  D = Xj - Xi is the difference, exact or within 2^-92
+// of the tiles' largest coordinate; its upper 64 bits, shifted, are the
+// aligned components that the square sum takes, and each component rounds
+// once to FP64 for the accumulations -- without the FP64 pipe and as exact as
+// its subtraction (64-bit integers are not: a component much smaller than
+// the others then loses bits that FP64 keeps).  Pairs closer than 2^-7 of the
+// scale, and those with a component below 2^-30 of the largest, are left to
+// FP64.
 // ---------------------------------------------------------------------------
 
 // Exponent fields E for which every difference taken is in the range above.
 NB_HD bool fix_in_range(uint32_t E) { return E - (kDExpMin + 8) <= kDExpSpan - 16; }
 
-NB_HD int64_t to_fix(double x, uint32_t E) {
+struct Fix {
+  uint32_t w[3];  // two's complement, w[2] the uppermost
+};
+NB_HD Fix fix_of(unsigned __int128 v) {
+  Fix f;
+  f.w[0] = static_cast<uint32_t>(v);
+  f.w[1] = static_cast<uint32_t>(v >> 32);
+  f.w[2] = static_cast<uint32_t>(v >> 64);
+  return f;
+}
+// Beyond every coordinate: the place of a lane outside the system.
+NB_HD Fix fix_pad() { return fix_of(static_cast<unsigned __int128>(1) << 93); }
+
+NB_HD Fix to_fix(double x, uint32_t E) {
   const uint64_t b = bits(x);
-  const uint32_t hi = hi32(b), ex = (hi >> 20) & 0x7ffu;
-  const uint32_t s = E - ex < 63u ? E - ex : 63u;
+  const uint32_t hi = hi32(b), s = E - ((hi >> 20) & 0x7ffu);
   const uint64_t m = make64(lo32(b), (hi & 0x000fffffu) | 0x00100000u);  // (a subnormal x: shifted out)
-  const int64_t v = static_cast<int64_t>((((m << 9) >> s) + 1) >> 1);
-  return static_cast<int32_t>(hi) < 0 ? -v : v;
+  const unsigned __int128 v = s <= 40u ? static_cast<unsigned __int128>(m) << (40u - s) : s < 104u ? m >> (s - 40u) : 0u;
+  return fix_of(static_cast<int32_t>(hi) < 0 ? -v : v);
 }
 
-// A difference from fixed point: magnitudes (h, l) with the largest h in
+// a - b, and |a - b| with the sign in *neg (all ones if negative).
+NB_HD void fix_abs_diff(const Fix &a, const Fix &b, uint32_t (&m)[3], uint32_t *neg) {
+#ifdef __CUDA_ARCH__
+  uint32_t d0, d1, d2;
+  asm("sub.cc.u32 %0, %3, %6;\n\tsubc.cc.u32 %1, %4, %7;\n\tsubc.u32 %2, %5, %8;"
+      : "=r"(d0), "=r"(d1), "=r"(d2)
+      : "r"(a.w[0]), "r"(a.w[1]), "r"(a.w[2]), "r"(b.w[0]), "r"(b.w[1]), "r"(b.w[2]));
+  const uint32_t s = static_cast<uint32_t>(static_cast<int32_t>(d2) >> 31);
+  asm("sub.cc.u32 %0, %3, %6;\n\tsubc.cc.u32 %1, %4, %6;\n\tsubc.u32 %2, %5, %6;"
+      : "=r"(m[0]), "=r"(m[1]), "=r"(m[2])
+      : "r"(d0 ^ s), "r"(d1 ^ s), "r"(d2 ^ s), "r"(s));
+  *neg = s;
+#else
+  auto whole = [](const Fix &f) {
+    return static_cast<__int128>((static_cast<unsigned __int128>(static_cast<int64_t>(static_cast<int32_t>(f.w[2]))) << 64) |
+                                 make64(f.w[0], f.w[1]));
+  };
+  const __int128 d = whole(a) - whole(b);
+  const Fix f = fix_of(static_cast<unsigned __int128>(d < 0 ? -d : d));
+  m[0] = f.w[0];
+  m[1] = f.w[1];
+  m[2] = f.w[2];
+  *neg = d < 0 ? ~0u : 0u;
+#endif
+}
+
+// A difference from fixed point: magnitudes (h, l, t) with the largest h in
 // [2^29, 2^30), signs, em as above; ok false where FP64 has to take it.
 struct FixDiff {
-  uint32_t h[3], l[3], sign[3];
+  uint32_t h[3], l[3], t[3], sign[3];
   uint32_t em;
   bool ok;
 };
-NB_HD FixDiff fix_diff(const int64_t (&xj)[3], const int64_t (&xi)[3], uint32_t E) {
+NB_HD FixDiff fix_diff(const Fix (&xj)[3], const Fix (&xi)[3], uint32_t E) {
   FixDiff f;
   uint32_t mx = 0u, mn = ~0u;
 #ifdef __CUDACC__
 #pragma unroll
 #endif
   for (int c = 0; c < 3; ++c) {
-    const int64_t d = xj[c] - xi[c];
-    const int64_t s = d >> 63;
-    const uint64_t a = static_cast<uint64_t>((d ^ s) - s);
-    f.sign[c] = hi32(static_cast<uint64_t>(s)) & 0x80000000u;
-    f.h[c] = hi32(a);
-    f.l[c] = lo32(a);
-    mx = f.h[c] > mx ? f.h[c] : mx;
+    uint32_t m[3], neg;
+    fix_abs_diff(xj[c], xi[c], m, &neg);
+    f.sign[c] = neg & 0x80000000u;
+    f.h[c] = m[2];
+    f.l[c] = m[1];
+    f.t[c] = m[0];
+    mx = m[2] > mx ? m[2] : mx;
   }
   f.ok = mx >= (1u << 22);
-  const uint32_t n = clz32(mx), s = n - 2u;  // (|D| < 2^62: n >= 2)
+  const uint32_t n = clz32(mx), s = n - 2u;  // (|D| < 2^94: n >= 2)
 #ifdef __CUDACC__
 #pragma unroll
 #endif
   for (int c = 0; c < 3; ++c) {
     f.h[c] = fshl(f.l[c], f.h[c], s);
-    f.l[c] <<= s & 31u;
+    f.l[c] = fshl(f.t[c], f.l[c], s);
+    f.t[c] <<= s & 31u;
     mn = f.h[c] < mn ? f.h[c] : mn;
   }
   f.ok = f.ok && mn != 0u;
@@ -380,7 +422,7 @@ NB_HD uint64_t square_sum(const FixDiff &f) {
 // Component c, rounded to FP64.
 NB_HD double fix_value(const FixDiff &f, int c) {
   const uint32_t m = clz32(f.h[c]), s = m - 1u;  // (2 <= m < 32)
-  const uint64_t v = make64(f.l[c] << (s & 31u), fshl(f.l[c], f.h[c], s)) + 0x200u;  // leading one at bit 62
+  const uint64_t v = make64(fshl(f.t[c], f.l[c], s), fshl(f.l[c], f.h[c], s)) + 0x200u;  // leading one at bit 62
   const uint32_t hi = (hi32(v) >> 10) + ((f.em + 1u - m) << 20);
   return from_bits(fshr(lo32(v), hi32(v), 10), hi | f.sign[c]);
 }

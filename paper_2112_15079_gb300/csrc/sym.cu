@@ -4,11 +4,11 @@
 // SM sub-partition).  The pair (p, j) and its reaction share the difference
 // and |d|^-3, so evaluating each unordered pair once takes 20 FP64 operations
 // for two interactions.  |d|^2, |d|^-3 and the mass products, 11 of them, and
-// the differences run on the integer pipes (inv_cube.h), about 170
+// the differences run on the integer pipes (inv_cube.h), about 185
 // instructions beside the 6 FP64 accumulations that are left.  Measured on
 // GB300, 10,425 bodies: 2.03 ms per step with 20 FP64 operations, 0.94 ms with
-// 9 (FP64 differences), 0.67 ms with 6 (the launch 0.60 ms, 6 x 76 cycles a pair
-// and warp step: the FP64 pipe stays the bound).
+// 9 (FP64 differences), 0.69 ms with 6 (the launch 0.62 ms; 6 x 76 cycles a pair
+// and warp step are 0.61: the FP64 pipe stays the bound).
 //
 // Decomposition: each system's bodies are cut into blocks of 64 (two warp
 // tiles of 32); the work items are the block pairs (I, J), I <= J, handed
@@ -109,20 +109,21 @@ __device__ __forceinline__ void sym_tile(const double4_32a &pi, const double4_32
   if (masses && ic::fix_in_range(E)) {
     const ic::Mass mi = ic::pack_mass(pi.w);
     ic::Mass mj = ic::pack_mass(pj.w);
+    ic::Fix xi[3] = {ic::to_fix(pi.x, E), ic::to_fix(pi.y, E), ic::to_fix(pi.z, E)};
+    ic::Fix xj[3] = {ic::to_fix(pj.x, E), ic::to_fix(pj.y, E), ic::to_fix(pj.z, E)};
     // (a lane outside the system: beyond every body of the tiles, massless)
-    const int64_t pad = int64_t(1) << 61;
-    const int64_t xi[3] = {ri ? ic::to_fix(pi.x, E) : pad, ri ? ic::to_fix(pi.y, E) : pad,
-                           ri ? ic::to_fix(pi.z, E) : pad};
-    int64_t xj[3] = {rj ? ic::to_fix(pj.x, E) : pad, rj ? ic::to_fix(pj.y, E) : pad, rj ? ic::to_fix(pj.z, E) : pad};
+    if (!ri) xi[0] = xi[1] = xi[2] = ic::fix_pad();
+    if (!rj) xj[0] = xj[1] = xj[2] = ic::fix_pad();
     auto rotate_source = [&]() {
-      xj[0] = __shfl_sync(0xffffffffu, xj[0], src);
-      xj[1] = __shfl_sync(0xffffffffu, xj[1], src);
-      xj[2] = __shfl_sync(0xffffffffu, xj[2], src);
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int u = 0; u < 3; ++u) xj[c].w[u] = __shfl_sync(0xffffffffu, xj[c].w[u], src);
       mj.u = __shfl_sync(0xffffffffu, mj.u, src);
       mj.w = __shfl_sync(0xffffffffu, mj.w, src);
     };
     int close = 0;  // steps that had a close pair
-#pragma unroll 2
+#pragma unroll 1
     for (; k < kEnd && close < kCloseSteps; ++k) {
       if (SELF) {
         rotate();

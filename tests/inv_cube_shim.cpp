@@ -39,7 +39,7 @@ extern "C" void ic_differences(int64_t n, const double *xi, const double *xj, co
                                double *cube, int32_t *taken) {
   using namespace nb::ic;
   for (int64_t i = 0; i < n; ++i) {
-    int64_t a[3], b[3];
+    Fix a[3], b[3];
     for (int c = 0; c < 3; ++c) {
       a[c] = to_fix(xi[c * n + i], static_cast<uint32_t>(E[i]));
       b[c] = to_fix(xj[c * n + i], static_cast<uint32_t>(E[i]));

@@ -109,11 +109,11 @@ def test_left_to_the_series(ic, d, mu):
 
 @pytest.mark.parametrize("kind", ["any", "near the origin", "pairs far from it", "flat", "another body sets the scale"])
 def test_fixed_point_differences(ic, kind):
-    """x in units of 2^(E - 1083) (exact within 2^-8 of the largest coordinate,
-    half a unit else) gives a difference within one unit, 2^-54 of its largest
-    component at least, plus the rounding to FP64, 2^-53 of each component:
-    1.5 x 2^-53 of the largest.  |d|^-3 then is off by 3 x sqrt(3) 2^-54 at
-    most, plus its own 0.77 units in the last place."""
+    """96-bit integers hold a coordinate exactly down to 2^-40 of the largest
+    and to 2^-92 of it below, so a component (at least 2^-37 of the scale,
+    where it is taken) is exact to 2^-55 and then rounds to FP64: 0.63 units in
+    the last place of the component itself.  |d|^-3 is off by 3 x sqrt(3) 2^-61
+    from the 62-bit alignment, plus its own 0.77 units in the last place."""
     if np.finfo(np.longdouble).nmant < 63:
         pytest.skip("no extended precision here")
     rng = np.random.default_rng(9)
@@ -136,12 +136,12 @@ def test_fixed_point_differences(ic, kind):
         return
     assert ok.mean() > (0.2 if kind in ("pairs far from it", "another body sets the scale") else 0.9)
     want = xj.astype(np.longdouble) - xi.astype(np.longdouble)
-    big = np.abs(want).max(0)
-    assert (np.abs(got - want) / big)[:, ok].max() <= 1.5 * 2.0**-53
+    ulp = np.spacing(np.abs(want.astype(np.float64)))
+    assert (np.abs(got.astype(np.longdouble) - want) / ulp)[:, ok].max() <= 0.63
     r2 = (want * want).sum(0)
     ref = (1 / (r2 * np.sqrt(r2)))[ok]
     err = np.abs((cube[ok] - ref) / ref).astype(float)
-    assert err.max() <= 3 * np.sqrt(3) * 2.0**-54 + 0.77 * 2.0**-52
+    assert err.max() <= 3 * np.sqrt(3) * 2.0**-61 + 0.77 * 2.0**-52
 
 
 def test_fixed_point_leaves_close_pairs(ic):
