@@ -117,24 +117,25 @@ cudaError_t launch_boxes(const void *stage, int64_t n_pairs, float4 *boxes, cuda
 //   FP64 pairs for the FP64 path, float pairs for the mixed path), its loads
 //   issued kUnroll rows at a time; for kLanes > 1 a fixed-shape shuffle tree
 //   then combines the lanes, so the summation order never changes.
-//   Phase B (one body per thread): for kModeStep,
+//   Phase B (one component of a body per thread): for kModeStep,
 //     Eq. 4  v_{i+1} = v_i + dt/2 (a_i + a_{i+1}),
 //     the caller's position receives r_{i+1} (the staged positions),
 //     Eq. 3  r_{i+2} = r_{i+1} + v_{i+1} dt + dt^2/2 a_{i+1} -> next stage.
 // GB300 runs FP64 at 1/64 of the FP32 rate and charges a warp instruction
 // for all 32 lanes whatever the active mask, so FP64 work runs one body per
-// lane: the mixed path sums its float-pair rows 8 lanes per body (short
-// latency) and hands the sums to warp 0 for phase B; the FP64 path, whose
-// row sums are FP64 themselves, sums one body per lane.
+// lane, and warp c < 3 of a CTA of 32 bodies takes component c: the mixed path
+// sums its float-pair rows 8 lanes per body (short latency) and hands the sums
+// to those warps for phase B; the FP64 path, whose row sums are FP64
+// themselves, sums them there too.  (One thread for all three components
+// left most sub-partitions idle at 10,425 bodies: 55 -> 37 us per launch with
+// its 163 rows.)
 // ---------------------------------------------------------------------------
 template <int PREC>
 struct VerletShape {
-  // FP64: one lane per body and 64 bodies per CTA, so the FP64 work spreads
-  // over ~N/64 CTAs (every SM at N = 10k); mixed: 8 lanes per body, 32 bodies.
-  static constexpr int kBlock = PREC == 0 ? 64 : 256;
-  static constexpr int kLanes = PREC == 0 ? 1 : 8;   // threads per body in phase A
+  static constexpr int kBodies = 32;
+  static constexpr int kLanes = PREC == 0 ? 1 : 8;   // threads per body (FP64: and component) in phase A
+  static constexpr int kBlock = PREC == 0 ? 96 : 256;
   static constexpr int kUnroll = PREC == 0 ? 8 : 4;  // rows per lane whose loads go out together
-  static constexpr int kBodies = kBlock / kLanes;
 };
 
 // (hi, lo) pair sums: FP64 pairs for the FP64 path, float pairs for mixed.
@@ -144,77 +145,91 @@ __device__ __forceinline__ void pair_add(T &hi, T &lo, T vhi, T vlo) {
   lo += vlo;
 }
 
-// Phase A of the per-body kernels: body p's force partials (rows 0..rows-1)
-// summed in a fixed order by L = VerletShape<PREC>::kLanes threads; the sum,
-// an unevaluated (hi, lo) pair per component, ends in lane 0.  FP64 adds
-// each group of U rows plainly before it enters the pair (see below); the
-// mixed path feeds every row through the pair.
-template <int PREC, typename T>
-__device__ __forceinline__ void sum_partial_rows(const double *partial, int rows, size_t N, int p, int lane, T &sx,
-                                                 T &ex, T &sy, T &ey, T &sz, T &ez) {
-  typedef typename std::conditional<PREC == 0, double, float2>::type E;  // one partial-row entry
-  constexpr int L = VerletShape<PREC>::kLanes, U = VerletShape<PREC>::kUnroll;
-  sx = sy = sz = ex = ey = ez = 0;
-  const E *part = reinterpret_cast<const E *>(partial);  // row c of body p: part[c*3N + k*N + p]
-  auto add = [&](T &s, T &e, const E &v) {
-    if constexpr (PREC == 0) {
-      two_sum_acc(s, e, v);
-    } else {
-      pair_add<T>(s, e, v.x, v.y);
-    }
-  };
+// Phase A of the per-body kernels, FP64: component c of body p's force partials
+// (rows 0..rows-1).  The (up to) U loaded rows are added plainly in row order,
+// then the group sum goes into the (hi, lo) pair: one TwoSum per U rows (the
+// pair-once kernel leaves a row per 64-body block, ~160 per body at
+// N = 10,425; each row is a sum of at most 128 terms).
+__device__ __forceinline__ double sum_rows_fp64(const double *partial, int rows, size_t N, int p, int c) {
+  constexpr int U = VerletShape<0>::kUnroll;
+  double s = 0.0, e = 0.0;
+  for (int r0 = 0; r0 < rows; r0 += U) {
+    double v[U], g = 0.0;
+#pragma unroll
+    for (int u = 0; u < U; ++u)  // all loads first, then the sums in row order
+      v[u] = r0 + u < rows ? __ldg(partial + (static_cast<size_t>(r0 + u) * 3 + c) * N + p) : 0.0;
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (r0 + u < rows) g += v[u];
+    two_sum_acc(s, e, g);
+  }
+  return s + e;
+}
+
+// Mixed: the same by 8 lanes per body, every row through the float pair; the
+// sums of the three components, unevaluated (hi, lo) pairs, end in lane 0.
+__device__ __forceinline__ void sum_rows_mixed(const double *partial, int rows, size_t N, int p, int lane, float &sx,
+                                               float &ex, float &sy, float &ey, float &sz, float &ez) {
+  constexpr int L = VerletShape<1>::kLanes, U = VerletShape<1>::kUnroll;
+  sx = sy = sz = ex = ey = ez = 0.f;
+  const float2 *part = reinterpret_cast<const float2 *>(partial);  // row c of body p: part[c*3N + k*N + p]
   for (int c0 = lane; c0 < rows; c0 += U * L) {
-    E vx_[U], vy_[U], vz_[U];
+    float2 vx_[U], vy_[U], vz_[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {  // all loads first, then the sums in row order
       const int c = c0 + u * L;
       if (c < rows) {
-        const E *row = part + static_cast<size_t>(c) * 3 * N;
+        const float2 *row = part + static_cast<size_t>(c) * 3 * N;
         vx_[u] = __ldg(row + p);
         vy_[u] = __ldg(row + N + p);
         vz_[u] = __ldg(row + 2 * N + p);
       }
     }
-    if constexpr (PREC == 0) {
-      // FP64: the (up to) U loaded rows added plainly in row order, then the
-      // group sum into the (hi, lo) pair: one TwoSum per U rows (the
-      // pair-once kernel leaves a row per 64-body block, ~160 per body at
-      // N = 10,425; each row is a sum of at most 128 terms).
-      E gx = 0.0, gy = 0.0, gz = 0.0;
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        if (c0 + u * L < rows) {
-          gx += vx_[u];
-          gy += vy_[u];
-          gz += vz_[u];
-        }
-      }
-      add(sx, ex, gx);
-      add(sy, ey, gy);
-      add(sz, ez, gz);
-    } else {
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        if (c0 + u * L < rows) {
-          add(sx, ex, vx_[u]);
-          add(sy, ey, vy_[u]);
-          add(sz, ez, vz_[u]);
-        }
+    for (int u = 0; u < U; ++u) {
+      if (c0 + u * L < rows) {
+        pair_add(sx, ex, vx_[u].x, vx_[u].y);
+        pair_add(sy, ey, vy_[u].x, vy_[u].y);
+        pair_add(sz, ez, vz_[u].x, vz_[u].y);
       }
     }
   }
-  if constexpr (L > 1) {
 #pragma unroll
-    for (int off = 1; off < L; off <<= 1) {
-      const T hx = __shfl_down_sync(0xffffffffu, sx, off), lx = __shfl_down_sync(0xffffffffu, ex, off);
-      const T hy = __shfl_down_sync(0xffffffffu, sy, off), ly = __shfl_down_sync(0xffffffffu, ey, off);
-      const T hz = __shfl_down_sync(0xffffffffu, sz, off), lz = __shfl_down_sync(0xffffffffu, ez, off);
-      if ((lane & (2 * off - 1)) == 0) {
-        pair_add<T>(sx, ex, hx, lx);
-        pair_add<T>(sy, ey, hy, ly);
-        pair_add<T>(sz, ez, hz, lz);
-      }
+  for (int off = 1; off < L; off <<= 1) {
+    const float hx = __shfl_down_sync(0xffffffffu, sx, off), lx = __shfl_down_sync(0xffffffffu, ex, off);
+    const float hy = __shfl_down_sync(0xffffffffu, sy, off), ly = __shfl_down_sync(0xffffffffu, ey, off);
+    const float hz = __shfl_down_sync(0xffffffffu, sz, off), lz = __shfl_down_sync(0xffffffffu, ez, off);
+    if ((lane & (2 * off - 1)) == 0) {
+      pair_add(sx, ex, hx, lx);
+      pair_add(sy, ey, hy, ly);
+      pair_add(sz, ez, hz, lz);
     }
+  }
+}
+
+// Phase A of a CTA: the acceleration component `comp` of body p0 + k for the
+// thread's phase B (0 beyond component 2).  rows_a: the rows of the thread's
+// phase A body.  Mixed: every thread of the CTA takes part.
+template <int PREC>
+__device__ __forceinline__ double sum_rows(const double *partial, size_t N, int p0, int rows_a, int comp, int k) {
+  if constexpr (PREC == 0) {
+    return sum_rows_fp64(partial, rows_a, N, p0 + k, comp);
+  } else {
+    constexpr int L = VerletShape<1>::kLanes, NB = VerletShape<1>::kBodies;
+    __shared__ float s_hi[3][NB], s_lo[3][NB];
+    const int b = threadIdx.x / L, lane = threadIdx.x % L;
+    float sx, sy, sz, ex, ey, ez;
+    sum_rows_mixed(partial, rows_a, N, p0 + b, lane, sx, ex, sy, ey, sz, ez);
+    if (lane == 0) {
+      s_hi[0][b] = sx;
+      s_lo[0][b] = ex;
+      s_hi[1][b] = sy;
+      s_lo[1][b] = ey;
+      s_hi[2][b] = sz;
+      s_lo[2][b] = ez;
+    }
+    __syncthreads();
+    return comp < 3 ? static_cast<double>(s_hi[comp][k]) + static_cast<double>(s_lo[comp][k]) : 0.0;
   }
 }
 
@@ -260,122 +275,81 @@ __device__ __forceinline__ void stage_position(void *nxt, int q, size_t o, doubl
   }
 }
 
+// The same, component c by itself (c = 0 also writes mu).
+template <int PREC>
+__device__ __forceinline__ void stage_component(void *nxt, int q, size_t o, int c, double r, double mu, float muf) {
+  if (PREC == 0) {
+    double *w = reinterpret_cast<double *>(static_cast<double4_32a *>(nxt) + q);
+    w[c] = r;
+    if (c == 0) w[3] = mu;
+  } else {
+    float *w = static_cast<float *>(nxt) + o;
+    const float h = hi_part(r);
+    w[kXh + 2 * c] = h;
+    w[kXl + 2 * c] = lo_part(r, h);
+    if (c == 0) w[kMu] = muf;
+  }
+}
+
 template <int PREC, int MODE>  // MODE: kModeForce, kModeStep or kModeLeapfrog (a.mode)
 __global__ void __launch_bounds__(VerletShape<PREC>::kBlock) verlet_kernel(const VerletArgs a) {
   // Where the host says so the next kernel may launch now, so that its launch
   // overlaps this kernel (its own griddepcontrol.wait still waits for our
   // completion).  Otherwise release only at the end (below).
   if (a.release_early) grid_dependency_launch();
-  typedef typename std::conditional<PREC == 0, double, float>::type T;
   constexpr int L = VerletShape<PREC>::kLanes, NB = VerletShape<PREC>::kBodies;
-  // Phase B: FP64 path one thread per body (all three components); mixed
-  // path warp c < 3 takes component c of the CTA's 32 bodies, lane = body,
+  // Phase B: warp c < 3 takes component c of the CTA's 32 bodies, lane = body,
   // so each warp issues a third of the FP64 instructions (GB300's FP64 pipe
   // spends 64 cycles on every warp instruction, so this is the latency).
-  constexpr bool kSplit = PREC == 1;
-  __shared__ T s_hi[3][NB], s_lo[3][NB];
   const int p0 = a.p_begin + blockIdx.x * NB;  // bodies [p_begin, p_end) (a row shard, or all)
-  const int b = threadIdx.x / L, lane = threadIdx.x % L;
-  const int p = p0 + b;  // phase A body
-  const bool live = p < a.p_end;
+  const int comp = threadIdx.x >> 5, k = threadIdx.x & 31, q = p0 + k;
+  const bool own = comp < 3 && q < a.p_end;
   const size_t N = static_cast<size_t>(a.N);
-  const int warp = threadIdx.x >> 5;
-  const int k = kSplit ? (threadIdx.x & 31) : threadIdx.x;  // phase B body within the CTA
-  const int q = p0 + k;
-  const int comp = kSplit ? warp : 0;
-  const bool own = (kSplit ? warp < 3 : threadIdx.x < NB) && q < a.p_end;
   constexpr bool step = MODE != kModeForce;
   constexpr bool leap = MODE == kModeLeapfrog;
-  // This thread's component arrays (mixed split; the FP64 path uses all three).
+  // This thread's component arrays.
   auto pick = [&](double *x, double *y, double *z) { return comp == 0 ? x : comp == 1 ? y : z; };
   double *const Xc = pick(a.x, a.y, a.z), *const Vc = pick(a.vx, a.vy, a.vz), *const Ac = pick(a.ax, a.ay, a.az);
   double *const Rc = pick(a.Rx, a.Ry, a.Rz);
 
   // Before the wait: everything this step's force kernel does not write (it
   // writes only the partial rows), so these loads overlap its tail.
-  const int rows = live ? a.nsl[p] : 0;
-  double v[3] = {0, 0, 0}, ao[3] = {0, 0, 0}, r[3] = {0, 0, 0}, mu = 0.0;
+  const int pa = PREC == 0 ? q : p0 + static_cast<int>(threadIdx.x) / L;  // phase A body
+  const int rows = pa < a.p_end ? a.nsl[pa] : 0;
+  double v = 0.0, ao = 0.0, r = 0.0, mu = 0.0;
   float muf = 0.f;
   size_t o = 0;
   if (own && step) {
-    if (kSplit) {
-      v[0] = Vc[q];
-      ao[0] = Ac[q];
-      r[0] = Rc[q];
+    v = Vc[q];
+    ao = Ac[q];
+    if (PREC == 0) {
+      const double *rr = reinterpret_cast<const double *>(static_cast<const double4_32a *>(a.cur) + q);
+      r = rr[comp];
+      if (comp == 0) mu = rr[3];
+    } else {
+      r = Rc[q];
       o = pair_off(a.qidx[q]);
       if (comp == 0) muf = static_cast<const float *>(a.cur)[o + kMu];
-    } else {
-      v[0] = a.vx[q];
-      v[1] = a.vy[q];
-      v[2] = a.vz[q];
-      ao[0] = a.ax[q];
-      ao[1] = a.ay[q];
-      ao[2] = a.az[q];
-      const double4_32a rr = static_cast<const double4_32a *>(a.cur)[q];
-      r[0] = rr.x;
-      r[1] = rr.y;
-      r[2] = rr.z;
-      mu = rr.w;
     }
   }
   grid_dependency_wait();  // the force partials of this step are complete
 
-  // ---- phase A: the partial rows of body p --------------------------------
-  T sx, sy, sz, ex, ey, ez;
-  sum_partial_rows<PREC, T>(a.partial, rows, N, p, lane, sx, ex, sy, ey, sz, ez);
-  if (lane == 0) {
-    s_hi[0][b] = sx;
-    s_lo[0][b] = ex;
-    s_hi[1][b] = sy;
-    s_lo[1][b] = ey;
-    s_hi[2][b] = sz;
-    s_lo[2][b] = ez;
-  }
-  __syncthreads();
+  const double an = sum_rows<PREC>(a.partial, N, p0, rows, comp, k);  // phase A
   if (!own) {
     if (!a.release_early) grid_dependency_launch();
     return;
   }
-
-  // ---- phase B: Eqs. 4 and 3 ---------------------------------------------------
-  if (kSplit) {  // component `comp` of body q
-    const double an = static_cast<double>(s_hi[comp][k]) + static_cast<double>(s_lo[comp][k]);
-    if (!isfinite(an)) atomicOr(a.flags, kFlagNonFinite);
-    if (step) {
-      double vn = v[0], nr;
-      const double x = step_component(leap, r[0], vn, ao[0], an, a.dt, a.half_dt, a.half_dt2, &nr);
-      Rc[q] = nr;
-      float *w = static_cast<float *>(a.nxt) + o;
-      const float h = hi_part(nr);
-      w[kXh + 2 * comp] = h;
-      w[kXl + 2 * comp] = lo_part(nr, h);
-      if (comp == 0) w[kMu] = muf;
-      Xc[q] = x;
-      Vc[q] = vn;
-    }
-    Ac[q] = an;
-  } else {  // body q, all three components
-    double an[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) an[c] = static_cast<double>(s_hi[c][k]) + static_cast<double>(s_lo[c][k]);
-    if (!finite3(an[0], an[1], an[2])) atomicOr(a.flags, kFlagNonFinite);
-    if (step) {
-      double nr[3], x[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c)
-        x[c] = step_component(leap, r[c], v[c], ao[c], an[c], a.dt, a.half_dt, a.half_dt2, &nr[c]);
-      stage_position<PREC>(a.nxt, q, o, nr[0], nr[1], nr[2], mu, muf);
-      a.x[q] = x[0];
-      a.y[q] = x[1];
-      a.z[q] = x[2];
-      a.vx[q] = v[0];
-      a.vy[q] = v[1];
-      a.vz[q] = v[2];
-    }
-    a.ax[q] = an[0];
-    a.ay[q] = an[1];
-    a.az[q] = an[2];
+  // ---- phase B: Eqs. 4 and 3, component `comp` of body q ----------------------
+  if (!isfinite(an)) atomicOr(a.flags, kFlagNonFinite);
+  if (step) {
+    double vn = v, nr;
+    const double x = step_component(leap, r, vn, ao, an, a.dt, a.half_dt, a.half_dt2, &nr);
+    stage_component<PREC>(a.nxt, q, o, comp, nr, mu, muf);
+    if (PREC == 1) Rc[q] = nr;
+    Xc[q] = x;
+    Vc[q] = vn;
   }
+  Ac[q] = an;
   // Otherwise only now may the next force launch be placed: its CTAs then
   // land on an idle GPU, one share per slot, as the equal-share decomposition
   // assumes (an early launch let several CTAs pile onto the SMs that freed
@@ -420,103 +394,62 @@ cudaError_t launch_verlet(int precision, const VerletArgs &a, cudaStream_t s, bo
 template <int PREC>
 __global__ void __launch_bounds__(VerletShape<PREC>::kBlock) rk_stage_kernel(const RkArgs a) {
   if (a.release_early) grid_dependency_launch();
-  typedef typename std::conditional<PREC == 0, double, float>::type T;
   constexpr int L = VerletShape<PREC>::kLanes, NB = VerletShape<PREC>::kBodies;
-  constexpr bool kSplit = PREC == 1;  // mixed: warp c < 3 takes component c (as the Verlet kernel)
-  __shared__ T s_hi[3][NB], s_lo[3][NB];
   const int p0 = blockIdx.x * NB;
-  const int b = threadIdx.x / L, lane = threadIdx.x % L;
-  const int p = p0 + b;
-  const bool live = p < a.N;
+  const int c = threadIdx.x >> 5, k = threadIdx.x & 31, q = p0 + k;  // (as the Verlet kernel: warp c, component c)
+  const bool own = c < 3 && q < a.N;
   const size_t N = static_cast<size_t>(a.N);
-  const int warp = threadIdx.x >> 5;
-  const int k0 = kSplit ? (threadIdx.x & 31) : threadIdx.x;
-  const int q = p0 + k0;
-  const int comp = kSplit ? warp : 0;
-  const bool own = (kSplit ? warp < 3 : threadIdx.x < NB) && q < a.N;
-  const int rows = live ? a.nsl[p] : 0;
-  auto sel = [](int c, double *x, double *y, double *z) { return c == 0 ? x : c == 1 ? y : z; };
-  // Prefetch what the force launch does not write (the state, the RK sums):
-  // component comp (mixed) or all three (FP64).
-  constexpr int NC = kSplit ? 1 : 3;
-  double rn[NC], vn[NC], vs[NC], ar[NC], av[NC], mu = 0.0;
+  const int pa = PREC == 0 ? q : p0 + static_cast<int>(threadIdx.x) / L;  // phase A body
+  const int rows = pa < a.N ? a.nsl[pa] : 0;
+  auto sel = [&](double *x, double *y, double *z) { return c == 0 ? x : c == 1 ? y : z; };
+  const size_t i = c * N + q;
+  // Prefetch what the force launch does not write (the state, the RK sums).
+  double rn = 0.0, vn = 0.0, vs = 0.0, ar = 0.0, av = 0.0, mu = 0.0;
   float muf = 0.f;
   size_t o = 0;
-#pragma unroll
-  for (int j = 0; j < NC; ++j) rn[j] = vn[j] = vs[j] = ar[j] = av[j] = 0.0;
   if (own) {
-#pragma unroll
-    for (int j = 0; j < NC; ++j) {
-      const int c = kSplit ? comp : j;
-      rn[j] = sel(c, a.x, a.y, a.z)[q];
-      vn[j] = sel(c, a.vx, a.vy, a.vz)[q];
-      if (a.stage <= 4) {
-        vs[j] = a.V[c * N + q];
-        ar[j] = a.AR[c * N + q];
-        av[j] = a.AV[c * N + q];
-      }
+    rn = sel(a.x, a.y, a.z)[q];
+    vn = sel(a.vx, a.vy, a.vz)[q];
+    if (a.stage <= 4) {
+      vs = a.V[i];
+      ar = a.AR[i];
+      av = a.AV[i];
     }
     if (PREC == 0) {
-      mu = static_cast<const double4_32a *>(a.cur)[q].w;
+      if (c == 0) mu = static_cast<const double4_32a *>(a.cur)[q].w;
     } else {
       o = pair_off(a.qidx[q]);
-      if (comp == 0) muf = static_cast<const float *>(a.cur)[o + kMu];
+      if (c == 0) muf = static_cast<const float *>(a.cur)[o + kMu];
     }
   }
   grid_dependency_wait();  // the force partials of this stage are complete
-  T sx, sy, sz, ex, ey, ez;
-  sum_partial_rows<PREC, T>(a.partial, rows, N, p, lane, sx, ex, sy, ey, sz, ez);
-  if (lane == 0) {
-    s_hi[0][b] = sx;
-    s_lo[0][b] = ex;
-    s_hi[1][b] = sy;
-    s_lo[1][b] = ey;
-    s_hi[2][b] = sz;
-    s_lo[2][b] = ez;
-  }
-  __syncthreads();
+  const double as = sum_rows<PREC>(a.partial, N, p0, rows, c, k);
   if (!own) {
     if (!a.release_early) grid_dependency_launch();
     return;
   }
-  bool finite = true;
-  double rnext[NC];
-#pragma unroll
-  for (int j = 0; j < NC; ++j) {
-    const int c = kSplit ? comp : j;
-    const size_t i = c * N + q;
-    const double as = static_cast<double>(s_hi[c][k0]) + static_cast<double>(s_lo[c][k0]);
-    finite = finite && isfinite(as);
-    if (a.stage == 2 || a.stage == 3) {
-      const double cc = a.stage == 2 ? 0.5 * a.dt : a.dt;
-      a.AR[i] = ar[j] + 2.0 * vs[j];
-      a.AV[i] = av[j] + 2.0 * as;
-      rnext[j] = rn[j] + cc * vs[j];
-      a.V[i] = vn[j] + cc * as;
-    } else if (a.stage == 4) {
-      const double h = a.dt / 6.0;
-      rnext[j] = rn[j] + h * (ar[j] + vs[j]);
-      sel(c, a.x, a.y, a.z)[q] = rnext[j];
-      sel(c, a.vx, a.vy, a.vz)[q] = vn[j] + h * (av[j] + as);
-    } else {  // s = 5: A at the new state, then stage 1 of the next step
-      sel(c, a.ax, a.ay, a.az)[q] = as;
-      const double cc = 0.5 * a.dt;
-      a.AR[i] = vn[j];
-      a.AV[i] = as;
-      rnext[j] = rn[j] + cc * vn[j];
-      a.V[i] = vn[j] + cc * as;
-    }
+  double rnext;
+  if (a.stage == 2 || a.stage == 3) {
+    const double cc = a.stage == 2 ? 0.5 * a.dt : a.dt;
+    a.AR[i] = ar + 2.0 * vs;
+    a.AV[i] = av + 2.0 * as;
+    rnext = rn + cc * vs;
+    a.V[i] = vn + cc * as;
+  } else if (a.stage == 4) {
+    const double h = a.dt / 6.0;
+    rnext = rn + h * (ar + vs);
+    sel(a.x, a.y, a.z)[q] = rnext;
+    sel(a.vx, a.vy, a.vz)[q] = vn + h * (av + as);
+  } else {  // s = 5: A at the new state, then stage 1 of the next step
+    sel(a.ax, a.ay, a.az)[q] = as;
+    const double cc = 0.5 * a.dt;
+    a.AR[i] = vn;
+    a.AV[i] = as;
+    rnext = rn + cc * vn;
+    a.V[i] = vn + cc * as;
   }
-  if (!finite) atomicOr(a.flags, kFlagNonFinite);
-  if (kSplit) {
-    float *w = static_cast<float *>(a.nxt) + o;
-    const float h = hi_part(rnext[0]);
-    w[kXh + 2 * comp] = h;
-    w[kXl + 2 * comp] = lo_part(rnext[0], h);
-    if (comp == 0) w[kMu] = muf;
-  } else {
-    stage_position<PREC>(a.nxt, q, o, rnext[0], rnext[NC > 1 ? 1 : 0], rnext[NC > 2 ? 2 : 0], mu, muf);
-  }
+  if (!isfinite(as)) atomicOr(a.flags, kFlagNonFinite);
+  stage_component<PREC>(a.nxt, q, o, c, rnext, mu, muf);
   if (!a.release_early) grid_dependency_launch();
 }
 

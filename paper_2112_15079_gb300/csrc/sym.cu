@@ -201,7 +201,6 @@ __global__ void __launch_bounds__(kSymThreads) force_sym_kernel(const SymArgs a)
   __shared__ double s_b[2][2][3][32];  // reaction sums [warp][J tile][component][lane]
   __shared__ int s_item;
   grid_dependency_wait();    // staged sources of this step are complete
-  grid_dependency_launch();  // the Verlet kernel may start launching
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   const size_t N = static_cast<size_t>(a.N);
   for (;;) {
@@ -209,7 +208,13 @@ __global__ void __launch_bounds__(kSymThreads) force_sym_kernel(const SymArgs a)
     if (tid == 0) s_item = atomicAdd(a.ctr, 1);
     __syncthreads();
     const int item = s_item;
-    if (item >= a.n_pairs) break;
+    if (item >= a.n_pairs) {
+      // The Verlet kernel may launch as the CTAs run out of items.  (Let in at
+      // the start, its CTAs that found no room beside ours piled onto the SMs
+      // that finished first: 10,425 bodies 691 us per step, 650 so; 3,001 87 and 73.)
+      grid_dependency_launch();
+      break;
+    }
     const int4 pr = a.pairs[item];  // (first body of the system, its bodies, block I, block J)
     const int64_t sb = pr.x;
     const int ns = pr.y, I = pr.z, J = pr.w;
@@ -286,7 +291,6 @@ __global__ void __launch_bounds__(kSymWideThreads) force_sym_wide_kernel(const S
   extern __shared__ double s_acc[];  // [3][32 T]: block J's reaction sums of the item
   __shared__ int s_item;
   grid_dependency_wait();    // staged sources of this step are complete
-  grid_dependency_launch();  // the Verlet kernel may start launching
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   const int T = a.tiles, BT = 32 * T;
   const size_t N = static_cast<size_t>(a.N);
