@@ -376,8 +376,9 @@ int sym_block(const nbody_ctx *c) {
 // 4 VJP).  An item is (first stage entry of the system, its bodies, I, J).
 nbody_status build_sym_work(nbody_ctx *c, Work &wk, int row_doubles, int B) {
   free_work(c, wk);
-  if (B != nb::kSymBlock && row_doubles != 3) return fail(c, NBODY_EINVAL, "wide pair-once blocks are force-only");
   const bool mixed = c->o.precision == NBODY_MIXED;
+  if (B != (mixed ? 32 * nb::kMsymMinTiles : nb::kSymBlock) && row_doubles != 3)
+    return fail(c, NBODY_EINVAL, "wide pair-once blocks are force-only");
   std::vector<int4> off_diag, diag;
   int64_t rows = 1;
   std::vector<uint16_t> nsl(static_cast<size_t>(c->N), 0);
@@ -403,8 +404,10 @@ nbody_status build_sym_work(nbody_ctx *c, Work &wk, int row_doubles, int B) {
   }
   if (rows > 65535 || pairs.size() > static_cast<size_t>(INT32_MAX))
     return fail(c, NBODY_EINVAL, "too many pair-once blocks (%lld in a system)", static_cast<long long>(rows));
-  const int occ = mixed ? nb::force_msym_ctas_per_sm(B / 32, B / 128) : nb::force_sym_ctas_per_sm(B / 32);
-  if (occ < 1) return fail(c, NBODY_ECUDA, "the pair-once FP64 kernel does not fit on an SM");
+  const int occ = mixed && row_doubles == 4 ? nb::vjp_msym_ctas_per_sm()
+                  : mixed                    ? nb::force_msym_ctas_per_sm(B / 32, B / 128)
+                                             : nb::force_sym_ctas_per_sm(B / 32);
+  if (occ < 1) return fail(c, NBODY_ECUDA, "the pair-once kernel does not fit on an SM");
   wk.nsl_rank = nsl;
   wk.plan_off = c->tgt_off;
   wk.plan_soff = c->tgt_soff;
@@ -1149,8 +1152,11 @@ nbody_status ensure_adjoint(nbody_ctx *c, int64_t n_steps) {
     t.tj = kVjpTile;
     t.jsplit = 0;
     t.ctas_per_sm = 32;
-    if (sym_block(c) == nb::kSymBlock) {  // FP64: the VJP evaluates each pair once too (64-body blocks)
-      if ((st = build_sym_work(c, A.vj, 4, nb::kSymBlock)) != NBODY_OK) return st;
+    // With the narrowest pair-once blocks (FP64 64 bodies, mixed 128 entries) the
+    // VJP evaluates each pair once too.
+    const int B = prec == NBODY_MIXED ? 32 * nb::kMsymMinTiles : nb::kSymBlock;
+    if (sym_block(c) == B) {
+      if ((st = build_sym_work(c, A.vj, 4, B)) != NBODY_OK) return st;
     } else {
       const size_t smem = nb::vjp_smem_bytes(prec, t.tj);
       int occ = 0;
@@ -1810,7 +1816,18 @@ nbody_status nbody_grad(nbody_ctx *c, int64_t n_steps, const double *dL_dr_T, co
   vj.N = c->N;
   vj.tj = kVjpTile;
   auto product = [&](const void *pos, int mode) -> nbody_status {
-    if (A.vj.sym_pairs) {  // pair-once (FP64): no bounded wait to stall
+    if (A.vj.sym_pairs && prec == NBODY_MIXED) {
+      nb::VjpMsymArgs vs{};
+      vs.pos = pos;
+      vs.w = A.w;
+      vs.partial = A.vj.partial;
+      vs.pairs = A.vj.sym_pairs;
+      vs.perm = c->perm;
+      vs.n_pairs = A.vj.n_sym;
+      vs.ctr = A.vj.dyn_ctr;
+      vs.N = c->N;
+      NB_CUDA(c, nb::launch_vjp_msym(vs, A.vj.grid, c->stream));
+    } else if (A.vj.sym_pairs) {  // pair-once: no bounded wait to stall
       nb::VjpSymArgs vs{};
       vs.pos = static_cast<const double4_32a *>(pos);
       vs.w = static_cast<const double4_32a *>(A.w);

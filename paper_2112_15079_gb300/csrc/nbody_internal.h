@@ -173,6 +173,18 @@ struct VjpSymArgs {
   int32_t N;
 };
 
+// The same on the mixed path (sym_mixed.cu): 128-entry stage blocks, rows of 4
+// float pairs per body.
+struct VjpMsymArgs {
+  const void *pos, *w;     // stage entries of the positions and of w (VjpArgs)
+  double *partial;         // [blocks][4][N] float pairs
+  const int4 *pairs;       // as MsymArgs::pairs
+  const int32_t *perm;
+  int32_t n_pairs;
+  int32_t *ctr;
+  int32_t N;
+};
+
 // Close-encounter handling (close.cu): clusters of close pairs sub-cycled in
 // FP64 after each step's Verlet kernel.  Members and pairs as CloseSet in
 // close_pairs.h (global member / pair indices).
@@ -268,6 +280,8 @@ size_t force_sym_smem_bytes(int tiles);
 cudaError_t launch_force_msym(const MsymArgs &a, int grid, cudaStream_t s, bool chained);
 int force_msym_ctas_per_sm(int tiles, int warps);  // resident CTAs per SM (raises the smem limit)
 size_t force_msym_smem_bytes(int tiles, int warps);
+int vjp_msym_ctas_per_sm();
+cudaError_t launch_vjp_msym(const VjpMsymArgs &a, int grid, cudaStream_t s);
 cudaError_t launch_close(const CloseArgs &a, int n_clusters, cudaStream_t s, bool chained);
 cudaError_t launch_close_far(const CloseArgs &a, cudaStream_t s, bool chained);
 cudaError_t launch_energy(const EnergyArgs &a, cudaStream_t s);

@@ -597,6 +597,216 @@ __global__ void __launch_bounds__(32 * kBlkWarps, 4) force_msym_block_kernel(con
   }
 }
 
+// The adjoint's vector-Jacobian product of Eq. 1 (see vjp.cu), each pair once,
+// mixed: 128-entry blocks and items as above, hi/lo differences throughout.
+// Warp w takes the 64 targets of half w >> 1 of block I, two per lane, and the
+// 64 entries of chunk w & 1 of block J, all 32 rotation steps.  With
+// f_q = mu_q |d|^-3, f_j = mu_j |d|^-3, al = w_j . d and be = -w_q . d the term
+//   t = f_q w_j - f_j w_q - 3 |d|^-2 (f_q al + f_j be) d
+// goes to q and -t to j, |d|^-3 al to q's mass sum and |d|^-3 be to j's: 43
+// packed operations for the two interactions of two source pairs against 72
+// in the ordered-pair kernel.  A product, reverse step and recomputed forward
+// step together: 2,131 bodies 64.6 -> 34.7 us, 10,425 bodies 209 -> 179.
+//
+// Sums: a target has 32 terms per half and warp; its halves are added plainly
+// (64 terms), its two warps' sums through TwoSum; a source has 64 terms from
+// each of its two warps, added through TwoSum.
+struct VjpBlockShared {
+  float4 src[2][2][4][64];     // [buffer][block I, J][piece][pair block]
+  float4 wsrc[2][2][2][64];    // the same of w: (wx0 wx1 wy0 wy1), (wz0 wz1 - -)
+  f2 ti[kBlkWarps][2][4][32];  // per warp and target slot: negated lo parts (0..2), then the packed sums
+  f2 tj[kBlkWarps][4][32];     // per warp: reaction sums of its chunk's pair blocks
+};
+
+template <bool MASKED>
+__device__ __forceinline__ void vjp_rotate(const float4 *cb, const float4 *wb, const f2 (&nx)[2][3],
+                                           const f2 (&mq)[2], const f2 (&nw)[2][3], const f2 (*tlo)[4][32], int lane,
+                                           int et0, int jc, f2 (&acc)[2][4], f2 (&b)[4]) {
+  const f2 m3 = pk(-3.f, -3.f);
+#pragma unroll 2
+  for (int k = 0; k < 32; ++k) {
+    const int m = (lane + k) & 31;
+    const float4 A = cb[m], B = cb[64 + m], C = cb[128 + m], W = wb[m];
+    const float2 D = *reinterpret_cast<const float2 *>(cb + 192 + m), V = *reinterpret_cast<const float2 *>(wb + 64 + m);
+    const f2 sh[3] = {pk(A.x, A.y), pk(A.z, A.w), pk(B.x, B.y)}, sl[3] = {pk(C.x, C.y), pk(C.z, C.w), pk(D.x, D.y)};
+    const f2 wj[3] = {pk(W.x, W.y), pk(W.z, W.w), pk(V.x, V.y)}, sm = pk(B.z, B.w);
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      f2 d[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) d[c] = add2(add2(sh[c], nx[a][c]), add2(sl[c], tlo[a][c][lane]));
+      f2 r2 = mul2(d[0], d[0]);
+      r2 = fma2(d[1], d[1], r2);
+      r2 = fma2(d[2], d[2], r2);
+      float ra, rb;
+      upk(r2, ra, rb);
+      float w0 = 1.f, w1 = 1.f;
+      if (MASKED) {  // a pair counts only if the target's entry precedes the source's
+        const int et = et0 + 32 * a, es = jc + 2 * m;
+        w0 = et < es ? 1.f : 0.f;
+        w1 = et < es + 1 ? 1.f : 0.f;
+        ra = w0 != 0.f ? ra : 1.f;
+        rb = w1 != 0.f ? rb : 1.f;
+      }
+      const f2 q = pk(rsqrt_approx(ra), rsqrt_approx(rb));
+      const f2 q2 = mul2(q, q);
+      f2 s3 = mul2(q, q2);
+      if (MASKED) s3 = mul2(s3, pk(w0, w1));
+      const f2 fq = mul2(mq[a], s3), fj = mul2(sm, s3);
+      f2 al = mul2(wj[0], d[0]);
+      al = fma2(wj[1], d[1], al);
+      al = fma2(wj[2], d[2], al);
+      f2 be = mul2(nw[a][0], d[0]);
+      be = fma2(nw[a][1], d[1], be);
+      be = fma2(nw[a][2], d[2], be);
+      const f2 g = mul2(mul2(fma2(fj, be, mul2(fq, al)), q2), m3);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const f2 t = fma2(g, d[c], fma2(fj, nw[a][c], mul2(fq, wj[c])));
+        acc[a][c] = add2(acc[a][c], t);
+        b[c] = add2(b[c], t);
+      }
+      acc[a][3] = fma2(s3, al, acc[a][3]);
+      b[3] = fma2(s3, be, b[3]);
+    }
+    const int src = (lane + 1) & 31;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) b[c] = __shfl_sync(0xffffffffu, b[c], src);
+  }
+}
+
+__global__ void __launch_bounds__(32 * kBlkWarps, 4) vjp_msym_block_kernel(const VjpMsymArgs a) {
+  extern __shared__ __align__(16) unsigned char msym_smem[];
+  VjpBlockShared &sh = *reinterpret_cast<VjpBlockShared *>(msym_smem);
+  __shared__ int s_item;
+  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+  const int half = w >> 1, chunk = w & 1;
+  const size_t N = static_cast<size_t>(a.N);
+  auto describe = [&](int item) { return item < a.n_pairs ? a.pairs[item] : make_int4(0, 0, 0, 0); };
+  auto stage_item = [&](const int4 &pr, int bb) {
+    if (pr.y > 0) {
+      const int nst = (pr.y + 1) & ~1;
+#pragma unroll
+      for (int u = 0; u < 6; ++u) {  // per block: 64 pair blocks x (4 + 2) pieces, 128 threads
+        const int blk = u / 3, pb = tid >> 1, v = u % 3, q = 2 * (v & 1) + (tid & 1);
+        const int e0 = 128 * (blk ? pr.w : pr.z) + 2 * pb;
+        const size_t block = static_cast<size_t>((pr.x + e0) >> 1);
+        float4 *dst = v < 2 ? &sh.src[bb][blk][q][pb] : &sh.wsrc[bb][blk][tid & 1][pb];
+        if (e0 < nst) {
+          cp_async16(dst, v < 2 ? reinterpret_cast<const float4 *>(a.pos) + block * 4 + q
+                                : reinterpret_cast<const float4 *>(a.w) + block * 2 + (tid & 1));
+        } else {  // past the end of the system: inert, each entry at a position of its own
+          const float x0 = 2.f * kPadCoord + 1e12f * static_cast<float>(e0 - nst), x1 = x0 + 1e12f;
+          *dst = v == 2 || q >= 2 ? make_float4(0.f, 0.f, 0.f, 0.f)
+                 : q == 0         ? make_float4(x0, x1, x0, x1)
+                                  : make_float4(x0, x1, 0.f, 0.f);
+        }
+      }
+    }
+    cp_async_commit();
+  };
+  // (item numbers, descriptors and data run ahead as in force_msym_block_kernel)
+  int fetched = 0;  // thread 0
+  if (tid == 0) {
+    s_item = static_cast<int>(gridDim.x) + atomicAdd(a.ctr, 1);
+    fetched = static_cast<int>(gridDim.x) + atomicAdd(a.ctr, 1);
+  }
+  int4 pr = describe(blockIdx.x);
+  stage_item(pr, 0);
+  __syncthreads();
+  int4 pn = describe(s_item);
+  int bb = 0;
+  while (pr.y > 0) {
+    cp_async_wait_all();
+    __syncthreads();  // this item's blocks are in; the previous item's sums (and s_item) are consumed
+    if (tid == 0) {
+      s_item = fetched;
+      fetched = static_cast<int>(gridDim.x) + atomicAdd(a.ctr, 1);
+    }
+    stage_item(pn, bb ^ 1);
+    const int s0 = pr.x, ns = pr.y, I = pr.z, J = pr.w;
+    const int nst = (ns + 1) & ~1;
+    const bool diag = I == J;
+    const int i0 = 128 * I, j0 = 128 * J, jc = 64 * chunk;
+    const int bi = i0 + tid < ns ? a.perm[s0 + i0 + tid] : -1, bj = j0 + tid < ns ? a.perm[s0 + j0 + tid] : -1;
+    f2 acc[2][4], b[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[0][c] = acc[1][c] = b[c] = 0ull;
+    // (a diagonal item's second half precedes none of the first chunk)
+    if (j0 + jc < nst && i0 + 64 * half < nst && !(diag && half > chunk)) {
+      f2 nx[2][3], mq[2], nw[2][3];
+#pragma unroll
+      for (int s = 0; s < 2; ++s) {
+        // target entry 64 half + 32 s + lane: pair block 32 half + 16 s + lane / 2, half lane & 1
+        const int pb = 32 * half + 16 * s + (lane >> 1), h = lane & 1;
+        const float *p[4], *v[2];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) p[q] = reinterpret_cast<const float *>(&sh.src[bb][0][q][pb]) + h;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) v[q] = reinterpret_cast<const float *>(&sh.wsrc[bb][0][q][pb]) + h;
+        nx[s][0] = pk(-p[0][0], -p[0][0]);
+        nx[s][1] = pk(-p[0][2], -p[0][2]);
+        nx[s][2] = pk(-p[1][0], -p[1][0]);
+        mq[s] = pk(p[1][2], p[1][2]);
+        nw[s][0] = pk(-v[0][0], -v[0][0]);
+        nw[s][1] = pk(-v[0][2], -v[0][2]);
+        nw[s][2] = pk(-v[1][0], -v[1][0]);
+        sh.ti[w][s][0][lane] = pk(-p[2][0], -p[2][0]);
+        sh.ti[w][s][1][lane] = pk(-p[2][2], -p[2][2]);
+        sh.ti[w][s][2][lane] = pk(-p[3][0], -p[3][0]);
+      }
+      __syncwarp();
+      const float4 *cb = &sh.src[bb][1][0][32 * chunk], *wb = &sh.wsrc[bb][1][0][32 * chunk];
+      if (diag && half == chunk)
+        vjp_rotate<true>(cb, wb, nx, mq, nw, sh.ti[w], lane, 64 * half + lane, jc, acc, b);
+      else
+        vjp_rotate<false>(cb, wb, nx, mq, nw, sh.ti[w], lane, 64 * half + lane, jc, acc, b);
+      __syncwarp();  // the lo parts are read
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      sh.ti[w][0][c][lane] = acc[0][c];
+      sh.ti[w][1][c][lane] = acc[1][c];
+      sh.tj[w][c][lane] = b[c];  // (a whole rotation: pair block `lane`)
+    }
+    __syncthreads();
+    // thread t: target entry t and source entry t
+    float2 *part = reinterpret_cast<float2 *>(a.partial);
+    float2 *row_i = part + static_cast<size_t>(J) * 4 * N + max(bi, 0), *row_j = part + static_cast<size_t>(I) * 4 * N + max(bj, 0);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int tw = 2 * (tid >> 6), sw = tid >> 6, mb = (tid >> 1) & 31;
+      float e0, o0, e1, o1;
+      upk(sh.ti[tw][(tid >> 5) & 1][c][lane], e0, o0);
+      upk(sh.ti[tw + 1][(tid >> 5) & 1][c][lane], e1, o1);
+      float hi = e0 + o0, lo = 0.f;
+      two_sum_acc(hi, lo, e1 + o1);
+      const float sg = c < 3 ? -1.f : 1.f;
+      float rh = sg * *(reinterpret_cast<const float *>(&sh.tj[sw][c][mb]) + (tid & 1)), rl = 0.f;
+      two_sum_acc(rh, rl, sg * *(reinterpret_cast<const float *>(&sh.tj[2 + sw][c][mb]) + (tid & 1)));
+      if (diag) {
+        two_sum_acc(hi, lo, rh);
+        if (bi >= 0) row_i[c * N] = make_float2(hi, lo + rl);
+      } else {
+        if (bi >= 0) row_i[c * N] = make_float2(hi, lo);
+        if (bj >= 0) row_j[c * N] = make_float2(rh, rl);
+      }
+    }
+    pr = pn;
+    pn = describe(s_item);  // (written before the barrier above; used an item later)
+    bb ^= 1;
+  }
+  cp_async_wait_all();
+  __syncthreads();
+  if (tid == 0) {
+    __threadfence();
+    if (atomicAdd(a.ctr + 1, 1) == static_cast<int>(gridDim.x) - 1) {
+      atomicExch(a.ctr, 0);
+      atomicExch(a.ctr + 1, 0);
+    }
+  }
+}
+
 namespace {
 bool msym_mu_smem(int tiles) { return tiles == kMsymMaxTiles; }
 }  // namespace
@@ -638,6 +848,24 @@ int force_msym_ctas_per_sm(int tiles, int warps) {
     return 0;
   }
   return occ;
+}
+
+int vjp_msym_ctas_per_sm() {
+  int occ = 0;
+  cudaError_t e = cudaFuncSetAttribute(vjp_msym_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(sizeof(VjpBlockShared)));
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, vjp_msym_block_kernel, 32 * kBlkWarps, sizeof(VjpBlockShared));
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return occ;
+}
+
+cudaError_t launch_vjp_msym(const VjpMsymArgs &a, int grid, cudaStream_t s) {
+  vjp_msym_block_kernel<<<grid, 32 * kBlkWarps, sizeof(VjpBlockShared), s>>>(a);
+  return cudaGetLastError();
 }
 
 }  // namespace nb

@@ -295,9 +295,8 @@ __global__ void __launch_bounds__(THREADS) vjp_kernel(const VjpArgs a) {
 // and update, FP64 work whose cost does not depend on the active lanes, are
 // spread over four sub-partitions and N / 32 CTAs.  (One thread per body in
 // CTAs of 256 kept 9 SMs busy at 2,131 bodies, with 276 FP64 operations in a
-// row where a warp now has 69.)  Mixed
-// rows are many at 128-entry blocks, so kAdjParts warps share a component's
-// rows, part p taking rows p, p + kAdjParts, ...
+// row where a warp now has 69.)  Mixed rows are many with 128-entry blocks, so
+// kParts warps share a component's rows, part p taking rows p, p + kParts, ...
 template <int PREC>
 struct AdjShape {
   static constexpr int kParts = PREC == 0 ? 1 : 2;

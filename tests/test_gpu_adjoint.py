@@ -242,3 +242,21 @@ def test_grad_vs_gpu_central_difference(nb, precision, h):
         fd = (loss(s.r + h * ur, s.v + h * uv, s.m + h * um) - loss(s.r - h * ur, s.v - h * uv, s.m - h * um)) / (2 * h)
         ad = float((dr * ur).sum() + (dv * uv).sum() + (dm * um).sum())
         assert abs(fd - ad) <= tol * abs(ad) + 1e-12, (fd, ad)
+
+
+@pytest.mark.parametrize("n", [2048, 2049, 4352])
+def test_mixed_product_each_pair_once(nb, n):
+    """Sizes at which the mixed product runs on 128-entry pair-once blocks (a
+    full last block, one entry past it, and the largest single round), one step
+    with checkpoints: every element within 1e-3 of its magnitude sum, the mixed
+    gate."""
+    s = inputs.solar_system(n, seed=4, moon_omega_dt_max=0.5)
+    rng = np.random.default_rng(n)
+    gr, gv = rng.normal(size=(3, n)), rng.normal(size=(3, n))
+    b = nb.NBody(s.r, s.v, s.m, G=s.G, dt=s.dt, precision="mixed", ckpt_every=1)
+    assert b.pair_once_block == 128
+    got = [t.cpu().numpy() for t in b.grad(2, gr, gv)]
+    b.close()
+    ref = oracle.grad(s.G, s.dt, 2, s.r, s.v, s.m, gr, gv, magnitudes=True)
+    for g, want, mag in zip(got, ref[:3], ref[3:]):
+        assert np.all(np.abs(g - want) <= 1e-3 * mag)
