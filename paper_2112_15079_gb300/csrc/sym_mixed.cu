@@ -224,7 +224,6 @@ __global__ void __launch_bounds__(32 * kMsymMaxWarps, 1) force_msym_kernel(const
   __shared__ int s_item;
   __shared__ volatile int s_done[kMsymMaxWarps];  // phases each warp has finished
   grid_dependency_wait();    // staged sources and boxes of this step are complete
-  grid_dependency_launch();  // the Verlet kernel may start launching
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   const int W = a.warps, T = a.tiles, BT = 32 * T, NC = T / 2;
   MsymWarp &ws = reinterpret_cast<MsymWarp *>(msym_smem)[w];
@@ -241,7 +240,10 @@ __global__ void __launch_bounds__(32 * kMsymMaxWarps, 1) force_msym_kernel(const
     for (int k = tid; k < 6 * BT; k += 32 * W) s_j[k] = 0.f;
     __syncthreads();
     const int item = s_item;
-    if (item >= a.n_pairs) break;
+    if (item >= a.n_pairs) {
+      grid_dependency_launch();  // the Verlet kernel may launch as the CTAs run out of items
+      break;
+    }
     const int4 pr = a.pairs[item];  // (first stage entry of the system, its bodies, block I, block J)
     const int s0 = pr.x, ns = pr.y, I = pr.z, J = pr.w;
     const int nst = (ns + 1) & ~1;  // the system's stage entries (padded to even)
@@ -418,7 +420,6 @@ __global__ void __launch_bounds__(32 * kBlkWarps, 4) force_msym_block_kernel(con
   MsymBlockShared &sh = *reinterpret_cast<MsymBlockShared *>(msym_smem);
   __shared__ int s_item;
   grid_dependency_wait();    // staged sources and boxes of this step are complete
-  grid_dependency_launch();  // the Verlet kernel may start launching
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   const int chunk = w >> 1, K0 = 16 * (w & 1);
   const size_t N = static_cast<size_t>(a.N);
@@ -585,6 +586,10 @@ __global__ void __launch_bounds__(32 * kBlkWarps, 4) force_msym_block_kernel(con
     pn = describe(s_item);  // (written before the barrier above; used an item later)
     bb ^= 1;
   }
+  // The Verlet kernel may launch as the CTAs run out of items (let in at the
+  // start, its CTAs that found no room piled onto the SMs that finished first:
+  // 4,096 bodies 19.3 us per step, 17.4 so; 65,536 1.498 and 1.487 ms).
+  grid_dependency_launch();
   cp_async_wait_all();
   __syncthreads();
   // The last CTA out resets the item counter for the next launch.
