@@ -89,13 +89,17 @@ __device__ __forceinline__ void close_stage(const CloseArgs &a, int b, int c, do
 // a group working on component c, ten groups to a warp.  Group t evaluates
 // the force term on one side of one pair (t = 2 pair + side), another group
 // holds one member; positions and terms pass through shared memory, with a
-// barrier over the warps in use only (one warp up to 5 pairs).  mu |d|^-3
-// comes from the integer pipes.  The chain of a sub-step is then 4 FP64
-// operations (drift, difference, term, kick; plus one per further partner)
-// and one integer chain.  Measured on GB300, 10,425 bodies with 23 close pairs
-// in 13 clusters, k <= 292: 2.1 -> 0.78 us per sub-step, 0.76 -> 0.32 ms per
-// mixed step (one thread per pair and per member, 29 FP64 operations and two
-// barriers of 256 threads a sub-step before).
+// barrier over the warps in use only (one warp up to 5 pairs).  Measured on
+// GB300, 131 bodies with 23 close pairs in 13 clusters, k <= 292: 2.07 ->
+// 0.92 us per sub-step (one thread per pair and per member and two barriers
+// of 256 threads a sub-step before).
+//
+// The near forces keep the FP64 series and the two half kicks of the scheme as
+// written, although the integer factors (inv_cube.h) and one kick for two
+// would take 0.74 us: a member's position is rounded at its heliocentric
+// magnitude, some 1e-11 of a fast moon's orbit, and each such rounding that
+// falls the other way moves the orbit's phase by as much per radian, so other
+// low bits in the near force part two runs by 1e-9 within a few steps.
 constexpr int kGroups = 10;  // groups of three lanes per warp
 constexpr int kCloseWarps = kCloseThreads / 32;
 // Members a group holds at most: one unless every warp is in use.
@@ -104,7 +108,7 @@ constexpr int kHeldMax = (kCloseThreads + kGroups * kCloseWarps - 1) / (kGroups 
 struct CloseShared {
   double (*r)[3];       // positions of the members
   double (*u)[3];       // term of side t & 1 of pair t >> 1
-  const ic::Mass *mu;
+  const double *mu;
   const int16_t *ia, *ib;  // the pairs' members
   const int16_t *task;     // the members' terms, each in ascending partner order
 };
@@ -158,13 +162,13 @@ __device__ __forceinline__ void close_run(const CloseArgs &a, const CloseShared 
   // This lane's first pair side (with few pairs the only one).
   const int t1 = live && group < 2 * np ? group : 0;
   const int ia1 = sh.ia[t1 >> 1], ib1 = sh.ib[t1 >> 1];
-  const ic::Mass mu1 = sh.mu[t1 & 1 ? ia1 : ib1];
-  auto term = [&](int t, int ia, int ib, const ic::Mass &mu, bool real) {
+  const double mu1 = sh.mu[t1 & 1 ? ia1 : ib1];
+  auto term = [&](int t, int ia, int ib, double mu, bool real) {
     const double d = sh.r[ib][c] - sh.r[ia][c];
     const int l0 = lane - c;
     const double dx = __shfl_sync(0xffffffffu, d, l0), dy = __shfl_sync(0xffffffffu, d, min(l0 + 1, 31)),
                  dz = __shfl_sync(0xffffffffu, d, min(l0 + 2, 31));
-    if (real) sh.u[t][c] = source_factor<false>(dx, dy, dz, mu, false) * (t & 1 ? -d : d);
+    if (real) sh.u[t][c] = mu * inv_r3(fma(dz, dz, fma(dy, dy, dx * dx))) * (t & 1 ? -d : d);
   };
   // A_near at the positions in sh.r, into an.
   auto near = [&]() {
@@ -189,21 +193,21 @@ __device__ __forceinline__ void close_run(const CloseArgs &a, const CloseShared 
   for (int sub = 0; sub < k; ++sub) {
     // (the previous near() ended with a barrier after its last read of the
     // positions, so they may be overwritten now)
-    const double kick = sub == 0 ? hh : h;  // the half kicks of two sub-steps at once
 #pragma unroll
     for (int s = 0; s < HELD; ++s) {
       if (!own[s]) continue;
-      vh[s] = fma(kick, an[s], vh[s]);
+      vh[s] = fma(hh, an[s], vh[s]);
       r[s] = fma(h, vh[s], r[s]);
       sh.r[group + s * stride][c] = r[s];
     }
     near();
+#pragma unroll
+    for (int s = 0; s < HELD; ++s) vh[s] = fma(hh, an[s], vh[s]);
   }
 #pragma unroll
   for (int s = 0; s < HELD; ++s) {
     if (!own[s]) continue;
     const int mi = m0 + group + s * stride, b = a.mem_body[mi];
-    vh[s] = fma(hh, an[s], vh[s]);
     if (!(isfinite(an[s]) && isfinite(vh[s]))) atomicOr(a.flags, kFlagNonFinite);
     a.vh[c * M + mi] = vh[s];
     a.an[c * M + mi] = an[s];
@@ -214,7 +218,7 @@ __device__ __forceinline__ void close_run(const CloseArgs &a, const CloseShared 
 __global__ void __launch_bounds__(kCloseThreads) close_kernel(const CloseArgs a) {
   __shared__ double s_r[kCloseThreads][3];
   __shared__ double s_u[2 * kCloseMaxPairs][3];  // term of side t & 1 of pair t >> 1
-  __shared__ ic::Mass s_mu[kCloseThreads];
+  __shared__ double s_mu[kCloseThreads];
   __shared__ int16_t s_ia[kCloseMaxPairs], s_ib[kCloseMaxPairs];
   __shared__ int16_t s_task[2 * kCloseMaxPairs];  // the members' terms, each in ascending partner order
   grid_dependency_wait();    // the far forces, and the state and stage the Verlet kernel wrote
@@ -229,7 +233,7 @@ __global__ void __launch_bounds__(kCloseThreads) close_kernel(const CloseArgs a)
   }
   for (int t = threadIdx.x; t < nm; t += kCloseThreads) {
     const int b = a.mem_body[m0 + t];
-    s_mu[t] = ic::pack_mass(a.G * a.m[b]);
+    s_mu[t] = a.G * a.m[b];
     s_r[t][0] = a.x[b];
     s_r[t][1] = a.y[b];
     s_r[t][2] = a.z[b];
