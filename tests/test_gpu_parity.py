@@ -191,10 +191,10 @@ def test_grid_kernel_vs_general_and_oracle(nb, n, steps):
         assert np.max(np.linalg.norm(a - a_ref, axis=0) / np.linalg.norm(a_ref, axis=0)) <= FP64_TOL
 
 
-@pytest.mark.parametrize("n", [152, 153, 305, 456, 457, 609, 1216, 1217, 2432, 2433])
+@pytest.mark.parametrize("n", [152, 153, 305, 456, 457, 609, 1216, 1217, 1824, 1825])
 def test_grid_kernel_shapes(nb, n):
-    """The edges of the grid kernel's shapes (1 to 16 targets to a CTA, 4, 2
-    or 1 warps to a target, on 152 SMs; 2,433 bodies take the general path)
+    """The edges of the grid kernel's shapes (1 to 12 targets to a CTA, 4, 2
+    or 1 warps to a target, on 152 SMs; 1,825 bodies take the general path)
     against the oracle, in the tolerance of the test above."""
     steps = 5
     s = inputs.solar_system(n, seed=74, n_moons=0)
