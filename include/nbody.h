@@ -141,9 +141,13 @@ typedef struct {
    *   in a spatial order).  Automatic: for a largest system of at least
    *   65,536 bodies, the narrowest of 128 .. 2,048 that leaves it at most 128
    *   partial sums per body, if the block pairs keep 8 warps per SM busy and
-   *   the sums take at most 16 GiB (else, and below 65,536 bodies, every
-   *   ordered pair is evaluated).  Or set: a power of two from 128 to 2,048.
-   *   Force only (nbody_grad's VJP evaluates every ordered pair).
+   *   the sums take at most 16 GiB.  Below 65,536 bodies: 128 while the sums
+   *   stay in the L2 cache and the block pairs fill the GPU at most once or
+   *   at least five times (on 152 SMs one system of 2,048 to 4,352 or 9,857
+   *   to about 20,600 bodies, or many systems), 512 where the sums would
+   *   leave the cache; else every ordered pair is evaluated.  Or set: a power
+   *   of two from 128 to 2,048.  128 applies to the VJP of nbody_grad too,
+   *   wider blocks to the force only.
    * A set size is used whatever the systems' sizes (for contexts that are
    * not row shards) if the partial sums take at most 16 GiB and 65,535 blocks
    * per system, else nbody_init returns EINVAL. */
@@ -153,19 +157,19 @@ typedef struct {
 /* Launch nbody_step's kernels directly instead of replaying CUDA graphs. */
 #define NBODY_FLAG_NO_GRAPH 1
 /* Never use the single-launch kernels (one FP64 Verlet system of at most
- * 4,096 bodies runs every step of an nbody_step call in one launch: of an
+ * 12 bodies per SM, 1,824 on 152 SMs, runs every step of an nbody_step call in one launch: of an
  * 8- or 16-CTA cluster up to 96 bodies, of a cooperative grid beyond,
  * unless this flag is set). */
 #define NBODY_FLAG_NO_SMALL 2
 /* Use the force kernel that evaluates every ordered pair (p, j) on its
  * own, instead of the default one that evaluates each pair once and applies
  * it to both bodies (a_p += mu_j |d|^-3 d, a_j -= mu_p |d|^-3 d: Eq. 1 to
- * rounding, 20 FP64 operations per two interactions instead of 32; mixed:
+ * rounding, 6 FP64 operations per two interactions instead of 12; mixed:
  * 16 FP32 operations per two interactions of a far pair instead of 24).
  * FP64 uses it for contexts that are not row shards, when the systems hold
  * at least 1.5 block pairs per SM (64-body blocks: about 1,200 bodies in one
  * system; below that the other kernel is faster) and the partial sums fit;
- * mixed for systems of at least 65,536 bodies (nbody_opts.pair_once_block). */
+ * mixed by the sizes at nbody_opts.pair_once_block. */
 #define NBODY_FLAG_NO_SYM 4
 
 /* Work decomposition of the force kernels (see nbody_set_tiles).  The work
@@ -215,7 +219,7 @@ nbody_status nbody_init(nbody_ctx **out, int64_t n_systems, const int64_t *offse
  * at the new positions, so the context's acceleration always belongs to the
  * current state.  Consecutive steps are replayed from cached CUDA graphs
  * unless NBODY_FLAG_NO_GRAPH is set or the stream is already being
- * captured.  One FP64 Verlet system of at most 4,096 bodies instead runs
+ * captured.  One small FP64 Verlet system (at most 12 bodies per SM) runs
  * all n_steps in a single launch (see NBODY_FLAG_NO_SMALL). */
 nbody_status nbody_step(nbody_ctx *ctx, int64_t n_steps);
 

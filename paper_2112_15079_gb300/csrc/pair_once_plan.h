@@ -9,12 +9,14 @@
 //   (rows <= 1.6 GB at 65,536); else the narrowest wide block (256 .. 4,096
 //   bodies) whose rows fit in kSymRowBudget, else 4,096 if they fit in
 //   kSymRowLimit (else none); used when the systems hold at least 1.5 block
-//   pairs per SM (with fewer, one CTA carries a system's whole sum and the
-//   stream-K kernel is faster: measured on GB300, 1,031 bodies / 153 pairs
-//   60.8 against 55.3 us per step, 1,283 bodies / 231 pairs 62.5 against
-//   96.2).
+//   pairs per SM (with fewer, one CTA carries a system's whole sum; measured
+//   on GB300, us per step, pair-once against every ordered pair: 600 bodies
+//   44.5 / 30.6, 1,031 bodies / 153 pairs 45.8 / 51.9, 1,283 bodies / 231 pairs
+//   46.3 / 60.6, 10,425 bodies 649 / 1,240; since both kernels take their
+//   reciprocal cubes from the integer pipes they meet near 800 bodies, which
+//   only contexts without the single-launch kernels see).
 //   Mixed (stage entries per block): for a largest system of at least
-//   kMsymMinBodies (measured on GB300: 65,536 bodies 1.50 against 1.82 ms
+//   kMsymMinBodies (measured on GB300: 65,536 bodies 1.49 against 1.82 ms
 //   per step, 1,048,576 bodies 340 against 430 ms), the narrowest block (128 ..
 //   2,048 entries) that leaves the largest system at most kMsymMaxRows rows
 //   per body, if the rows fit in kSymRowLimit and the block pairs give at
@@ -99,10 +101,10 @@ inline int pair_once_block(const std::vector<int64_t> &sizes, bool mixed, int64_
 // Mixed systems below kMsymMinBodies: 128-entry blocks (force_msym_block_kernel,
 // four warps to a block pair), or 512, or 0 for the every-ordered-pair
 // kernel.  Measured on GB300, us per step, every ordered pair / 128 / 512:
-//   bodies          31    300   1,031  2,131  4,096  5,003  8,192  10,425  20,011  32,768  50,001
-//   ordered        9.6   10.5    14.3   17.7   23.3   26.8   45.7    68.1     208     517    1077
-//   128            9.8   10.1    10.2   12.9   20.2   35.6   47.5    61.3     185     702    2057
-//   512                                                              86.9     194     431     915
+//   bodies     31   300  1,031  2,131  4,096  5,003  8,192  9,000  10,425  20,011  32,768  50,001
+//   ordered   8.9  10.7   14.8   18.0   24.0   27.1   46.3   53.9    68.6     207     516    1075
+//   128      10.0  10.2   11.0   12.5   18.0   36.2   47.4   49.9    62.4     184     702    2057
+//   512      18.5  41.1   58.7   58.8   59.4   60.1   60.9   84.8    86.3     197     429     893
 //   systems x bodies  64 x 40..400  2,000 x 500  10 x 5,000  100 x 5,000  64 x 1,000..20,000
 //   ordered                   22.4          610         171         1338                4529
 //   128                       14.1          484         140         1871                9027

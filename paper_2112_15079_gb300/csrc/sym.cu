@@ -7,7 +7,7 @@
 // the differences run on the integer pipes (inv_cube.h), about 185
 // instructions beside the 6 FP64 accumulations that are left.  Measured on
 // GB300, 10,425 bodies: 2.03 ms per step with 20 FP64 operations, 0.94 ms with
-// 9 (FP64 differences), 0.69 ms with 6 (the launch 0.62 ms; 6 x 76 cycles a pair
+// 9 (FP64 differences), 0.65 ms with 6 (the launch 0.62 ms; 6 x 76 cycles a pair
 // and warp step are 0.61: the FP64 pipe stays the bound).
 //
 // Decomposition: each system's bodies are cut into blocks of 64 (two warp

@@ -194,7 +194,7 @@ class NBody:
     @property
     def pair_once(self) -> bool:
         """Whether the force launches evaluate each pair once (FP64 from ~1,200
-        bodies, mixed from 65,536; see ``pair_once_block``)."""
+        bodies, mixed by size, most from 2,048; see ``pair_once_block``)."""
         return self.pair_once_block > 0
 
     @property
