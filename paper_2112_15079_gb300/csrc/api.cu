@@ -1826,8 +1826,10 @@ nbody_status nbody_grad(nbody_ctx *c, int64_t n_steps, const double *dL_dr_T, co
       vs.n_pairs = A.vj.n_sym;
       vs.ctr = A.vj.dyn_ctr;
       vs.N = c->N;
+      vs.flags = c->flags;
+      vs.stall = ++c->wait_seq == c->stall_at ? 1 : 0;
       NB_CUDA(c, nb::launch_vjp_msym(vs, A.vj.grid, c->stream));
-    } else if (A.vj.sym_pairs) {  // pair-once: no bounded wait to stall
+    } else if (A.vj.sym_pairs) {  // pair-once (FP64): no bounded wait to stall
       nb::VjpSymArgs vs{};
       vs.pos = static_cast<const double4_32a *>(pos);
       vs.w = static_cast<const double4_32a *>(A.w);

@@ -180,9 +180,11 @@ struct VjpMsymArgs {
   double *partial;         // [blocks][4][N] float pairs
   const int4 *pairs;       // as MsymArgs::pairs
   const int32_t *perm;
+  unsigned *flags;
   int32_t n_pairs;
   int32_t *ctr;
   int32_t N;
+  int32_t stall;           // test hook: CTA 0 leaves out one arrival
 };
 
 // Close-encounter handling (close.cu): clusters of close pairs sub-cycled in

@@ -69,6 +69,10 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// One arrival on `bar` when this thread's copies so far have landed.
+__device__ __forceinline__ void cp_async_arrive(uint64_t *bar) {
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Union of the widened boxes of the stage groups that hold entries [e0, e1).
@@ -616,6 +620,10 @@ __global__ void __launch_bounds__(32 * kBlkWarps, 4) force_msym_block_kernel(con
 // Sums: a target has 32 terms per half and warp; its halves are added plainly
 // (64 terms), its two warps' sums through TwoSum; a source has 64 terms from
 // each of its two warps, added through TwoSum.
+//
+// An item's copies arrive on the mbarrier of its buffer, and the CTA waits for
+// them with a limit: a wait that runs out sets kFlagTimeout and the CTA leaves.
+// Test hook: with a.stall set, thread 0 of CTA 0 leaves out its first arrival.
 struct VjpBlockShared {
   float4 src[2][2][4][64];     // [buffer][block I, J][piece][pair block]
   float4 wsrc[2][2][2][64];    // the same of w: (wx0 wx1 wy0 wy1), (wz0 wz1 - -)
@@ -684,11 +692,12 @@ __global__ void __launch_bounds__(32 * kBlkWarps, 4) vjp_msym_block_kernel(const
   extern __shared__ __align__(16) unsigned char msym_smem[];
   VjpBlockShared &sh = *reinterpret_cast<VjpBlockShared *>(msym_smem);
   __shared__ int s_item;
+  __shared__ __align__(8) uint64_t bar[2];
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   const int half = w >> 1, chunk = w & 1;
   const size_t N = static_cast<size_t>(a.N);
   auto describe = [&](int item) { return item < a.n_pairs ? a.pairs[item] : make_int4(0, 0, 0, 0); };
-  auto stage_item = [&](const int4 &pr, int bb) {
+  auto stage_item = [&](const int4 &pr, int bb, bool stall) {
     if (pr.y > 0) {
       const int nst = (pr.y + 1) & ~1;
 #pragma unroll
@@ -707,28 +716,34 @@ __global__ void __launch_bounds__(32 * kBlkWarps, 4) vjp_msym_block_kernel(const
                                   : make_float4(x0, x1, 0.f, 0.f);
         }
       }
+      if (!stall) cp_async_arrive(&bar[bb]);
     }
-    cp_async_commit();
   };
   // (item numbers, descriptors and data run ahead as in force_msym_block_kernel)
   int fetched = 0;  // thread 0
   if (tid == 0) {
     s_item = static_cast<int>(gridDim.x) + atomicAdd(a.ctr, 1);
     fetched = static_cast<int>(gridDim.x) + atomicAdd(a.ctr, 1);
+    mbar_init(&bar[0], 32 * kBlkWarps);
+    mbar_init(&bar[1], 32 * kBlkWarps);
+    mbar_init_fence();
   }
   int4 pr = describe(blockIdx.x);
-  stage_item(pr, 0);
   __syncthreads();
+  stage_item(pr, 0, a.stall != 0 && blockIdx.x == 0 && tid == 0);
   int4 pn = describe(s_item);
   int bb = 0;
+  uint32_t parity = 0;
   while (pr.y > 0) {
-    cp_async_wait_all();
-    __syncthreads();  // this item's blocks are in; the previous item's sums (and s_item) are consumed
+    if (__syncthreads_or(!mbar_wait(&bar[bb], parity))) {
+      if (tid == 0) atomicOr(a.flags, kFlagTimeout);
+      break;
+    }  // this item's blocks are in; the previous item's sums (and s_item) are consumed
     if (tid == 0) {
       s_item = fetched;
       fetched = static_cast<int>(gridDim.x) + atomicAdd(a.ctr, 1);
     }
-    stage_item(pn, bb ^ 1);
+    stage_item(pn, bb ^ 1, false);
     const int s0 = pr.x, ns = pr.y, I = pr.z, J = pr.w;
     const int nst = (ns + 1) & ~1;
     const bool diag = I == J;
@@ -800,6 +815,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, 4) vjp_msym_block_kernel(const
     pr = pn;
     pn = describe(s_item);  // (written before the barrier above; used an item later)
     bb ^= 1;
+    parity ^= bb ^ 1;  // each buffer's every second use
   }
   cp_async_wait_all();
   __syncthreads();
