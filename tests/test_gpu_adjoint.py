@@ -260,3 +260,21 @@ def test_mixed_product_each_pair_once(nb, n):
     ref = oracle.grad(s.G, s.dt, 2, s.r, s.v, s.m, gr, gv, magnitudes=True)
     for g, want, mag in zip(got, ref[:3], ref[3:]):
         assert np.all(np.abs(g - want) <= 1e-3 * mag)
+
+
+@pytest.mark.parametrize("precision,n", [("fp64", 131), ("fp64", 1283), ("mixed", 131), ("mixed", 2049)])
+def test_gradient_independent_of_checkpoints(nb, precision, n):
+    """Seven steps in seven, three and one segments (the first and the last
+    segment reuse a force of the forward sweep): the recomputed states, hence
+    every element, are the same bits."""
+    s = inputs.solar_system(n, seed=6, moon_omega_dt_max=0.5)
+    rng = np.random.default_rng(n)
+    gr, gv = rng.normal(size=(3, n)), rng.normal(size=(3, n))
+    runs = []
+    for every in (1, 3, 7, 100):
+        b = nb.NBody(s.r, s.v, s.m, G=s.G, dt=s.dt, precision=precision, ckpt_every=every)
+        runs.append([t.cpu().numpy() for t in b.grad(7, gr, gv)])
+        b.close()
+    for got in runs[1:]:
+        for x, y in zip(got, runs[0]):
+            assert np.array_equal(x, y)
