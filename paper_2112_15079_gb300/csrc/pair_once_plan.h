@@ -37,7 +37,7 @@ constexpr int kSymBlock = 64;
 constexpr int kSymThreads = 64;       // two warps: one 32-body tile of block I each
 constexpr int kSymMaxBodies = 65536;  // per system, by default (the partial rows are [blocks][3][N])
 // FP64 wide blocks of 32 T bodies (force_sym_wide_kernel) above that: T tiles.
-constexpr int kSymWideWarps = 4;
+constexpr int kSymWideWarps = 4;       // per CTA (the widest blocks: 8)
 constexpr int kSymWideThreads = 32 * kSymWideWarps;
 constexpr int kSymWideMinTiles = 8;    // 256 bodies
 constexpr int kSymWideMaxTiles = 128;  // 4,096 bodies (96 KB of shared sums)

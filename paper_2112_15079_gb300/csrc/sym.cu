@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(kSymThreads) force_sym_kernel(const SymArgs a)
 // Wide blocks, for systems whose 64-body blocks would need too many partial
 // rows (one per block): blocks of B = 32 T bodies (T tiles, a power of two,
 // kSymWideMinTiles .. kSymWideMaxTiles), so a body has one row per B bodies
-// of its system.  A CTA of kSymWideWarps warps takes an item (I, J).  In
+// of its system.  A CTA of W warps takes an item (I, J).  In
 // round r warp w holds tile p = r W + w of block I in registers; in phase
 // t = 0 .. T-1 it rotates tile q = (p + t) mod T of block J past it, as
 // force_sym_kernel does, and adds the tile's reaction sums into block J's
@@ -287,17 +287,20 @@ __global__ void __launch_bounds__(kSymThreads) force_sym_kernel(const SymArgs a)
 // tile pairs q >= p only (q == p as the 16-step half rotation); each warp
 // adds its tile's own sums into the shared sums after its round, and the
 // total goes to row I.  Tiles past the end of the system are skipped.
-__global__ void __launch_bounds__(kSymWideThreads) force_sym_wide_kernel(const SymArgs a) {
+// W is kSymWideWarps, four CTAs to an SM, and twice that for the widest
+// blocks, whose 96 KB of shared sums leave two CTAs: 16 warps an SM either way.
+// With 8, 1,048,576 bodies took 8.48 s per step, 6.24 so.
+__global__ void __launch_bounds__(2 * kSymWideThreads, 2) force_sym_wide_kernel(const SymArgs a) {
   extern __shared__ double s_acc[];  // [3][32 T]: block J's reaction sums of the item
   __shared__ int s_item;
   grid_dependency_wait();    // staged sources of this step are complete
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-  const int T = a.tiles, BT = 32 * T;
+  const int T = a.tiles, BT = 32 * T, W = blockDim.x >> 5;
   const size_t N = static_cast<size_t>(a.N);
   for (;;) {
     __syncthreads();  // the previous item's shared sums are consumed
     if (tid == 0) s_item = atomicAdd(a.ctr, 1);
-    for (int k = tid; k < 3 * BT; k += kSymWideThreads) s_acc[k] = 0.0;
+    for (int k = tid; k < 3 * BT; k += 32 * W) s_acc[k] = 0.0;
     __syncthreads();
     const int item = s_item;
     if (item >= a.n_pairs) break;
@@ -306,7 +309,7 @@ __global__ void __launch_bounds__(kSymWideThreads) force_sym_wide_kernel(const S
     const int ns = pr.y, I = pr.z, J = pr.w;
     const bool diag = I == J;
     const int i0 = I * BT, j0 = J * BT;  // first body of each block within the system
-    for (int r = 0; r < T; r += kSymWideWarps) {
+    for (int r = 0; r < T; r += W) {
       const int p = r + w;
       const bool p_live = i0 + p * 32 < ns;  // warp-uniform
       const double4_32a pi = sym_load(a.cur, sb, i0 + p * 32 + lane, ns, 1e15 * (lane + 1));
@@ -354,7 +357,7 @@ __global__ void __launch_bounds__(kSymWideThreads) force_sym_wide_kernel(const S
     __syncthreads();
     // block J's sums (on a diagonal item, the block's whole sums) to row I
     double *row = a.partial + static_cast<size_t>(I) * 3 * N;
-    for (int k = tid; k < BT && j0 + k < ns; k += kSymWideThreads) {
+    for (int k = tid; k < BT && j0 + k < ns; k += 32 * W) {
       row[sb + j0 + k] = s_acc[k];
       row[N + sb + j0 + k] = s_acc[BT + k];
       row[2 * N + sb + j0 + k] = s_acc[2 * BT + k];
@@ -506,10 +509,14 @@ size_t force_sym_smem_bytes(int tiles) {
   return tiles == 2 ? 0 : sizeof(double) * 3 * 32 * static_cast<size_t>(tiles);
 }
 
+namespace {
+int sym_wide_threads(int tiles) { return tiles == kSymWideMaxTiles ? 2 * kSymWideThreads : kSymWideThreads; }
+}  // namespace
+
 cudaError_t launch_force_sym(const SymArgs &a, int grid, cudaStream_t s, bool chained) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(a.tiles == 2 ? kSymThreads : kSymWideThreads);
+  cfg.blockDim = dim3(a.tiles == 2 ? kSymThreads : sym_wide_threads(a.tiles));
   cfg.dynamicSmemBytes = force_sym_smem_bytes(a.tiles);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -531,7 +538,7 @@ int force_sym_ctas_per_sm(int tiles) {
     e = cudaFuncSetAttribute(force_sym_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(force_sym_smem_bytes(kSymWideMaxTiles)));
     if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, force_sym_wide_kernel, kSymWideThreads, smem);
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, force_sym_wide_kernel, sym_wide_threads(tiles), smem);
   }
   if (e != cudaSuccess) {
     cudaGetLastError();

@@ -125,6 +125,15 @@ def test_wide_fp64_schedule(T):
     _check_diagonal(seen, 32 * T)
 
 
+@pytest.mark.parametrize("T", [8, 16])
+def test_wide_fp64_schedule_eight_warps(T):
+    """The widest blocks' CTAs of eight warps, in fewer tiles."""
+    for diag, check in ((False, _check_off_diagonal), (True, _check_diagonal)):
+        ex, seen = wide_fp64_item(T, diag=diag, warps=8)
+        assert ex
+        check(seen, 32 * T)
+
+
 @pytest.mark.parametrize("T", [4, 8, 16])
 def test_mixed_schedule(T):
     ex, folds, seen = mixed_item(T, diag=False)
