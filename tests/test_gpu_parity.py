@@ -228,6 +228,28 @@ def test_small_systems_beyond_the_integer_path(nb, n, r_scale, m_scale):
     b.close()
 
 
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 96, 97, 131, 521, 1824])
+def test_a_body_among_massless_ones_feels_nothing(nb, n):
+    """Eq. 1 over massless bodies is exactly zero, and so is a single body's
+    sum: the star of a system of test particles keeps a = 0 and its position to
+    the bit in the single-launch kernels, whose lanes without a source take a
+    massless stand-in."""
+    s = inputs.solar_system(max(n, 31), seed=75, n_moons=0)
+    r, v, m = s.r[:, :n].copy(), s.v[:, :n].copy(), np.zeros(n)
+    m[0] = 1.0
+    v[:, 0] = 0.0
+    b = nb.NBody(r, v, m, G=s.G, dt=s.dt, precision="fp64")
+    b.step(3)
+    a = b.accel().cpu().numpy()
+    assert np.array_equal(a[:, 0], np.zeros(3))
+    assert np.array_equal(b.r.cpu().numpy()[:, 0], r[:, 0])
+    if n > 1:
+        d = b.r.cpu().numpy()[:, :1] - b.r.cpu().numpy()[:, 1:]
+        ref = s.G * d / np.linalg.norm(d, axis=0) ** 3
+        assert np.max(_rel_err(a[:, 1:], ref)) <= FP64_TOL
+    b.close()
+
+
 def test_grid_kernel_wait_timeout_reports_and_recovers(nb, monkeypatch):
     """NBODY_INJECT_WAIT_STALL=1 makes CTA 0 of the cooperative grid kernel
     (257 bodies) skip its first barrier arrival: every CTA's bounded wait
