@@ -145,9 +145,11 @@ typedef struct {
    *   stay in the L2 cache and the block pairs fill the GPU at most once or
    *   at least five times (on 152 SMs one system of 2,048 to 4,352 or 9,857
    *   to about 20,600 bodies, or many systems), 512 where the sums would
-   *   leave the cache; else every ordered pair is evaluated.  Or set: a power
-   *   of two from 128 to 2,048.  128 applies to the VJP of nbody_grad too,
-   *   wider blocks to the force only.
+   *   leave the cache (at most 4 GiB of sums, a third more for nbody_grad);
+   *   else every ordered pair is evaluated, as in contexts of several systems
+   *   whose largest coordinates lie more than a factor 2^20 apart.  Or set: a
+   *   power of two from 128 to 2,048.  128 applies to the VJP of nbody_grad
+   *   too, wider blocks to the force only.
    * A set size is used whatever the systems' sizes (for contexts that are
    * not row shards) if the partial sums take at most 16 GiB and 65,535 blocks
    * per system, else nbody_init returns EINVAL. */

@@ -5,6 +5,7 @@
 // CUDA-graph replay of Verlet, leapfrog and RK4 steps, the adjoint sweep,
 // energy, tiles/autotuning and device-fault reporting.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -108,6 +109,7 @@ struct nbody_ctx {
   int32_t *perm = nullptr;           // [n_stage] body of each stage entry (mixed; padding: any body)
   float4 *boxes = nullptr;           // mixed: [n_stage / 64 rounded up][2] source-group boxes of the next force launch
   std::vector<int32_t> qidx_h;       // host copy of qidx (mixed)
+  int unit_lo = 0, unit_hi = 0;      // exponents of the systems' largest coordinates, least and greatest (mixed)
   // mixed, for planning (see chunk_costs): per stage entry its hi parts and
   // the magnitudes of its lo parts ([n_stage][6]); per source group of
   // 2 kBoxPairs entries its widened box
@@ -359,12 +361,14 @@ nbody_status build_work(nbody_ctx *c, Work &wk, const nbody_tiles &t, int occ, i
 
 // Block size of the pair-once force kernels for this context
 // (pair_once_plan.h), or 0 where the every-ordered-pair kernel runs: row
-// shards, NBODY_FLAG_NO_SYM, and the cases pair_once_block turns down.
+// shards, NBODY_FLAG_NO_SYM, mixed systems whose positions share no unit, and
+// the cases pair_once_block turns down.
 int sym_block(const nbody_ctx *c) {
   if (c->sh_world > 0 || (c->o.flags & NBODY_FLAG_NO_SYM)) return 0;
   std::vector<int64_t> sizes(static_cast<size_t>(c->n_sys));
   for (int64_t s = 0; s < c->n_sys; ++s) sizes[s] = c->offsets[s + 1] - c->offsets[s];
   const bool mixed = c->o.precision == NBODY_MIXED;
+  if (mixed && c->o.pair_once_block == 0 && !nb::stage_unit_fits(c->unit_lo, c->unit_hi)) return 0;
   const int B = nb::pair_once_block(sizes, mixed, c->nsm, c->o.pair_once_block);
   return B == 0 && mixed ? nb::msym_small_block(sizes, c->nsm) : B;
 }
@@ -501,6 +505,13 @@ State bound_state(nbody_ctx *c) {
   return {c->x, c->y, c->z, c->vx, c->vy, c->vz, c->a, c->a + N, c->a + 2 * N};
 }
 
+// Mixed pair-once contexts: lengths are staged in units of 2^-k of the caller's
+// (pair_once_plan.h): positions as 2^k r, mu as 2^3k G m.
+int stage_unit(const nbody_ctx *c) {
+  if (c->o.precision != NBODY_MIXED || c->sh_world > 0 || !c->fw.sym_pairs) return 0;
+  return nb::stage_unit_exp(c->unit_lo, c->unit_hi);
+}
+
 nb::PrepArgs prep_args(nbody_ctx *c, const State &s, int drift, int check, void *stage = nullptr) {
   const size_t N = c->N;
   nb::PrepArgs p{};
@@ -516,7 +527,8 @@ nb::PrepArgs prep_args(nbody_ctx *c, const State &s, int drift, int check, void 
   p.N = c->N;
   p.drift = drift;
   p.check = check;
-  p.G = c->o.G;
+  p.unit = stage_unit(c);
+  p.G = std::ldexp(c->o.G, 3 * p.unit);
   p.dt = c->o.dt;
   p.half_dt2 = 0.5 * c->o.dt * c->o.dt;
   return p;
@@ -559,6 +571,7 @@ nb::CloseArgs close_args(nbody_ctx *c, const State &s, void *nxt, int complete) 
   a.n_mem = static_cast<int32_t>(cs.mem_body.size());
   a.complete = complete;
   a.precision = c->o.precision;
+  a.unit = stage_unit(c);
   a.G = c->o.G;
   a.dt = c->o.dt;
   a.half_dt = 0.5 * c->o.dt;
@@ -676,6 +689,7 @@ nb::VerletArgs verlet_args(nbody_ctx *c, const State &s, const void *cur, void *
   a.p_end = c->sh_world > 0 ? static_cast<int32_t>(c->sh_end) : c->N;
   a.mode = mode;
   a.release_early = release_early(c);
+  a.unit = stage_unit(c);
   a.dt = c->o.dt;
   a.half_dt = 0.5 * c->o.dt;
   a.half_dt2 = 0.5 * c->o.dt * c->o.dt;
@@ -700,7 +714,8 @@ nb::RkArgs rk_args(nbody_ctx *c, const State &s, const void *cur, void *nxt, int
   a.N = c->N;
   a.stage = stage;
   a.release_early = release_early(c);
-  a.G = c->o.G;
+  a.unit = stage_unit(c);
+  a.G = std::ldexp(c->o.G, 3 * a.unit);  // (mu of rk_prep only)
   a.dt = c->o.dt;
   return a;
 }
@@ -983,6 +998,18 @@ nbody_status spatial_order(nbody_ctx *c) {
   NB_CUDA(c, cudaMemcpyAsync(h.data() + N, c->y, b, cudaMemcpyDeviceToHost, c->stream));
   NB_CUDA(c, cudaMemcpyAsync(h.data() + 2 * N, c->z, b, cudaMemcpyDeviceToHost, c->stream));
   NB_CUDA(c, cudaStreamSynchronize(c->stream));
+  // Exponents of the systems' largest coordinates, for the stage's unit.
+  c->unit_lo = INT_MAX;
+  c->unit_hi = INT_MIN;
+  for (int64_t s = 0; s < c->n_sys; ++s) {
+    double top = 0.0;
+    for (int k = 0; k < 3; ++k)
+      for (int64_t p = c->offsets[s]; p < c->offsets[s + 1]; ++p) top = std::max(top, std::fabs(h[k * N + p]));
+    if (!(top > 0.0) || !std::isfinite(top)) continue;  // (staging reports what is not finite)
+    c->unit_lo = std::min(c->unit_lo, std::ilogb(top));
+    c->unit_hi = std::max(c->unit_hi, std::ilogb(top));
+  }
+  if (c->unit_lo > c->unit_hi) c->unit_lo = c->unit_hi = 0;
   c->qidx_h.assign(N, 0);
   std::vector<int32_t> perm(static_cast<size_t>(c->n_stage), 0);
   std::vector<std::pair<uint64_t, int32_t>> key;
@@ -1140,11 +1167,18 @@ nbody_status ensure_adjoint(nbody_ctx *c, int64_t n_steps) {
   const size_t N = c->N;
   const int64_t K = c->o.ckpt_every;
   nbody_status st;
-  if (!A.shadow) {  // first use, or an earlier attempt failed part way: start clean
+  // With the narrowest pair-once blocks (FP64 64 bodies, mixed 128 entries) the
+  // VJP evaluates each pair once too.
+  const int B = prec == NBODY_MIXED ? 32 * nb::kMsymMinTiles : nb::kSymBlock;
+  const bool once = c->fw.sym_pairs && 32 * c->fw.sym_tiles == B;
+  // First use, an earlier attempt that failed part way, or a reset that changed
+  // the force kernel: start clean.
+  if (!A.shadow || once != (A.vj.sym_pairs != nullptr)) {
     free_work(c, A.vj);
-    for (void *q : {static_cast<void *>(A.rho), static_cast<void *>(A.nu), static_cast<void *>(A.gm), A.w})
+    for (void *q : {static_cast<void *>(A.rho), static_cast<void *>(A.nu), static_cast<void *>(A.gm), A.w,
+                    static_cast<void *>(A.shadow)})
       dfree(c, q);
-    A.rho = A.nu = A.gm = nullptr;
+    A.rho = A.nu = A.gm = A.shadow = nullptr;
     A.w = nullptr;
     nbody_tiles t{};
     t.threads = nb::vjp_threads(prec);
@@ -1152,10 +1186,7 @@ nbody_status ensure_adjoint(nbody_ctx *c, int64_t n_steps) {
     t.tj = kVjpTile;
     t.jsplit = 0;
     t.ctas_per_sm = 32;
-    // With the narrowest pair-once blocks (FP64 64 bodies, mixed 128 entries) the
-    // VJP evaluates each pair once too.
-    const int B = prec == NBODY_MIXED ? 32 * nb::kMsymMinTiles : nb::kSymBlock;
-    if (sym_block(c) == B) {
+    if (once) {
       if ((st = build_sym_work(c, A.vj, 4, B)) != NBODY_OK) return st;
     } else {
       const size_t smem = nb::vjp_smem_bytes(prec, t.tj);
@@ -1808,6 +1839,7 @@ nbody_status nbody_grad(nbody_ctx *c, int64_t n_steps, const double *dL_dr_T, co
   ad.qidx = c->qidx;
   ad.flags = c->flags;
   ad.N = c->N;
+  ad.unit = stage_unit(c);
   ad.G = c->o.G;
   ad.dt = c->o.dt;
   ad.half_dt = 0.5 * c->o.dt;

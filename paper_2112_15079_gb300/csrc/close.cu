@@ -78,6 +78,7 @@ __device__ __forceinline__ void close_stage(const CloseArgs &a, int b, int c, do
   } else {
     Rc[b] = r;
     float *w = static_cast<float *>(a.stage) + pair_off(a.qidx[b]);
+    r = times_pow2(r, a.unit);
     const float h = hi_part(r);
     w[kXh + 2 * c] = h;
     w[kXl + 2 * c] = lo_part(r, h);

@@ -209,9 +209,10 @@ __device__ __forceinline__ void sum_rows_mixed(const double *partial, int rows, 
 
 // Phase A of a CTA: the acceleration component `comp` of body p0 + k for the
 // thread's phase B (0 beyond component 2).  rows_a: the rows of the thread's
-// phase A body.  Mixed: every thread of the CTA takes part.
+// phase A body; unit: VerletArgs::unit.  Mixed: every thread of the CTA takes part.
 template <int PREC>
-__device__ __forceinline__ double sum_rows(const double *partial, size_t N, int p0, int rows_a, int comp, int k) {
+__device__ __forceinline__ double sum_rows(const double *partial, size_t N, int p0, int rows_a, int comp, int k,
+                                           int32_t unit) {
   if constexpr (PREC == 0) {
     return sum_rows_fp64(partial, rows_a, N, p0 + k, comp);
   } else {
@@ -229,7 +230,8 @@ __device__ __forceinline__ double sum_rows(const double *partial, size_t N, int 
       s_lo[2][b] = ez;
     }
     __syncthreads();
-    return comp < 3 ? static_cast<double>(s_hi[comp][k]) + static_cast<double>(s_lo[comp][k]) : 0.0;
+    if (comp >= 3) return 0.0;
+    return times_pow2(static_cast<double>(s_hi[comp][k]) + static_cast<double>(s_lo[comp][k]), -unit);
   }
 }
 
@@ -256,14 +258,18 @@ __device__ __forceinline__ double step_component(bool leap, double r, double &v,
 
 // Stage position (rx, ry, rz) of body q for the next force launch, with mu
 // copied from the current stage: FP64 double4 at q, or the mixed hi/lo pair
-// block at qidx[q] (mixed: *o is the pair offset, *muf the staged mu).
+// block at qidx[q] (mixed: *o is the pair offset, *muf the staged mu; the
+// position in units of 2^-unit).
 template <int PREC>
 __device__ __forceinline__ void stage_position(void *nxt, int q, size_t o, double rx, double ry, double rz, double mu,
-                                               float muf) {
+                                               float muf, int32_t unit) {
   if (PREC == 0) {
     static_cast<double4_32a *>(nxt)[q] = make_double4_32a(rx, ry, rz, mu);
   } else {
     float *w = static_cast<float *>(nxt) + o;
+    rx = times_pow2(rx, unit);
+    ry = times_pow2(ry, unit);
+    rz = times_pow2(rz, unit);
     const float hx = hi_part(rx), hy = hi_part(ry), hz = hi_part(rz);
     w[kXh] = hx;
     w[kYh] = hy;
@@ -277,13 +283,15 @@ __device__ __forceinline__ void stage_position(void *nxt, int q, size_t o, doubl
 
 // The same, component c by itself (c = 0 also writes mu).
 template <int PREC>
-__device__ __forceinline__ void stage_component(void *nxt, int q, size_t o, int c, double r, double mu, float muf) {
+__device__ __forceinline__ void stage_component(void *nxt, int q, size_t o, int c, double r, double mu, float muf,
+                                                int32_t unit) {
   if (PREC == 0) {
     double *w = reinterpret_cast<double *>(static_cast<double4_32a *>(nxt) + q);
     w[c] = r;
     if (c == 0) w[3] = mu;
   } else {
     float *w = static_cast<float *>(nxt) + o;
+    r = times_pow2(r, unit);
     const float h = hi_part(r);
     w[kXh + 2 * c] = h;
     w[kXl + 2 * c] = lo_part(r, h);
@@ -334,7 +342,7 @@ __global__ void __launch_bounds__(VerletShape<PREC>::kBlock) verlet_kernel(const
   }
   grid_dependency_wait();  // the force partials of this step are complete
 
-  const double an = sum_rows<PREC>(a.partial, N, p0, rows, comp, k);  // phase A
+  const double an = sum_rows<PREC>(a.partial, N, p0, rows, comp, k, a.unit);  // phase A
   if (!own) {
     if (!a.release_early) grid_dependency_launch();
     return;
@@ -344,7 +352,7 @@ __global__ void __launch_bounds__(VerletShape<PREC>::kBlock) verlet_kernel(const
   if (step) {
     double vn = v, nr;
     const double x = step_component(leap, r, vn, ao, an, a.dt, a.half_dt, a.half_dt2, &nr);
-    stage_component<PREC>(a.nxt, q, o, comp, nr, mu, muf);
+    stage_component<PREC>(a.nxt, q, o, comp, nr, mu, muf, a.unit);
     if (PREC == 1) Rc[q] = nr;
     Xc[q] = x;
     Vc[q] = vn;
@@ -423,7 +431,7 @@ __global__ void __launch_bounds__(VerletShape<PREC>::kBlock) rk_stage_kernel(con
     }
   }
   grid_dependency_wait();  // the force partials of this stage are complete
-  const double as = sum_rows<PREC>(a.partial, N, p0, rows, c, k);
+  const double as = sum_rows<PREC>(a.partial, N, p0, rows, c, k, a.unit);
   if (!own) {
     if (!a.release_early) grid_dependency_launch();
     return;
@@ -449,7 +457,7 @@ __global__ void __launch_bounds__(VerletShape<PREC>::kBlock) rk_stage_kernel(con
     a.V[i] = vn + cc * as;
   }
   if (!isfinite(as)) atomicOr(a.flags, kFlagNonFinite);
-  stage_component<PREC>(a.nxt, q, o, c, rnext, mu, muf);
+  stage_component<PREC>(a.nxt, q, o, c, rnext, mu, muf, a.unit);
   if (!a.release_early) grid_dependency_launch();
 }
 
@@ -489,7 +497,7 @@ __global__ void rk_prep_kernel(const RkArgs a) {
   }
   const double mu = a.G * a.m[q];
   const size_t o = PREC == 0 ? 0 : pair_off(a.qidx[q]);
-  stage_position<PREC>(a.nxt, q, o, r2[0], r2[1], r2[2], mu, static_cast<float>(mu));
+  stage_position<PREC>(a.nxt, q, o, r2[0], r2[1], r2[2], mu, static_cast<float>(mu), a.unit);
 }
 
 cudaError_t launch_rk_prep(int precision, const RkArgs &a, cudaStream_t s) {
@@ -506,8 +514,9 @@ cudaError_t launch_rk_prep(int precision, const RkArgs &a, cudaStream_t s) {
 // Stage the sources of the next force launch: r (drift == 0) or the Eq. 3
 // drift of (r, v, a) (drift == 1), with mu = G m.
 //   FP64: double4 (x, y, z, mu) at index p.
-//   Mixed: FP64 positions R[p], and hi = fl32(r), lo = fl32(r - hi), mu into
-//   the pair block of stage entry q = qidx[p] (layout in step_kernel.cuh).
+//   Mixed: FP64 positions R[p], and hi = fl32(r'), lo = fl32(r' - hi) with
+//   r' = 2^a.unit r, mu into the pair block of stage entry q = qidx[p] (layout
+//   in step_kernel.cuh).
 // ---------------------------------------------------------------------------
 template <int PREC>
 __global__ void prep_kernel(const PrepArgs a) {
@@ -538,6 +547,9 @@ __global__ void prep_kernel(const PrepArgs a) {
     a.Rz[p] = rz;
     const int q = a.qidx[p];
     float *w = static_cast<float *>(a.stage) + pair_off(q);
+    rx = times_pow2(rx, a.unit);
+    ry = times_pow2(ry, a.unit);
+    rz = times_pow2(rz, a.unit);
     const float hx = hi_part(rx), hy = hi_part(ry), hz = hi_part(rz);
     w[kXh] = hx;
     w[kYh] = hy;

@@ -291,6 +291,14 @@ __device__ __forceinline__ double drift(double r, double v, double a, double dt,
   return fma(half_dt2, a, fma(v, dt, r));
 }
 
+// 2^k x, |k| <= 200, without the FP64 pipe.  What lies beyond 2^+-767 stays as
+// it is: zero or infinite in FP32 either way.
+__device__ __forceinline__ double times_pow2(double x, int32_t k) {
+  const int32_t h = __double2hiint(x);
+  const uint32_t e = (static_cast<uint32_t>(h) >> 20) & 0x7ffu;
+  return __hiloint2double(e - 256u <= 1534u ? h + k * (1 << 20) : h, __double2loint(x));
+}
+
 __device__ __forceinline__ float hi_part(double x) { return __double2float_rn(x); }
 __device__ __forceinline__ float lo_part(double x, float hi) {
   return __double2float_rn(x - static_cast<double>(hi));

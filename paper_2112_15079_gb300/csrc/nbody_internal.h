@@ -67,6 +67,7 @@ struct VerletArgs {
   int32_t p_begin, p_end;  // the bodies this launch completes: [p_begin, p_end) (all: 0, N)
   int32_t mode;
   int32_t release_early;  // 1: the next kernel may launch at once
+  int32_t unit;           // mixed: staged coordinates and partial sums are 2^unit times the caller's
   double dt, half_dt, half_dt2;
 };
 
@@ -98,6 +99,7 @@ struct AdjArgs {
   unsigned *flags;
   int32_t N;
   int32_t mode;  // 0: step, stage alpha'+dt/2 nu'; 1: step, stage alpha'; 2: last product only
+  int32_t unit;  // mixed: as VerletArgs::unit (the products' mass sums are 2^(-2 unit) times the caller's)
   double G, dt, half_dt, half_dt2;
 };
 
@@ -129,6 +131,7 @@ struct PrepArgs {
   int32_t N;
   int32_t drift;  // 0: stage r; 1: stage the Eq. 3 drift of r; 2: stage r + dt/2 v (leapfrog)
   int32_t check;  // validate inputs (finite state, m >= 0)
+  int32_t unit;   // mixed: as VerletArgs::unit (G then carries 2^(3 unit))
   double G, dt, half_dt2;
 };
 
@@ -211,6 +214,7 @@ struct CloseArgs {
   int32_t n_mem;
   int32_t complete;                  // 1: first finish the step the Verlet kernel closed
   int32_t precision;
+  int32_t unit;                      // mixed: as VerletArgs::unit
   double G, dt, half_dt;
 };
 
@@ -267,6 +271,7 @@ struct RkArgs {
   int32_t N;
   int32_t stage;
   int32_t release_early;
+  int32_t unit;  // mixed: as VerletArgs::unit
   double G, dt;
 };
 cudaError_t launch_rk_stage(int precision, const RkArgs &a, cudaStream_t s, bool chained);

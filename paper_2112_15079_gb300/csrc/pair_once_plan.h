@@ -75,6 +75,28 @@ inline int64_t pair_once_items(const std::vector<int64_t> &sizes, int64_t B) {
   return pairs;
 }
 
+// Unit of the mixed pair-once stage.  These kernels share |d|^-3 between a
+// pair's two terms and multiply by mu afterwards; in FP32 |d|^-3 alone loses
+// bits from |d| = 2^42 on and overflows below 2^-43, where the every-ordered-pair
+// kernel's (mu |d|^-1)(|d|^-2) does neither.  (That form here would cost an
+// operation of 16 and 3 % of the time: 65,536 bodies 1.504 -> 1.556 ms per
+// step, 10,425 bodies 62.0 -> 63.6 us.)  So the stage has a unit of length of its
+// own: positions 2^k r, mu 2^3k G m, accelerations 2^k a, the same bits as
+// without where FP32's range holds both.  lo, hi: the smallest and the largest,
+// over the systems, of the exponent of a system's largest |coordinate|.  k = 0
+// while these leave room on both sides (astronomical units: 5); else the
+// largest becomes 2^20, 2^62 above the closest pair that FP32 then takes and 2^21
+// below the farthest.  Systems whose sizes lie further apart than 2^20 cannot
+// share a unit and keep the ordered-pair kernel (unless a block size was asked
+// for).
+constexpr int kUnitLow = -4, kUnitHigh = 24, kUnitTo = 20, kUnitSpread = 20;
+
+inline bool stage_unit_fits(int lo, int hi) { return hi - lo <= kUnitSpread; }
+inline int stage_unit_exp(int lo, int hi) {
+  if (lo >= kUnitLow && hi <= kUnitHigh) return 0;
+  return std::min(100, std::max(-100, kUnitTo - hi));
+}
+
 // sizes: bodies per system; nsm: the GPU's SMs; requested: the caller's
 // block size (0 = automatic).  Returns the block size, or 0 for the
 // every-ordered-pair kernel.

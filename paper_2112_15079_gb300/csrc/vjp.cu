@@ -352,6 +352,9 @@ __global__ void __launch_bounds__(AdjShape<PREC>::kThreads) adjoint_kernel(const
       fe += o.y;
     }
     sum = static_cast<double>(fs) + static_cast<double>(fe);
+    // staged positions are 2^unit r: K goes as mu |d|^-3 with mu 2^(3 unit) its
+    // own, the mass sum as |d|^-2
+    if (c == 3) sum = times_pow2(sum, 2 * a.unit);
   }
   if (!live) return;
   if (!isfinite(sum)) atomicOr(a.flags, kFlagNonFinite);

@@ -373,3 +373,48 @@ def test_pairs_left_to_fp64_differences(nb, block, kind):
     # (the sums of a random cluster cancel: relative to the terms' magnitudes)
     err = np.linalg.norm(a - oracle.accel(1.0, r, m, openmp=True), axis=0) / oracle.term_norm(1.0, r, m, openmp=True)
     assert err.max() <= 1e-13
+
+
+@pytest.mark.parametrize("n,kw", [(2049, {}), (2049, {"integrator": "leapfrog"}), (2049, {"integrator": "rk4"}),
+                                  (2049, {"close_omega_dt": 0.5}), (5003, {"pair_once_block": 512}),
+                                  (5003, {"pair_once_block": 2048})])
+def test_mixed_units_are_the_callers(nb, n, kw):
+    """The same model in other length units (positions and velocities times
+    2^j, G times 2^3j: kilometres to micrometres and kiloparsecs beyond if
+    the first were astronomical units): every figure of a mixed run, and of
+    its gradient, is a power of two times the first one's, to the bit."""
+    s = inputs.solar_system(n, seed=81, moon_omega_dt_max=None if "close_omega_dt" in kw else 0.5)
+    rng = np.random.default_rng(n)
+    gr = rng.normal(size=(3, n))
+    runs = {}
+    for j in (0, -50, -31, 24, 37, 44, 57):
+        u = 2.0**j
+        b = nb.NBody(s.r * u, s.v * u, s.m, G=s.G * u**3, dt=s.dt, precision="mixed", ckpt_every=2, **kw)
+        assert b.pair_once_block == kw.get("pair_once_block", 128)
+        g = () if set(kw) - {"pair_once_block"} else b.grad(3, gr)
+        b.step(4)
+        out = [t.cpu().numpy() / u for t in (b.accel(), b.r, b.v)]
+        out += [t.cpu().numpy() / f for t, f in zip(g, (1.0, 1.0, u))]
+        b.close()
+        runs[j] = out
+    assert np.all(np.isfinite(runs[0][0])) and np.abs(runs[0][0]).min() > 0.0
+    for j, out in runs.items():
+        for x, y in zip(out, runs[0]):
+            assert np.array_equal(x, y), (j, np.abs(x - y).max())
+
+
+def test_mixed_systems_of_unlike_sizes(nb):
+    """Two systems whose lengths differ by 2^25 share no unit in FP32: they keep
+    the ordered-pair kernel, and the mixed gate holds in both."""
+    parts = [inputs.solar_system(2049, seed=k) for k in (82, 83)]
+    scale = (1.0, 2.0**-25)
+    r = np.concatenate([p.r * u for p, u in zip(parts, scale)], 1)
+    v = np.concatenate([p.v * u for p, u in zip(parts, scale)], 1)
+    m = np.concatenate([p.m * u for p, u in zip(parts, scale)])
+    off = np.array([0, 2049, 4098])
+    a, used = _mixed_accel(nb, r, v, m, off)
+    assert used == 0
+    for b, e in zip(off[:-1], off[1:]):
+        x, w = np.ascontiguousarray(r[:, b:e]), m[b:e]
+        err = np.linalg.norm(a[:, b:e] - oracle.accel(inputs.G_AU_DAY, x, w, openmp=True), axis=0)
+        assert np.all(err <= 2e-6 * oracle.term_norm(inputs.G_AU_DAY, x, w))
