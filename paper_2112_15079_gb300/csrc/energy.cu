@@ -98,10 +98,10 @@ __global__ void __launch_bounds__(32 * kWarps) energy_kernel(const EnergyArgs a)
   DD pot = {0.0, 0.0}, kin = {0.0, 0.0};
   for (int r = w; r < T && i0 + 32 * r < ns; r += kWarps) {
     const int il = i0 + 32 * r + lane;
-    const double4_32a p = energy_load(a, b, il, ns, 1e15 * (lane + 1));
+    const double4_32a p = energy_load(a, b, il, ns, kInertPlace * (lane + 1));
     const double mp = il < ns ? a.m[b + il] : 0.0;
     for (int q = diag ? r : 0; q < T && j0 + 32 * q < ns; ++q) {
-      const double4_32a j = energy_load(a, b, j0 + 32 * q + lane, ns, 1e15 * (lane + 1) + 5e14);
+      const double4_32a j = energy_load(a, b, j0 + 32 * q + lane, ns, kInertPlace * (lane + 1) + 0.5 * kInertPlace);
       const double t = diag && q == r ? tile_potential<true>(p, j, lane) : tile_potential<false>(p, j, lane);
       two_sum_acc(pot.hi, pot.lo, -mp * t);
     }

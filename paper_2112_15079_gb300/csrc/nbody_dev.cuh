@@ -216,6 +216,13 @@ __device__ __forceinline__ VjpFactors vjp_factors(double dx, double dy, double d
   return f;
 }
 
+// Where the bodies that stand in for lanes outside a system sit: at
+// (kInertPlace (lane + 1), 0, 0) as targets, half of it farther as sources.
+// They are massless, so their terms are zero as long as they coincide with no
+// body, hence a place (about 2^180, every mantissa bit in use) that no model's
+// unit of length reaches, within the range of the integer path.
+constexpr double kInertPlace = 0x1.3c0ca428c59fbp+180;
+
 // Mixed: positions split as x = hi + lo (hi = fl32(x), lo = fl32(x - hi)).
 // d = (hi_j - hi_p) + (lo_j - lo_p): the hi difference is exact whenever the
 // two coordinates are within a factor 2 (Sterbenz), so close pairs keep the

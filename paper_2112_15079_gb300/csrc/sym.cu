@@ -35,7 +35,7 @@ namespace {
 
 __device__ __forceinline__ double4_32a sym_load(const double4_32a *cur, int64_t sb, int il, int ns, double pad) {
   if (il < ns) return cur[sb + il];
-  // outside the system: inert (massless, far away, distinct per lane)
+  // outside the system: inert (massless, far away, distinct per lane: kInertPlace)
   return make_double4_32a(pad, 0.0, 0.0, 0.0);
 }
 
@@ -218,12 +218,13 @@ __global__ void __launch_bounds__(kSymThreads) force_sym_kernel(const SymArgs a)
     const int4 pr = a.pairs[item];  // (first body of the system, its bodies, block I, block J)
     const int64_t sb = pr.x;
     const int ns = pr.y, I = pr.z, J = pr.w;
-    const double4_32a pi = sym_load(a.cur, sb, I * kSymBlock + w * 32 + lane, ns, 1e15 * (lane + 1));
+    const double4_32a pi = sym_load(a.cur, sb, I * kSymBlock + w * 32 + lane, ns, kInertPlace * (lane + 1));
     double ax = 0.0, ay = 0.0, az = 0.0;
     for (int t = 0; t < 2; ++t) {
       double bx = 0.0, by = 0.0, bz = 0.0;
       if (!(I == J && t < w)) {  // tile pair (w, t) with t < w of a diagonal item is (t, w), warp t's
-        const double4_32a pj0 = sym_load(a.cur, sb, J * kSymBlock + t * 32 + lane, ns, 1e15 * (lane + 1) + 5e14);
+        const double4_32a pj0 = sym_load(a.cur, sb, J * kSymBlock + t * 32 + lane, ns,
+                                         kInertPlace * (lane + 1) + 0.5 * kInertPlace);
         const bool ri = I * kSymBlock + w * 32 + lane < ns, rj = J * kSymBlock + t * 32 + lane < ns;
         if (I == J && t == w)
           sym_tile<true>(pi, pj0, ri, rj, lane, ax, ay, az, bx, by, bz);
@@ -312,15 +313,16 @@ __global__ void __launch_bounds__(2 * kSymWideThreads, 2) force_sym_wide_kernel(
     for (int r = 0; r < T; r += W) {
       const int p = r + w;
       const bool p_live = i0 + p * 32 < ns;  // warp-uniform
-      const double4_32a pi = sym_load(a.cur, sb, i0 + p * 32 + lane, ns, 1e15 * (lane + 1));
+      const double4_32a pi = sym_load(a.cur, sb, i0 + p * 32 + lane, ns, kInertPlace * (lane + 1));
       double ax = 0.0, ay = 0.0, az = 0.0;
       // the next phase's J tile, loaded a phase ahead
       int q = p;
-      double4_32a pn = sym_load(a.cur, sb, j0 + q * 32 + lane, ns, 1e15 * (lane + 1) + 5e14);
+      double4_32a pn = sym_load(a.cur, sb, j0 + q * 32 + lane, ns, kInertPlace * (lane + 1) + 0.5 * kInertPlace);
       for (int t = 0; t < T; ++t) {
         const double4_32a pj0 = pn;
         const int qn = (p + t + 1) & (T - 1);
-        if (t + 1 < T) pn = sym_load(a.cur, sb, j0 + qn * 32 + lane, ns, 1e15 * (lane + 1) + 5e14);
+        if (t + 1 < T) pn = sym_load(a.cur, sb, j0 + qn * 32 + lane, ns,
+                                     kInertPlace * (lane + 1) + 0.5 * kInertPlace);
         if (p_live && j0 + q * 32 < ns && !(diag && q < p)) {  // (q < p on a diagonal item: tile q's warp's pair)
           double tx = 0.0, ty = 0.0, tz = 0.0, bx, by, bz;
           const bool ri = i0 + p * 32 + lane < ns, rj = j0 + q * 32 + lane < ns;
@@ -402,7 +404,7 @@ __global__ void __launch_bounds__(kSymThreads) vjp_sym_kernel(const VjpSymArgs a
     const int64_t sb = pr.x;
     const int ns = pr.y, I = pr.z, J = pr.w;
     const int iq = I * kSymBlock + w * 32 + lane;
-    const double4_32a pq = sym_load(a.pos, sb, iq, ns, 1e15 * (lane + 1));
+    const double4_32a pq = sym_load(a.pos, sb, iq, ns, kInertPlace * (lane + 1));
     const double4_32a wq = iq < ns ? a.w[sb + iq] : make_double4_32a(0.0, 0.0, 0.0, 0.0);
     const ic::Mass mq = ic::pack_mass(pq.w);
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
@@ -410,7 +412,7 @@ __global__ void __launch_bounds__(kSymThreads) vjp_sym_kernel(const VjpSymArgs a
       double b[4] = {0.0, 0.0, 0.0, 0.0};
       if (!(I == J && t < w)) {  // tile pair (w, t) with t < w of a diagonal item is (t, w), warp t's
         const int ij = J * kSymBlock + t * 32 + lane;
-        const double4_32a pj0 = sym_load(a.pos, sb, ij, ns, 1e15 * (lane + 1) + 5e14);
+        const double4_32a pj0 = sym_load(a.pos, sb, ij, ns, kInertPlace * (lane + 1) + 0.5 * kInertPlace);
         const double4_32a wj0 = ij < ns ? a.w[sb + ij] : make_double4_32a(0.0, 0.0, 0.0, 0.0);
         double xj = pj0.x, yj = pj0.y, zj = pj0.z, wjx = wj0.x, wjy = wj0.y, wjz = wj0.z;
         ic::Mass mj = ic::pack_mass(pj0.w);

@@ -418,3 +418,23 @@ def test_mixed_systems_of_unlike_sizes(nb):
         x, w = np.ascontiguousarray(r[:, b:e]), m[b:e]
         err = np.linalg.norm(a[:, b:e] - oracle.accel(inputs.G_AU_DAY, x, w, openmp=True), axis=0)
         assert np.all(err <= 2e-6 * oracle.term_norm(inputs.G_AU_DAY, x, w))
+
+
+@pytest.mark.parametrize("x", [1e15, 1.5e15, 7e15, 2.55e16])
+def test_no_round_coordinate_is_taken_by_a_stand_in(nb, x):
+    """Lanes past the end of a system hold massless stand-ins; a body may sit at
+    any round coordinate (1e15 metres from the origin, say) without meeting one:
+    energy (ragged tiles of 32) and the pair-once force (a last tile without a
+    body), in the tolerances of those tests."""
+    for n in (1, 33, 1283):
+        s = inputs.solar_system(max(n, 31), seed=84)
+        r, v, m = s.r[:, :n].copy(), s.v[:, :n].copy(), s.m[:n].copy()
+        r[:, 0] = [x, 0.0, 0.0]
+        b = nb.NBody(r, v, m, G=s.G, dt=s.dt, precision="fp64", small=False, pair_once_block=64)
+        e, a = b.energy()[0], b.accel().cpu().numpy()
+        b.close()
+        kin, pot = oracle.energy(s.G, r, v, m)
+        assert abs(e - (kin + pot)) <= 1e-13 * (abs(kin) + abs(pot))
+        if n > 1:
+            err = np.linalg.norm(a - oracle.accel(s.G, r, m), axis=0)
+            assert np.all(err <= 1e-13 * oracle.term_norm(s.G, r, m))
