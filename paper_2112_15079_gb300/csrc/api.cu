@@ -101,6 +101,7 @@ struct nbody_ctx {
   int alloc_seq = 0;  // device allocations made so far (fault injection counts these)
   int64_t wait_seq = 0;      // launches with a stallable bounded wait (adjoint products, single-launch steps)
   int64_t stall_at = 0;      // test hook (NBODY_INJECT_WAIT_STALL=k): the k-th of them stalls
+  int64_t force_seq = 0, force_stall_at = 0;  // the same of mixed pair-once force launches (NBODY_INJECT_FORCE_STALL)
   double *a = nullptr;               // [3][N] acceleration at the current positions
   void *stage[2] = {nullptr, nullptr};  // ping-pong staged sources (layout per precision)
   int64_t n_stage = 0;               // stage entries (mixed: systems padded to even length)
@@ -744,6 +745,7 @@ nbody_status launch_force_kernel(nbody_ctx *c, const void *cur, cudaStream_t st,
       m.N = static_cast<int32_t>(c->N);
       m.tiles = c->fw.sym_tiles;
       m.warps = c->fw.sym_tiles / 4;
+      if (m.tiles > nb::kMsymMinTiles) m.stall = ++c->force_seq == c->force_stall_at ? 1 << 20 : 0;
       NB_CUDA(c, nb::launch_force_msym(m, c->fw.grid, st, chained));
       return NBODY_OK;
     }
@@ -1317,9 +1319,13 @@ nbody_status nbody_init(nbody_ctx **out, int64_t n_systems, const int64_t *offse
   // bounded wait in the context's k-th launch that has one: the first source
   // tile of CTA 0 stays unissued in an adjoint product (VJP launch), or CTA 0
   // leaves out one barrier arrival in a single-launch step call.  The wait
-  // runs out and nbody_grad / nbody_sync report ETIMEOUT.  (The force kernels
-  // carry no test code.)
+  // runs out and nbody_grad / nbody_sync report ETIMEOUT.
+  // NBODY_INJECT_FORCE_STALL=k does so in the context's k-th force launch on
+  // mixed blocks of 256 entries and more (the first is nbody_init's own): the
+  // warps wait for progress that their neighbours never make.  (The other
+  // force kernels carry no test code.)
   if (const char *inj = std::getenv("NBODY_INJECT_WAIT_STALL")) c->stall_at = std::atoll(inj);
+  if (const char *inj = std::getenv("NBODY_INJECT_FORCE_STALL")) c->force_stall_at = std::atoll(inj);
 
   auto bail = [&](nbody_status st) {
     g_init_error = c->err;

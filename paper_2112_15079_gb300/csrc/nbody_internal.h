@@ -162,6 +162,7 @@ struct MsymArgs {
   int32_t N;
   int32_t tiles;           // T: 32-entry tiles per block, kMsymMinTiles .. kMsymMaxTiles (a power of two)
   int32_t warps;           // W = T / 4 warps per CTA
+  int32_t stall;           // test hook (blocks of 256 entries and more): phases that a neighbour is never seen to take
 };
 
 // The adjoint's VJP with each pair once (FP64, sym.cu): the same items,

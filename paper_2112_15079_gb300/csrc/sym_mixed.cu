@@ -50,7 +50,10 @@ namespace nb {
 namespace {
 
 // Polls of a neighbour's progress in shared memory before it is given up
-// (tens of milliseconds; a phase takes tens of microseconds).
+// (tens of milliseconds; a phase takes tens of microseconds).  The warp then
+// says so to the CTA, sets kFlagTimeout and takes no further phase, nor does a
+// warp that would wait for it, and the CTA takes no further item (the host
+// reports the timeout: the rows it wrote and left out are not used).
 constexpr int kMsymPolls = 1 << 21;
 
 // Per-warp shared scratch: two chunk buffers, the targets' negated lo parts
@@ -227,6 +230,7 @@ __global__ void __launch_bounds__(32 * kMsymMaxWarps, 1) force_msym_kernel(const
   extern __shared__ __align__(16) unsigned char msym_smem[];
   __shared__ int s_item;
   __shared__ volatile int s_done[kMsymMaxWarps];  // phases each warp has finished
+  __shared__ volatile int s_lost;                 // a wait ran out
   grid_dependency_wait();    // staged sources and boxes of this step are complete
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   const int W = a.warps, T = a.tiles, BT = 32 * T, NC = T / 2;
@@ -237,13 +241,14 @@ __global__ void __launch_bounds__(32 * kMsymMaxWarps, 1) force_msym_kernel(const
   f2 (*wmu)[32] = reinterpret_cast<f2 (*)[32]>(s_j + 6 * BT) + 4 * w;
   const size_t N = static_cast<size_t>(a.N);
   const float *cur = a.cur;
+  if (tid == 0) s_lost = 0;
   for (;;) {
     __syncthreads();  // the previous item's shared sums are consumed
     if (tid == 0) s_item = atomicAdd(a.ctr, 1);
     if (lane == 0) s_done[w] = 0;
     for (int k = tid; k < 6 * BT; k += 32 * W) s_j[k] = 0.f;
     __syncthreads();
-    const int item = s_item;
+    const int item = s_lost ? a.n_pairs : s_item;
     if (item >= a.n_pairs) {
       grid_dependency_launch();  // the Verlet kernel may launch as the CTAs run out of items
       break;
@@ -345,10 +350,15 @@ __global__ void __launch_bounds__(32 * kMsymMaxWarps, 1) force_msym_kernel(const
           __threadfence_block();
           if (lane == 0) s_done[w] = t + 1;
           const int next = w + 1 < W ? w + 1 : 0;
-          int polls = 0;
-          while (s_done[next] < t && polls < kMsymPolls) ++polls;
-          if (polls == kMsymPolls && lane == 0) atomicOr(a.flags, kFlagTimeout);
-          __syncwarp();
+          int polls = kMsymPolls;
+          while (s_done[next] < t + a.stall && polls > 0) polls = s_lost ? 0 : polls - 1;
+          if (__any_sync(0xffffffffu, polls == 0)) {
+            if (lane == 0) {
+              s_lost = 1;
+              atomicOr(a.flags, kFlagTimeout);
+            }
+            break;
+          }
           __threadfence_block();
         }
       }
@@ -384,6 +394,7 @@ __global__ void __launch_bounds__(32 * kMsymMaxWarps, 1) force_msym_kernel(const
       row[2 * N + b] = make_float2(s_j[4 * BT + k], s_j[5 * BT + k]);
     }
   }
+  cp_async_wait_all();  // (a chunk is on its way if a wait ran out)
   // The last CTA out resets the item counter for the next launch.
   if (tid == 0) {
     __threadfence();

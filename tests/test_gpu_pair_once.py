@@ -438,3 +438,35 @@ def test_no_round_coordinate_is_taken_by_a_stand_in(nb, x):
         if n > 1:
             err = np.linalg.norm(a - oracle.accel(s.G, r, m), axis=0)
             assert np.all(err <= 1e-13 * oracle.term_norm(s.G, r, m))
+
+
+@pytest.mark.parametrize("block", [256, 512, 2048])
+def test_mixed_neighbour_wait_timeout_reports_and_recovers(nb, block, monkeypatch):
+    """NBODY_INJECT_FORCE_STALL=2 makes a warp of CTA 0 hide its progress in the
+    second force launch (the first is nbody_init's): its neighbour's bounded
+    wait runs out, the CTA's other warps stop at their own next wait, the
+    kernel ends, and nbody_sync reports ETIMEOUT.  After the state is restored
+    and reset, the context steps bitwise like a fresh one."""
+    import time
+    torch = pytest.importorskip("torch")
+    s = inputs.solar_system(5003, seed=53, moon_omega_dt_max=0.5)
+    kw = dict(G=s.G, dt=s.dt, precision="mixed", pair_once_block=block, graphs=False)
+    fresh = nb.NBody(s.r, s.v, s.m, **kw)
+    fresh.step(5)
+    want = fresh.state.cpu().numpy()
+    fresh.close()
+    monkeypatch.setenv("NBODY_INJECT_FORCE_STALL", "2")
+    b = nb.NBody(s.r, s.v, s.m, **kw)
+    monkeypatch.delenv("NBODY_INJECT_FORCE_STALL")
+    t0 = time.time()
+    b.step(3)
+    with pytest.raises(nb.NBodyError) as ei:
+        b.sync()
+    assert ei.value.status == nb.NBODY_ETIMEOUT
+    assert time.time() - t0 < 30
+    b.state[0:3].copy_(torch.tensor(s.r))
+    b.state[3:6].copy_(torch.tensor(s.v))
+    b.reset()
+    b.step(5)
+    assert np.array_equal(b.state.cpu().numpy(), want)
+    b.close()
