@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(kFarThreads) close_far_kernel(const CloseArgs 
     for (int u = 0; u < ne; ++u) partner |= s_part[u] == j;
     if (partner) continue;
     const double dx = a.x[j] - px, dy = a.y[j] - py, dz = a.z[j] - pz;
-    const double f = source_factor<false>(dx, dy, dz, ic::pack_mass(a.G * a.m[j]), false);
+    const double f = source_factor(dx, dy, dz, ic::pack_mass(a.G * a.m[j]));
     sx = fma(f, dx, sx);
     sy = fma(f, dy, sy);
     sz = fma(f, dz, sz);

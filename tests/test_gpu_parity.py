@@ -250,6 +250,24 @@ def test_a_body_among_massless_ones_feels_nothing(nb, n):
     b.close()
 
 
+@pytest.mark.parametrize("n", [1, 2, 33, 131, 521])
+def test_the_targets_own_pair_in_the_ordered_kernel(nb, n):
+    """The FP64 ordered-pair kernel takes a target's own entry as a massless
+    source a unit away: exactly nothing is added, also where the target is the
+    only massive body, and its neighbours' sums keep the FP64 gate."""
+    s = inputs.solar_system(max(n, 31), seed=76, n_moons=0)
+    r, v = s.r[:, :n].copy(), s.v[:, :n].copy()
+    for m in (np.where(np.arange(n) == 0, 1.0, 0.0), s.m[:n].copy()):
+        b = nb.NBody(r, v, m, G=s.G, dt=s.dt, precision="fp64", small=False, pair_once=False)
+        a = b.accel().cpu().numpy()
+        b.close()
+        if n == 1 or m[1] == 0.0:
+            assert np.array_equal(a[:, 0], np.zeros(3))
+        if n > 1:
+            ref = oracle.accel(s.G, r, m)
+            assert np.max(_rel_err(a[:, 1:], ref[:, 1:])) <= FP64_TOL
+
+
 def test_grid_kernel_wait_timeout_reports_and_recovers(nb, monkeypatch):
     """NBODY_INJECT_WAIT_STALL=1 makes CTA 0 of the cooperative grid kernel
     (257 bodies) skip its first barrier arrival: every CTA's bounded wait
