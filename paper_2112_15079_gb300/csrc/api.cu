@@ -665,10 +665,13 @@ nb::ForceArgs force_args(nbody_ctx *c, const void *cur) {
 // come early, and does where that measured faster on GB300: pair-once items
 // are handed out dynamically (2,131 bodies 12.8 -> 11.8 us per step), and up
 // to 2,048 bodies the launches dominate (1,500: 15.7 -> 15.2); with larger
-// static shares it costs a little (6,001: 31.3 -> 31.8).
+// static shares it costs a little (6,001: 31.3 -> 31.8).  With close-encounter
+// handling the next kernel is the members' far force instead, whose CTAs, let
+// in early, took the SMs from the per-body kernel's: 10,425 bodies 130.4 us per
+// step, 98.5 released at the end (smaller systems the same either way).
 int release_early(const nbody_ctx *c) {
   const bool mixed = c->o.precision == NBODY_MIXED;
-  return c->fw.occ == 1 || (mixed && (c->fw.sym_pairs || c->N <= 2048)) ? 1 : 0;
+  return c->fw.occ == 1 || (mixed && !c->close_on && (c->fw.sym_pairs || c->N <= 2048)) ? 1 : 0;
 }
 
 nb::VerletArgs verlet_args(nbody_ctx *c, const State &s, const void *cur, void *nxt, int mode) {
