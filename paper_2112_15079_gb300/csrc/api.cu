@@ -66,6 +66,7 @@ struct Adjoint {
   int64_t n_ckpt = 0;
   void *store = nullptr;           // [K + 1] staged positions of one segment
   int64_t store_len = 0;
+  bool once = false;               // whether vj was to evaluate each pair once
 };
 
 }  // namespace
@@ -150,6 +151,7 @@ struct nbody_ctx {
   Work fw;
   Adjoint adj;
 
+  bool sym_off = false;  // the rows of the pair-once kernels found no memory
   bool small = false;  // the single-launch cluster kernel serves nbody_step
   bool grid = false;   // the single-launch cooperative grid kernel serves nbody_step
   int grid_warps = 0, grid_parts = 1, grid_ctas = 0;
@@ -362,10 +364,10 @@ nbody_status build_work(nbody_ctx *c, Work &wk, const nbody_tiles &t, int occ, i
 
 // Block size of the pair-once force kernels for this context
 // (pair_once_plan.h), or 0 where the every-ordered-pair kernel runs: row
-// shards, NBODY_FLAG_NO_SYM, mixed systems whose positions share no unit, and
-// the cases pair_once_block turns down.
+// shards, NBODY_FLAG_NO_SYM, mixed systems whose positions share no unit or
+// whose rows found no memory, and the cases pair_once_block turns down.
 int sym_block(const nbody_ctx *c) {
-  if (c->sh_world > 0 || (c->o.flags & NBODY_FLAG_NO_SYM)) return 0;
+  if (c->sh_world > 0 || (c->o.flags & NBODY_FLAG_NO_SYM) || c->sym_off) return 0;
   std::vector<int64_t> sizes(static_cast<size_t>(c->n_sys));
   for (int64_t s = 0; s < c->n_sys; ++s) sizes[s] = c->offsets[s + 1] - c->offsets[s];
   const bool mixed = c->o.precision == NBODY_MIXED;
@@ -453,19 +455,32 @@ void free_work(nbody_ctx *c, Work &w) {
   w = Work{};
 }
 
+// Whether the context may run the ordered-pair kernels where the rows of the
+// pair-once ones cannot be allocated: an automatic mixed choice.
+bool may_drop_pair_once(const nbody_ctx *c) {
+  return c->o.precision == NBODY_MIXED && c->o.pair_once_block == 0;
+}
+
 // Build the force kernel's tables for tiles t and make t current.  The new
 // tables are built aside: on failure the context keeps its previous tiles
 // and tables, which stay a matching pair.
 nbody_status build_items(nbody_ctx *c, const nbody_tiles &t) {
   drop_graphs(c);
   if (const int B = sym_block(c)) {  // the tiles stay the context's, for nbody_get_tiles; this kernel has none
-    Work nw;
-    const nbody_status st = build_sym_work(c, nw, 3, B);
-    if (st != NBODY_OK) return st;
-    free_work(c, c->fw);
-    c->fw = nw;
-    c->tiles = t;
-    return NBODY_OK;
+    nbody_status st = NBODY_OK;
+    if (!(c->fw.sym_pairs && 32 * c->fw.sym_tiles == B)) {  // (its tables depend on the systems' sizes alone)
+      Work nw;
+      if ((st = build_sym_work(c, nw, 3, B)) == NBODY_OK) {
+        free_work(c, c->fw);
+        c->fw = nw;
+      }
+    }
+    if (st == NBODY_OK) c->tiles = t;
+    // Rows of up to gigabytes that the caller did not ask for and that do not
+    // fit: the ordered-pair kernel, whose rows are a few per body.
+    if (!(st == NBODY_ENOMEM && may_drop_pair_once(c))) return st;
+    c->sym_off = true;
+    c->err.clear();
   }
   // The deepest ring (kMaxStages down to kStages tiles) at which the CTAs
   // per SM the tiles ask for still fit: a deeper ring lets the warps of a
@@ -1175,10 +1190,11 @@ nbody_status ensure_adjoint(nbody_ctx *c, int64_t n_steps) {
   // With the narrowest pair-once blocks (FP64 64 bodies, mixed 128 entries) the
   // VJP evaluates each pair once too.
   const int B = prec == NBODY_MIXED ? 32 * nb::kMsymMinTiles : nb::kSymBlock;
-  const bool once = c->fw.sym_pairs && 32 * c->fw.sym_tiles == B;
+  bool once = c->fw.sym_pairs && 32 * c->fw.sym_tiles == B;
   // First use, an earlier attempt that failed part way, or a reset that changed
   // the force kernel: start clean.
-  if (!A.shadow || once != (A.vj.sym_pairs != nullptr)) {
+  if (!A.shadow || once != A.once) {
+    A.once = once;
     free_work(c, A.vj);
     for (void *q : {static_cast<void *>(A.rho), static_cast<void *>(A.nu), static_cast<void *>(A.gm), A.w,
                     static_cast<void *>(A.shadow)})
@@ -1191,9 +1207,12 @@ nbody_status ensure_adjoint(nbody_ctx *c, int64_t n_steps) {
     t.tj = kVjpTile;
     t.jsplit = 0;
     t.ctas_per_sm = 32;
-    if (once) {
-      if ((st = build_sym_work(c, A.vj, 4, B)) != NBODY_OK) return st;
-    } else {
+    if (once && (st = build_sym_work(c, A.vj, 4, B)) != NBODY_OK) {
+      if (!(st == NBODY_ENOMEM && may_drop_pair_once(c))) return st;
+      once = false;  // (as build_items)
+      c->err.clear();
+    }
+    if (!once) {
       const size_t smem = nb::vjp_smem_bytes(prec, t.tj);
       int occ = 0;
       NB_CUDA(c, nb::vjp_prepare(prec, smem, &occ));

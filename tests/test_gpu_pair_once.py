@@ -470,3 +470,58 @@ def test_mixed_neighbour_wait_timeout_reports_and_recovers(nb, block, monkeypatc
     b.step(5)
     assert np.array_equal(b.state.cpu().numpy(), want)
     b.close()
+
+
+def test_mixed_rows_without_memory(nb, monkeypatch):
+    """An automatic pair-once choice whose tables or rows cannot be allocated
+    runs the ordered-pair kernel (bitwise the context without pair-once) rather
+    than refuse a context that fits; the product of a gradient likewise; a block
+    size that was asked for is refused."""
+    s = inputs.solar_system(2131, seed=55, moon_omega_dt_max=0.5)
+    kw = dict(G=s.G, dt=s.dt, precision="mixed")
+    rng = np.random.default_rng(1)
+    gr = rng.normal(size=(3, s.n))
+
+    def outputs(b):
+        g = [t.cpu().numpy() for t in b.grad(2, gr)]
+        b.step(4)
+        return [b.state.cpu().numpy()] + g
+
+    b = nb.NBody(s.r, s.v, s.m, pair_once=False, **kw)
+    want = outputs(b)
+    b.close()
+    k, fell_back = 0, 0
+    while True:  # every allocation of init in turn
+        k += 1
+        assert k < 64
+        monkeypatch.setenv("NBODY_INJECT_ALLOC_FAIL", str(k))
+        try:
+            b = nb.NBody(s.r, s.v, s.m, **kw)
+        except nb.NBodyError as e:
+            assert e.status == nb.NBODY_ENOMEM
+            continue
+        monkeypatch.delenv("NBODY_INJECT_ALLOC_FAIL")
+        if b.pair_once_block:
+            b.close()
+            break
+        fell_back += 1
+        for x, y in zip(outputs(b), want):
+            assert np.array_equal(x, y)
+        b.close()
+        monkeypatch.setenv("NBODY_INJECT_ALLOC_FAIL", str(k))
+        with pytest.raises(nb.NBodyError):
+            nb.NBody(s.r, s.v, s.m, pair_once_block=128, **kw)
+    assert fell_back == 4  # items, rows per body, counter, rows
+    n_init = k - 1
+    ref = oracle.grad(s.G, s.dt, 2, s.r, s.v, s.m, gr, np.zeros_like(gr), openmp=True, magnitudes=True)
+    for j in range(1, 5):  # the same four of the product
+        b = nb.NBody(s.r, s.v, s.m, **kw)
+        assert b.pair_once_block == 128
+        monkeypatch.setenv("NBODY_INJECT_ALLOC_FAIL", str(n_init + j))
+        got = [t.cpu().numpy() for t in b.grad(2, gr)]
+        monkeypatch.delenv("NBODY_INJECT_ALLOC_FAIL")
+        again = [t.cpu().numpy() for t in b.grad(2, gr)]
+        b.close()
+        for g, h, x, mag in zip(got, again, ref[:3], ref[3:]):
+            assert np.array_equal(g, h)
+            assert np.all(np.abs(g - x) <= 1e-3 * mag)
