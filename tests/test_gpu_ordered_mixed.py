@@ -1,0 +1,95 @@
+"""The mixed every-ordered-pair kernels at 2,131 bodies, where contexts run
+pair-once blocks by default: pair_once=False, each test asserting that it has
+reached them.  Tile decompositions (the mixed gate of the parity tests, every
+body), the shared-memory limit that contexts of unlike tiles share, and the
+autotuner."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2112_15079_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+MIXED_TOL = 2e-6
+N = 2131
+
+
+@pytest.fixture(scope="module")
+def nb():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2112_15079_gb300 import build
+    build.build()
+    from paper_2112_15079_gb300 import nbody
+    return nbody
+
+
+def _t(threads, ipt, tj, jsplit, cps):
+    return {"threads": threads, "ipt": ipt, "tj": tj, "jsplit": jsplit, "ctas_per_sm": cps}
+
+
+def _ordered(nb, s, tiles=None):
+    b = nb.NBody(s.r, s.v, s.m, G=s.G, dt=s.dt, precision="mixed", pair_once=False)
+    assert b.pair_once_block == 0
+    if tiles:
+        b.tiles = dict(b.tiles, **tiles)
+        b.reset()
+        assert b.pair_once_block == 0
+    return b
+
+
+def _gate(a, s):
+    ref, t = oracle.accel(s.G, s.r, s.m, openmp=True), oracle.term_norm(s.G, s.r, s.m, openmp=True)
+    d, n = np.linalg.norm(a - ref, axis=0), np.linalg.norm(ref, axis=0)
+    good = t / n <= 1e3
+    assert np.max(d / t) <= MIXED_TOL and np.max((d / n)[good]) <= MIXED_TOL
+
+
+@pytest.mark.parametrize("tiles", [None, _t(128, 1, 64, 0, 1), _t(256, 2, 128, 2, 2), _t(512, 1, 192, 8, 2),
+                                   _t(1024, 1, 2048, 1, 1), _t(512, 2, 512, 3, 1), _t(384, 2, 256, 0, 2),
+                                   _t(768, 2, 1024, 0, 1), _t(128, 4, 512, 0, 2), _t(256, 4, 64, 2, 1)])
+def test_tiles(nb, tiles):
+    s = inputs.solar_system(N, seed=N)
+    b = _ordered(nb, s, tiles)
+    _gate(b.accel().cpu().numpy(), s)
+    b.close()
+
+
+def test_contexts_of_unlike_tiles_share_the_kernel(nb):
+    """A context built later with smaller source tiles must not take away the
+    shared memory that an earlier one launches with."""
+    s = inputs.solar_system(N, seed=95)
+    big, small = _t(512, 1, 1024, 0, 2), _t(512, 1, 64, 0, 2)
+    want = {}
+    for name, t in (("big", big), ("small", small)):
+        r = _ordered(nb, s, t)
+        r.step(5)
+        want[name] = r.state.cpu().numpy()
+        r.close()
+    a, b = _ordered(nb, s, big), _ordered(nb, s, small)
+    a.step(5)
+    b.step(5)
+    assert np.array_equal(a.state.cpu().numpy(), want["big"])
+    assert np.array_equal(b.state.cpu().numpy(), want["small"])
+
+
+def test_autotune(nb):
+    """State restored, the winner current, steps bitwise a context's that was
+    given the winner's tiles."""
+    s = inputs.solar_system(N, seed=17)
+    b = _ordered(nb, s)
+    b.step(3)
+    before = b.state.cpu().numpy()
+    tiles, ms = b.autotune(probe_steps=2)
+    assert ms > 0 and b.tiles == tiles and b.pair_once_block == 0
+    assert np.array_equal(b.state.cpu().numpy(), before)
+    b.step(20)
+    c = _ordered(nb, s)
+    c.step(3)
+    c.tiles = tiles
+    c.step(20)
+    assert np.array_equal(c.state.cpu().numpy(), b.state.cpu().numpy())
+    d = _ordered(nb, s, tiles)
+    _gate(d.accel().cpu().numpy(), s)
