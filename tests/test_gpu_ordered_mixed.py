@@ -1,8 +1,10 @@
 """The mixed every-ordered-pair kernels at 2,131 bodies, where contexts run
 pair-once blocks by default: pair_once=False, each test asserting that it has
 reached them.  Tile decompositions (the mixed gate of the parity tests, every
-body), the shared-memory limit that contexts of unlike tiles share, and the
-autotuner."""
+body), the shared-memory limit that contexts of unlike tiles share, the
+autotuner, and the bounded waits of both kernels of the adjoint product."""
+import time
+
 import numpy as np
 import pytest
 
@@ -93,3 +95,34 @@ def test_autotune(nb):
     assert np.array_equal(c.state.cpu().numpy(), b.state.cpu().numpy())
     d = _ordered(nb, s, tiles)
     _gate(d.accel().cpu().numpy(), s)
+
+
+@pytest.mark.parametrize("precision,pair_once,block", [("mixed", False, 0), ("mixed", True, 128), ("fp64", False, 0)])
+def test_product_wait_timeout_reports_and_recovers(nb, precision, pair_once, block, monkeypatch):
+    """NBODY_INJECT_WAIT_STALL=2 makes the second adjoint product's bounded wait
+    run out: the ordered kernel's first source tile of CTA 0 stays unissued (the
+    CTA drains its other copies and leaves), the pair-once kernel's CTA 0 leaves
+    out an arrival.  nbody_grad reports ETIMEOUT, and the next gradient and
+    steps are a fresh context's to the bit."""
+    s = inputs.solar_system(N, seed=51)
+    gr = np.ones((3, s.n))
+    kw = dict(G=s.G, dt=s.dt, precision=precision, pair_once=pair_once)
+    fresh = nb.NBody(s.r, s.v, s.m, **kw)
+    assert fresh.pair_once_block == block
+    want = [t.cpu().numpy() for t in fresh.grad(3, gr)]
+    fresh.step(5)
+    state = fresh.state.cpu().numpy()
+    fresh.close()
+    monkeypatch.setenv("NBODY_INJECT_WAIT_STALL", "2")
+    b = nb.NBody(s.r, s.v, s.m, **kw)
+    monkeypatch.delenv("NBODY_INJECT_WAIT_STALL")
+    t0 = time.time()
+    with pytest.raises(nb.NBodyError) as ei:
+        b.grad(3, gr)
+    assert ei.value.status == nb.NBODY_ETIMEOUT
+    assert time.time() - t0 < 60
+    for x, y in zip(b.grad(3, gr), want):
+        assert np.array_equal(x.cpu().numpy(), y)
+    b.step(5)
+    assert np.array_equal(b.state.cpu().numpy(), state)
+    b.close()
