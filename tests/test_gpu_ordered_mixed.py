@@ -2,7 +2,8 @@
 pair-once blocks by default: pair_once=False, each test asserting that it has
 reached them.  Tile decompositions (the mixed gate of the parity tests, every
 body), the shared-memory limit that contexts of unlike tiles share, the
-autotuner, and the bounded waits of both kernels of the adjoint product."""
+autotuner, the bounded waits of both kernels of the adjoint product, and the
+two forms of its term."""
 import time
 
 import numpy as np
@@ -126,3 +127,28 @@ def test_product_wait_timeout_reports_and_recovers(nb, precision, pair_once, blo
     b.step(5)
     assert np.array_equal(b.state.cpu().numpy(), state)
     b.close()
+
+
+@pytest.mark.parametrize("n", [2049, 4352])
+def test_both_forms_of_the_product(nb, n):
+    """The pair-once product builds its term as f_q w_j - f_j w_q - 3 |d|^-2
+    (f_q a + f_j b) d, the ordered one from u = mu_q w_j - mu_j w_q: the same
+    rounding errors to a few FP32 ulps of the terms' magnitudes.  Against the
+    FP64 gradient both keep the mixed gate, and the one's error stays within
+    twice the other's in the root mean square over all elements (each 32-term
+    sum rounds on its own, so the two differ by far less than that)."""
+    s = inputs.solar_system(n, seed=23, moon_omega_dt_max=0.5)
+    rng = np.random.default_rng(n)
+    gr, gv = rng.normal(size=(3, n)), rng.normal(size=(3, n))
+    ref = oracle.grad(s.G, s.dt, 2, s.r, s.v, s.m, gr, gv, openmp=True, magnitudes=True)
+    rms = {}
+    for once in (True, False):
+        b = nb.NBody(s.r, s.v, s.m, G=s.G, dt=s.dt, precision="mixed", pair_once=once)
+        assert b.pair_once_block == (128 if once else 0)
+        got = [t.cpu().numpy() for t in b.grad(2, gr, gv)]
+        b.close()
+        for g, want, mag in zip(got, ref[:3], ref[3:]):
+            assert np.all(np.abs(g - want) <= 1e-3 * mag)
+        rms[once] = [np.sqrt(np.mean(((g - want) / mag) ** 2)) for g, want, mag in zip(got, ref[:3], ref[3:])]
+    for a, b in zip(rms[True], rms[False]):
+        assert a <= 2.0 * b, rms
