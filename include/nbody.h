@@ -285,7 +285,9 @@ nbody_status nbody_grad(nbody_ctx *ctx, int64_t n_steps, const double *dL_dr_T,
 nbody_status nbody_sync(nbody_ctx *ctx);
 
 /* Current work decomposition, and an override (validated; EINVAL if out of
- * range).  Changing tiles drops cached graphs and re-sizes scratch. */
+ * range).  Changing tiles drops cached graphs and re-sizes scratch.  Contexts
+ * on the pair-once kernels (nbody_pair_once) keep and report the tiles, but
+ * these shape the every-ordered-pair kernel only. */
 nbody_status nbody_get_tiles(const nbody_ctx *ctx, nbody_tiles *t);
 nbody_status nbody_set_tiles(nbody_ctx *ctx, const nbody_tiles *t);
 
@@ -293,12 +295,13 @@ nbody_status nbody_set_tiles(nbody_ctx *ctx, const nbody_tiles *t);
  * steps of the general (two-kernel) path, the one tiles shape, then the six
  * fastest again three times each over 4 x probe_steps steps, and keep the
  * one with the best time; a context whose nbody_step runs a single-launch
- * kernel keeps doing so.  (An FP64 context on the pair-once kernel, see
- * NBODY_FLAG_NO_SYM, has no decomposition to choose: its current tiles are
+ * kernel keeps doing so.  (A context on a pair-once kernel, FP64 or mixed, see
+ * nbody_pair_once, has no decomposition to choose: its current tiles are
  * timed and kept.)  The bound state is restored afterwards.  best (HOST, may be
  * NULL) receives the winner, best_ms its time per step.  With a tune_cache
- * (nbody_opts) the winner is also written there (replacing the entry with
- * the same key); if that file cannot be written the call returns
+ * (nbody_opts) the winner is also written there, replacing the entry with
+ * the same key (which a context on a pair-once kernel leaves as it is); if
+ * that file cannot be written the call returns
  * NBODY_EINVAL after keeping the winner.  Synchronous. */
 nbody_status nbody_autotune(nbody_ctx *ctx, int32_t probe_steps, nbody_tiles *best,
                             double *best_ms);

@@ -1688,7 +1688,7 @@ nbody_status nbody_autotune(nbody_ctx *c, int32_t probe_steps, nbody_tiles *best
           t.jsplit = js;
           cand.push_back(t);
         }
-  // the pair-once FP64 kernel has no tiles to choose: time the current ones only
+  // the pair-once kernels have no tiles to choose: time the current ones only
   if (sym_block(c)) cand.assign(1, c->tiles);
   cudaEvent_t e0, e1;
   NB_CUDA(c, cudaEventCreate(&e0));
@@ -1748,6 +1748,9 @@ nbody_status nbody_autotune(nbody_ctx *c, int32_t probe_steps, nbody_tiles *best
   if (best_ms) *best_ms = win_ms;
   if (!c->tune_cache.empty()) {
     nb::TuneEntry te;
+    // (one key serves contexts with and without pair-once blocks: tiles that
+    // shape nothing here do not replace those that another context found)
+    if (c->fw.sym_pairs && nb::tune_cache_lookup(c->tune_cache, tune_key(c), te)) return NBODY_OK;
     te.threads = win.threads;
     te.ipt = win.ipt;
     te.tj = win.tj;

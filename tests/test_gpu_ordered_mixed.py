@@ -98,6 +98,27 @@ def test_autotune(nb):
     _gate(d.accel().cpu().numpy(), s)
 
 
+def test_pair_once_context_leaves_tuned_tiles_in_the_cache(nb, tmp_path):
+    """One cache key covers 4,200 bodies (pair-once blocks: no tiles to choose)
+    and 5,003 (ordered pairs): autotuning the first must not replace what the
+    second found; without an entry it writes its own."""
+    path = tmp_path / "tune.json"
+    mk = lambda n: nb.NBody(*(lambda s: (s.r, s.v, s.m))(inputs.solar_system(n, seed=5)), G=inputs.G_AU_DAY,  # noqa: E731
+                            dt=inputs.DT_DAY, precision="mixed", tune_cache=str(path))
+    once = mk(4200)
+    assert once.pair_once_block == 128
+    once.autotune(probe_steps=1)
+    assert path.exists()
+    path.unlink()
+    a = mk(5003)
+    assert a.pair_once_block == 0
+    best, _ = a.autotune(probe_steps=1)
+    doc = path.read_text()
+    once.autotune(probe_steps=1)
+    assert path.read_text() == doc
+    assert mk(5003).tiles == best
+
+
 @pytest.mark.parametrize("precision,pair_once,block", [("mixed", False, 0), ("mixed", True, 128), ("fp64", False, 0)])
 def test_product_wait_timeout_reports_and_recovers(nb, precision, pair_once, block, monkeypatch):
     """NBODY_INJECT_WAIT_STALL=2 makes the second adjoint product's bounded wait
