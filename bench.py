@@ -301,7 +301,8 @@ def force_kernel_name(prec: str, block: int) -> str:
     if not block:
         return f"force_kernel<{prec}>"
     if prec == "mixed":
-        return f"force_msym_kernel (mixed, each pair once, {block}-entry blocks)"
+        name = "force_msym_block_kernel" if block == 128 else "force_msym_kernel"
+        return f"{name} (mixed, each pair once, {block}-entry blocks)"
     if block == 64:
         return "force_sym_kernel (FP64, each pair once, 64-body blocks)"
     return f"force_sym_wide_kernel (FP64, each pair once, {block}-body blocks)"
@@ -384,7 +385,7 @@ def run_ours(args):
                 b.reset()
             elif not args.no_autotune:
                 b.autotune(probe_steps=16 if prec == "mixed" else 2)
-            tiles[prec] = b.tiles
+            tiles[prec] = None if b.pair_once_block else b.tiles  # (the pair-once kernels have none)
             for _ in range(args.warmup):
                 b.step(inner)
             b.sync()
@@ -707,7 +708,9 @@ def extras(torch, nbody, inputs, stream, device, args, peaks=None):
         t = timed(torch, stream, lambda: b.step(n_ens))
     out["ensemble"] = {"systems": len(ens), "bodies": int(off[-1]), "steps": n_ens,
                        "interactions_per_s": pairs * n_ens / t, "verlet_steps_per_s": n_ens / t,
-                       "ms_per_step": t / n_ens * 1e3, "precision": "mixed", "tiles": b.tiles}
+                       "ms_per_step": t / n_ens * 1e3, "precision": "mixed",
+                       "force_kernel": force_kernel_name("mixed", b.pair_once_block),
+                       "tiles": None if b.pair_once_block else b.tiles}
     b.close()
     if args.dt_sweep:
         # Energy accuracy against dt (Section 4's criterion): the 10,425-body

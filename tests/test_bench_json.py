@@ -51,3 +51,15 @@ def test_roofline_against_measured_peaks():
     assert ro["peak_measured_tflops"] == 1.05 and ro["frac_of_measured"] == pytest.approx(0.7 / 1.05)
     assert bench.roofline(r, "mixed", None, peaks)["frac_of_measured"] == pytest.approx(0.7 / 77.4)
     assert "frac_of_measured" not in bench.roofline(r, "mixed", None)
+
+
+@pytest.mark.parametrize("prec,block,name", [("mixed", 0, "force_kernel<mixed>"), ("mixed", 128, "force_msym_block_kernel "),
+                                             ("mixed", 256, "force_msym_kernel "), ("mixed", 2048, "force_msym_kernel "),
+                                             ("fp64", 64, "force_sym_kernel "), ("fp64", 256, "force_sym_wide_kernel ")])
+def test_force_kernel_names(prec, block, name):
+    got = bench.force_kernel_name(prec, block)
+    assert got.startswith(name) and (block == 0 or f"{block}-" in got)
+    # the kernel that the library launches for this block size
+    csrc = os.path.join(ROOT, "paper_2112_15079_gb300", "csrc")
+    src = "".join(open(os.path.join(csrc, f)).read() for f in ("sym.cu", "sym_mixed.cu", "step_kernel.cuh"))
+    assert f"{name.split('<')[0].strip()}(const" in src
