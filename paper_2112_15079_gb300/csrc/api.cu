@@ -377,10 +377,11 @@ int sym_block(const nbody_ctx *c) {
 }
 
 // Work tables of the pair-once kernels: the block pairs (I, J), I <= J, of
-// every system, off-diagonal items first, blocks of B bodies (FP64: 64, or
-// wide: force only) or stage entries (mixed, force only); each body has one
-// partial row per block of its system (row_doubles values each: 3 force,
-// 4 VJP).  An item is (first stage entry of the system, its bodies, I, J).
+// every system, blocks of B bodies (FP64) or stage entries (mixed); each body
+// has one partial row per block of its system (row_doubles values each: 3
+// force, 4 VJP, which takes the narrowest blocks only: FP64 64, mixed 128).
+// Off-diagonal items go first, but on mixed 128-entry blocks the near ones,
+// diagonal first.  An item is (first stage entry of the system, its bodies, I, J).
 nbody_status build_sym_work(nbody_ctx *c, Work &wk, int row_doubles, int B) {
   free_work(c, wk);
   const bool mixed = c->o.precision == NBODY_MIXED;

@@ -308,7 +308,7 @@ __global__ void __launch_bounds__(VerletShape<PREC>::kBlock) verlet_kernel(const
   constexpr int L = VerletShape<PREC>::kLanes, NB = VerletShape<PREC>::kBodies;
   // Phase B: warp c < 3 takes component c of the CTA's 32 bodies, lane = body,
   // so each warp issues a third of the FP64 instructions (GB300's FP64 pipe
-  // spends 64 cycles on every warp instruction, so this is the latency).
+  // spends 76 cycles on every warp instruction, so this is the latency).
   const int p0 = a.p_begin + blockIdx.x * NB;  // bodies [p_begin, p_end) (a row shard, or all)
   const int comp = threadIdx.x >> 5, k = threadIdx.x & 31, q = p0 + k;
   const bool own = comp < 3 && q < a.p_end;

@@ -131,14 +131,19 @@ inline int pair_once_block(const std::vector<int64_t> &sizes, bool mixed, int64_
 //   ordered                   22.4          610         171         1338                4529
 //   128                       14.1          484         140         1871                9027
 //   512                       54.9          534         154         1135                3745
+//   (calls of 10 steps, ordered / 128)  2 x 2,048 20.5 / 13.8, 3 x 2,048 22.1 / 16.4, 2 x 3,000
+//   25.5 / 19.4, 2,048 + 100 22.1 / 11.3, 3,100 x 10 44.0 / 42.4, 10,000 x 31 419 / 146
 // 128: while the rows written per step (24 B per body and block) stay in the
 // L2 cache (kMsymRowBytes) or are few (kMsymFewRows per body), and the block
 // pairs fill the GPU's 4 x SMs CTAs once at most or at least five times
-// (between, the second round runs half empty), for a largest system of at
-// least kMsymSmallBodies or block pairs enough for five rounds (a few smaller
-// systems keep the ordered-pair kernel, whose tiles the caller can set, and
-// whose far test, a warp's 32 targets at a time, is finer); else 512 where
-// that gives 8 warps per SM and the rows would have left the cache.
+// (between, the second round runs half empty: 128 loses up to 8,192 bodies; it
+// wins from about 8,500, so the line at five rounds, 9,857 bodies, leaves up to
+// 9 % there), for a largest system of at least kMsymSmallBodies or block pairs
+// enough for five rounds; else 512 where that gives 8 warps per SM and the rows
+// would have left the cache.  Below kMsymSmallBodies 128 would win too (1,031
+// bodies by a quarter); contexts there keep the kernel whose tiles the caller
+// can set and tune.  (4 CTAs per SM and the 80 MB, 62 % of GB300's L2, are this
+// GPU's.)
 constexpr int64_t kMsymRowBytes = 80000000;
 constexpr int64_t kMsymFewRows = 8;
 constexpr int64_t kMsymSmallBodies = 2048;
