@@ -1019,18 +1019,6 @@ nbody_status spatial_order(nbody_ctx *c) {
   NB_CUDA(c, cudaMemcpyAsync(h.data() + N, c->y, b, cudaMemcpyDeviceToHost, c->stream));
   NB_CUDA(c, cudaMemcpyAsync(h.data() + 2 * N, c->z, b, cudaMemcpyDeviceToHost, c->stream));
   NB_CUDA(c, cudaStreamSynchronize(c->stream));
-  // Exponents of the systems' largest coordinates, for the stage's unit.
-  c->unit_lo = INT_MAX;
-  c->unit_hi = INT_MIN;
-  for (int64_t s = 0; s < c->n_sys; ++s) {
-    double top = 0.0;
-    for (int k = 0; k < 3; ++k)
-      for (int64_t p = c->offsets[s]; p < c->offsets[s + 1]; ++p) top = std::max(top, std::fabs(h[k * N + p]));
-    if (!(top > 0.0) || !std::isfinite(top)) continue;  // (staging reports what is not finite)
-    c->unit_lo = std::min(c->unit_lo, std::ilogb(top));
-    c->unit_hi = std::max(c->unit_hi, std::ilogb(top));
-  }
-  if (c->unit_lo > c->unit_hi) c->unit_lo = c->unit_hi = 0;
   c->qidx_h.assign(N, 0);
   std::vector<int32_t> perm(static_cast<size_t>(c->n_stage), 0);
   std::vector<std::pair<uint64_t, int32_t>> key;
@@ -1047,6 +1035,9 @@ nbody_status spatial_order(nbody_ctx *c) {
   } else {
     for (int64_t s = 0; s < c->n_sys; ++s) ranges.push_back({c->offsets[s], c->offsets[s + 1], c->soff[s], c->soff[s + 1]});
   }
+  // (exponents of the systems' largest coordinates, for the stage's unit)
+  c->unit_lo = INT_MAX;
+  c->unit_hi = INT_MIN;
   for (const Range &rg : ranges) {
     const int64_t b0 = rg.b, e0 = rg.e;
     double lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
@@ -1059,6 +1050,11 @@ nbody_status spatial_order(nbody_ctx *c) {
         hi[k] = std::max(hi[k], v);
       }
     const double span = std::max({hi[0] - lo[0], hi[1] - lo[1], hi[2] - lo[2]});
+    const double top = std::max({hi[0], -lo[0], hi[1], -lo[1], hi[2], -lo[2]});
+    if (finite && top > 0.0) {  // (staging reports what is not finite)
+      c->unit_lo = std::min(c->unit_lo, std::ilogb(top));
+      c->unit_hi = std::max(c->unit_hi, std::ilogb(top));
+    }
     key.clear();
     for (int64_t p = b0; p < e0; ++p) {
       uint64_t code = 0;
@@ -1080,6 +1076,7 @@ nbody_status spatial_order(nbody_ctx *c) {
     }
     for (int64_t slot = rg.q + (e0 - b0); slot < rg.qe; ++slot) perm[slot] = static_cast<int32_t>(std::min<int64_t>(b0, N - 1));
   }
+  if (c->unit_lo > c->unit_hi) c->unit_lo = c->unit_hi = 0;
   plan_boxes(c, h, perm);
   NB_CUDA(c, cudaMemcpyAsync(c->qidx, c->qidx_h.data(), sizeof(int32_t) * N, cudaMemcpyHostToDevice, c->stream));
   NB_CUDA(c, cudaMemcpyAsync(c->perm, perm.data(), sizeof(int32_t) * perm.size(), cudaMemcpyHostToDevice, c->stream));
