@@ -250,6 +250,20 @@ def test_a_body_among_massless_ones_feels_nothing(nb, n):
     b.close()
 
 
+@pytest.mark.parametrize("n", [31, 131])
+def test_single_launch_kernels_far_from_the_origin(nb, n):
+    """Coordinates whose squares overflow (1e160; an ulp is 1e144 there, so every
+    |d|^-3 underflows and Eq. 1 gives zeros): the massless stand-ins of the
+    single-launch kernels must not turn them into NaN."""
+    rng = np.random.default_rng(n)
+    r = 1e160 + np.round(rng.uniform(-1.0, 1.0, (3, n)) * 2.0**20) * 2.0**486
+    b = nb.NBody(r, 0.0 * r, rng.uniform(0.5, 1.0, n), G=1.0, dt=1e-200, precision="fp64")
+    b.step(2)
+    b.sync()
+    assert np.array_equal(b.accel().cpu().numpy(), np.zeros((3, n)))
+    b.close()
+
+
 @pytest.mark.parametrize("n", [1, 2, 33, 131, 521])
 def test_the_targets_own_pair_in_the_ordered_kernel(nb, n):
     """The FP64 ordered-pair kernel takes a target's own entry as a massless
