@@ -147,7 +147,7 @@ typedef struct {
    *   to about 20,600 bodies, or many systems), 512 where the sums would
    *   leave the cache (at most 4 GiB of sums, a third more for nbody_grad);
    *   else every ordered pair is evaluated, as in contexts of several systems
-   *   whose largest coordinates lie more than a factor 2^20 apart.  Or set: a
+   *   whose largest coordinates lie more than a factor 2^30 apart.  Or set: a
    *   power of two from 128 to 2,048.  128 applies to the VJP of nbody_grad
    *   too, wider blocks to the force only.
    * A set size is used whatever the systems' sizes (for contexts that are

@@ -85,11 +85,11 @@ inline int64_t pair_once_items(const std::vector<int64_t> &sizes, int64_t B) {
 // without where FP32's range holds both.  lo, hi: the smallest and the largest,
 // over the systems, of the exponent of a system's largest |coordinate|.  k = 0
 // while these leave room on both sides (astronomical units: 5); else the
-// largest becomes 2^20, 2^62 above the closest pair that FP32 then takes and 2^21
-// below the farthest.  Systems whose sizes lie further apart than 2^20 cannot
-// share a unit and keep the ordered-pair kernel (unless a block size was asked
-// for).
-constexpr int kUnitLow = -4, kUnitHigh = 24, kUnitTo = 20, kUnitSpread = 20;
+// largest becomes 2^24, 2^66 above the closest pair that FP32 then takes and 2^17
+// below the farthest.  Systems whose sizes lie further apart than 2^30 (the
+// smallest then has 2^36 left for its closest pairs) cannot share a unit and
+// keep the ordered-pair kernel (unless a block size was asked for).
+constexpr int kUnitLow = -4, kUnitHigh = 24, kUnitTo = 24, kUnitSpread = 30;
 
 inline bool stage_unit_fits(int lo, int hi) { return hi - lo <= kUnitSpread; }
 inline int stage_unit_exp(int lo, int hi) {

@@ -403,17 +403,19 @@ def test_mixed_units_are_the_callers(nb, n, kw):
             assert np.array_equal(x, y), (j, np.abs(x - y).max())
 
 
-def test_mixed_systems_of_unlike_sizes(nb):
-    """Two systems whose lengths differ by 2^25 share no unit in FP32: they keep
-    the ordered-pair kernel, and the mixed gate holds in both."""
+@pytest.mark.parametrize("exp,block", [(35, 0), (25, 128)])
+def test_mixed_systems_of_unlike_sizes(nb, exp, block):
+    """Two systems whose lengths differ by 2^35 share no unit in FP32: they keep
+    the ordered-pair kernel; by 2^25 they share one.  The mixed gate holds in
+    both."""
     parts = [inputs.solar_system(2049, seed=k) for k in (82, 83)]
-    scale = (1.0, 2.0**-25)
+    scale = (1.0, 2.0**-exp)
     r = np.concatenate([p.r * u for p, u in zip(parts, scale)], 1)
     v = np.concatenate([p.v * u for p, u in zip(parts, scale)], 1)
     m = np.concatenate([p.m * u for p, u in zip(parts, scale)])
     off = np.array([0, 2049, 4098])
     a, used = _mixed_accel(nb, r, v, m, off)
-    assert used == 0
+    assert used == block
     for b, e in zip(off[:-1], off[1:]):
         x, w = np.ascontiguousarray(r[:, b:e]), m[b:e]
         err = np.linalg.norm(a[:, b:e] - oracle.accel(inputs.G_AU_DAY, x, w, openmp=True), axis=0)
@@ -525,3 +527,42 @@ def test_mixed_rows_without_memory(nb, monkeypatch):
         for g, h, x, mag in zip(got, again, ref[:3], ref[3:]):
             assert np.array_equal(g, h)
             assert np.all(np.abs(g - x) <= 1e-3 * mag)
+
+
+def test_reset_between_like_and_unlike_sizes(nb):
+    """A reset onto positions that share no unit moves a context to the ordered-pair
+    kernels, adjoint product included, and one back onto the first positions to
+    the pair-once ones: each time bitwise what a new context computes (or
+    reports: the ordered product's |d|^-5 leaves FP32's range on the smaller
+    system's moons, 3e-15 units apart)."""
+    torch = pytest.importorskip("torch")
+
+    def grad(c):
+        try:
+            return [t.cpu().numpy() for t in c.grad(2, gr)]
+        except nb.NBodyError as e:
+            assert e.status == nb.NBODY_ENONFINITE
+            return [np.array([float(e.status)])]
+
+    parts = [inputs.solar_system(2049, seed=k) for k in (85, 86)]
+    v, m = np.zeros((3, 4098)), np.concatenate([p.m for p in parts])
+    off = np.array([0, 2049, 4098])
+    near = np.concatenate([p.r for p in parts], 1)
+    far = np.concatenate([parts[0].r, parts[1].r * 2.0**-35], 1)
+    kw = dict(G=inputs.G_AU_DAY, dt=1e-9, precision="mixed")
+    gr = np.random.default_rng(2).normal(size=(3, 4098))
+    b = nb.NBody(near, v, m, off, **kw)
+    for r, block in ((near, 128), (far, 0), (near, 128)):
+        b.state[0:3].copy_(torch.tensor(r))
+        b.state[3:6].copy_(torch.tensor(v))
+        b.reset()
+        fresh = nb.NBody(r, v, m, off, **kw)
+        assert b.pair_once_block == fresh.pair_once_block == block
+        for x, y in zip(grad(b), grad(fresh)):
+            assert np.array_equal(x, y)
+        b.step(3)
+        fresh.step(3)
+        assert np.array_equal(b.state.cpu().numpy(), fresh.state.cpu().numpy())
+        assert np.array_equal(b.accel().cpu().numpy(), fresh.accel().cpu().numpy())
+        fresh.close()
+    b.close()
