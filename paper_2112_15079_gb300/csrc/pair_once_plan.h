@@ -11,12 +11,10 @@
 //   kSymRowLimit (else none); used when the systems hold at least 1.5 block
 //   pairs per SM (with fewer, one CTA carries a system's whole sum; measured
 //   on GB300, us per step, pair-once against every ordered pair: 600 bodies
-//   44.5 / 30.6, 1,031 bodies / 153 pairs 45.8 / 51.9, 1,283 bodies / 231 pairs
-//   46.3 / 60.6, 10,425 bodies 649 / 1,240; since both kernels take their
-//   reciprocal cubes from the integer pipes they meet near 800 bodies, which
-//   only contexts without the single-launch kernels see).
+//   44.6 / 22.2, 1,031 bodies / 153 pairs 46.0 / 40.9, 1,283 bodies / 231 pairs
+//   47.0 / 51.2, 10,425 bodies 649 / 1,224).
 //   Mixed (stage entries per block): for a largest system of at least
-//   kMsymMinBodies (measured on GB300: 65,536 bodies 1.49 against 1.82 ms
+//   kMsymMinBodies (measured on GB300: 65,536 bodies 1.50 against 1.82 ms
 //   per step, 1,048,576 bodies 340 against 430 ms), the narrowest block (128 ..
 //   2,048 entries) that leaves the largest system at most kMsymMaxRows rows
 //   per body, if the rows fit in kSymRowLimit and the block pairs give at
